@@ -59,19 +59,24 @@ cudaError_t blocks_per_sm(const void *fn, int threads, size_t smem, int *out) {
     return cudaSuccess;
 }
 
-// Candidate slots per warp (a multiple of 32: 32 lanes x quota).  About 40% of
-// the rows, at least 512 (small n: every row fits).
-template <typename T> static int cap_for(int64_t npad) {
-    int64_t c = std::max<int64_t>(512, (npad * 2 / 5 + 31) & ~int64_t(31));
-    return (int)(std::min<int64_t>(npad, c) & ~int64_t(31));
+// Candidate slots of the 64-bit selection's list that hold its first bracket
+// at any width, 40% of the rows and at least 512 (or every row), and the bytes
+// such a list takes per warp beside its histogram.
+static int64_t list_slots(int64_t npad) {
+    const int64_t c = std::max<int64_t>(512, (npad * 2 / 5 + 31) & ~int64_t(31));
+    return std::min<int64_t>(npad, c) & ~int64_t(31);
+}
+static size_t list_bytes(int64_t slots) {
+    return std::max(al16(slots * 8) + 256, al16(slots * 4) + al16(slots * 2) + HIST_WORDS * 4);
 }
 
+// The limit on n is a fixed one (20,608 float, 16,000 double): the rows whose
+// column arrays and one warp with a full list fit a CTA.
 template <typename T> int64_t max_rows_pairs() {
     const size_t budget = 227 * 1024;
     int64_t n = ROW_PAD;
     while (n + ROW_PAD <= (int64_t)ROW_MASK + 1 &&
-           PairSmem<T>::col_bytes(n + ROW_PAD, false) +
-                   PairSmem<T>::warp_bytes(cap_for<T>(n + ROW_PAD)) <=
+           PairSmem<T>::col_bytes(n + ROW_PAD, false) + list_bytes(list_slots(n + ROW_PAD)) <=
                budget)
         n += ROW_PAD;
     return n;
@@ -95,21 +100,20 @@ template <typename T>
 static PairPlan plan_placement(int64_t npad, bool cs, int d0, const Tune &tune) {
     PairPlan p{0, 0, 0, 0, 0, 0, 0, 0, 0};
     const size_t cb = PairSmem<T>::col_bytes(npad, cs);
-    // Per-lane candidate quota wanted: the level-0 bracket (+-d0 of 64 weight
-    // samples) holds ~2.5% of the rows per sample position, i.e. mu = 0.025 d0
-    // n/32 per lane; ask for mu + 3.5 sqrt(mu) + 1 so that the busiest of 32
-    // lanes rarely overflows (an overflow costs one more pass).
+    // Slots of the 64-bit selection's list.  That selection is the rare
+    // fallback, and with a short list it narrows its bracket by a counting
+    // pass first, so 128 slots leave the room to more resident warps and to
+    // L1.  A caller's own d0 gets a list that holds a bracket of that width:
+    // ~2.5% of the rows per sample position, i.e. mu = 0.025 d0 n/32 per lane,
+    // and mu + 3.5 sqrt(mu) + 1 for the busiest of 32 lanes.
     const double mu = 0.025 * (double)d0 * (double)npad / 32.0;
     const int64_t qt_need = std::min<int64_t>(npad / 32, (int64_t)ceil(mu + 3.5 * sqrt(mu) + 1.0));
+    const int64_t slots = std::min<int64_t>(npad, 128);
     // Over 1-3 CTAs per SM and 1-16 warps per CTA (or the caller's choice),
     // up to 32 resident warps in one of the launch shapes (pair_shape), keep
-    // the plan with the most resident warps whose lists meet the quota in
-    // 228 KB of shared memory (1 KB reserved per CTA, static arrays included);
-    // on a tie the fewer, larger CTAs (column jhat staged fewer times, so
-    // longer lists per warp).  Measured, 2000 x 2000 float: 16 x 2 warps
-    // (64 registers) 14.1 ms, 8 x 3 (80 registers) 14.4 ms; 5000 x 1000:
-    // 16 x 1 (128 registers, x_ijhat in shared memory) 11.0 ms, 8 x 2 with
-    // x_ijhat in global memory 13.6 ms.
+    // the plan with the most resident warps that fits 228 KB of shared memory
+    // (1 KB reserved per CTA, static arrays included); on a tie the fewer,
+    // larger CTAs (column jhat staged fewer times).
     int w = 0, cap = 0, best = 0, nc = 0;
     const int c_hi = tune.ctas > 0 ? tune.ctas : 3, c_lo = tune.ctas > 0 ? tune.ctas : 1;
     const int w_hi = tune.warps > 0 ? tune.warps : 16, w_lo = tune.warps > 0 ? tune.warps : 1;
@@ -117,14 +121,19 @@ static PairPlan plan_placement(int64_t npad, bool cs, int d0, const Tune &tune) 
         const int64_t per_cta = 233472 / ctas - 1024 - 1024;
         for (int cand = w_hi; cand >= w_lo; --cand) {
             if (ctas * cand <= best || pair_shape(cand, ctas) < 0) continue;
-            const int64_t fit = PairSmem<T>::cap_fit((per_cta - (int64_t)cb) / cand);
-            const int64_t c32 = std::min<int64_t>(npad, fit) & ~int64_t(31);
-            if (fit > 0 && c32 >= 32 * qt_need) {
-                w = cand;
-                cap = (int)c32;
-                best = ctas * cand;
-                nc = ctas;
+            const int64_t room = (per_cta - (int64_t)cb) / cand;
+            int64_t c = slots;
+            if (tune.d0 > 0) {
+                c = std::min<int64_t>(npad, room / 8) & ~int64_t(31);
+                while (c > 0 && list_bytes(c) > (size_t)std::max<int64_t>(room, 0)) c -= 32;
+                if (c < 32 * qt_need) continue;
+            } else if (room < (int64_t)PairSmem<T>::warp_bytes(c)) {
+                continue;
             }
+            w = cand;
+            cap = (int)c;
+            best = ctas * cand;
+            nc = ctas;
         }
     }
     if (w == 0) return p;

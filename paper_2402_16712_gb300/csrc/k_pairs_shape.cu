@@ -9,34 +9,6 @@
 #ifndef L1L_SHAPE
 #error "compile with -DL1L_SHAPE=0|1|2"
 #endif
-// Loop unrolling of the 32-bit selection per shape (select32.cuh); measured
-// on the planner's launches, kernel time: 2000 x 2000 (64 registers)
-// level-0 loop unrolled by two 14.18 -> 13.51 ms, 1000 x 500 0.70 -> 0.67 ms;
-// 5000 x 1000 (128 registers) level-0 unroll 11.00 -> 11.46 ms (kept at one),
-// list loops unrolled by two 11.00 -> 10.88 ms.
-#if L1L_SHAPE == 2
-#ifndef L1L_L0_UNROLL
-#define L1L_L0_UNROLL 1
-#endif
-#ifndef L1L_LIST_UNROLL
-#define L1L_LIST_UNROLL 2
-#endif
-#else
-#ifndef L1L_L0_UNROLL
-#define L1L_L0_UNROLL 2
-#endif
-#ifndef L1L_LIST_UNROLL
-#define L1L_LIST_UNROLL 1
-#endif
-#endif
-// Lane balancing of the candidate lists (list32_balance), measured on the
-// 2000 x 2000 float fit, kernel time: 8 x 3 warps (80 registers) 14.36 ->
-// 13.86 ms, 16 x 2 warps (64 registers) 13.11 -> 13.61 ms, 16 x 1 warps (128
-// registers) 16.82 -> 16.80 ms; so only the 80-register shape balances.
-#ifndef L1L_BALANCE
-#define L1L_BALANCE (L1L_SHAPE == 0)
-#endif
-
 #include <algorithm>
 
 #include "batch.cuh"
@@ -66,7 +38,7 @@ __global__ void __launch_bounds__(ShapeBounds<S>::threads, ShapeBounds<S>::block
     k_pairs(ScanArgs<T> a, const __grid_constant__ LambdaPack lp, int t0, int nlc, int kchunk,
             int cap) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ Decide s_dec[NDEC];
+    __shared__ Dec32 s_dec[NDEC];
     const int64_t k0 = (int64_t)blockIdx.y * kchunk;
     const int64_t k1 = min(a.m, k0 + kchunk);
     const LamView lv{lp.lam, lp.tl_min, lp.tl_max};
@@ -108,7 +80,7 @@ __global__ void __launch_bounds__(ShapeBounds<S>::threads, ShapeBounds<S>::block
     k_pairs_persist(const __grid_constant__ BatchDesc<T> bd, unsigned char *ws, int64_t u0,
                     int64_t u1, int slot, int lay_npad, int cap) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ Decide s_dec[NDEC];
+    __shared__ Dec32 s_dec[NDEC];
     __shared__ long long s_unit;
     unsigned long long *counter = reinterpret_cast<unsigned long long *>(ws + 512) + slot;
     for (;;) {

@@ -2,9 +2,9 @@
 // weighted median (Lemma 1) and per-pair residual (Algorithm 1).
 //
 // Layout: one CTA per (jhat, k-chunk).  Column jhat is staged once in shared
-// memory -- x_ijhat, its float reciprocal and its fixed-point weight q_i -- and
-// shared by the CTA's warps; each warp owns one k at a time and keeps a short
-// candidate list of its own.
+// memory -- x_ijhat, its float reciprocal and its fixed-point weight -- and
+// shared by the CTA's warps; each warp owns one k at a time and keeps a small
+// histogram of its own.
 //
 // Per pair the warp never divides per row.  It orders rows by a COARSE key,
 // the 32-bit order-preserving image of the ratio rounded to float, and
@@ -12,27 +12,17 @@
 // float first for double input).  The approximation is within G keys of the
 // coarse key of the correctly rounded ratio (G = 8 float, 16 double; the bound
 // is derived in the design notes), so a row whose approximate key is more than
-// G away from a pivot is classified exactly without dividing; the few rows
-// inside a guard band, and the final <= 31 candidates, are divided exactly.
+// G away from a pivot is classified exactly without dividing; the final <= 31
+// candidates are divided exactly and decide the median by exact integer
+// arithmetic (the test of Lemma 1).
 //
-//   level 0  64 sampled rows are keyed and sorted across the warp; two pivots
-//            bracketing the estimated crossing of half the weight are taken;
-//            one pass over all rows sums the exact fixed-point weight below
-//            the lower pivot and compacts the rows between the pivots (guard
-//            bands included) into the candidate list;
-//   resolve  guard-band candidates are divided exactly; an exact 64-bin
-//            weight histogram of [P1, P2] and the exact weight below P1 decide
-//            whether the median lies between the pivots (else level 0 repeats
-//            on the indicated side) and in which bin; that bin's candidates
-//            are kept;
-//   levels   while more than 31 candidates remain: the same exact histogram
-//            over the surviving key range, keep the crossing bin;
-//   final    exact keys (double: 64-bit) of the <= 31 candidates plus the
-//            penalty point's key, one per lane; each lane's cumulative weight
-//            (a shuffle sum over the keys <= its own) is tested and the
-//            smallest passing key is the median (the test of Lemma 1, decided
-//            exactly);
-//   residual sum_i |x_ik - v x_ijhat| over all rows (Algorithm 1, objective).
+// The selection proper is in select32.cuh (32-bit weights, two passes over
+// the rows).  The 64-bit selection below is its fallback, for what the 32-bit
+// weights cannot settle: sampled pivots, a pass that compacts the rows between
+// them into a candidate list (or, when the list is too short, histograms all
+// rows), an exact 64-bin weight histogram of the list, narrowed to <= 31
+// candidates.  Then the residual sum_i |x_ik - v x_ijhat| over all rows
+// (Algorithm 1, objective).
 //
 // A decision the truncated fixed-point weights cannot settle, a column whose
 // magnitudes fall outside the approximation's range, or a candidate list that
@@ -86,25 +76,11 @@ template <typename T> struct PairSmem {
         return (cs ? al16(npad * sizeof(T)) : 0) + al16(npad * 4) + al16(npad * 4) +
                al16(NSAMP * 2);
     }
-    // per warp, 64-bit selection: candidate keys (uint32), row indices
-    // (uint16; bit 15 = exact key) and the histogram (4 x 64 uint32)
-    __host__ __device__ static size_t bytes64(int64_t cap) {
-        return al16(cap * 4) + al16(cap * 2) + al16(HIST_WORDS * 4);
-    }
-    // per warp, 32-bit selection: 8-byte entries and a 64-word histogram,
-    // overlaid by the arrays of its 64-bit fallback
-    __host__ __device__ static size_t bytes32(int64_t cap) { return al16(cap * 8) + al16(64 * 4); }
+    // per warp: the histogram (256 words, of either selection), then the
+    // 64-bit selection's candidate keys (uint32) and row indices (uint16; bit
+    // 15 = exact key)
     __host__ __device__ static size_t warp_bytes(int64_t cap) {
-        const size_t a = bytes32(cap), b = bytes64(cap);
-        return a > b ? a : b;
-    }
-    // the largest capacity (a multiple of 32) whose per-warp region fits `bytes`
-    __host__ __device__ static int64_t cap_fit(int64_t bytes) {
-        const int64_t c64 = (bytes - HIST_WORDS * 4 - 32) / 6;
-        const int64_t c32 = (bytes - 64 * 4 - 16) / 8;
-        int64_t c = (c64 < c32 ? c64 : c32) & ~int64_t(31);
-        while (c > 0 && warp_bytes(c) > (size_t)bytes) c -= 32;
-        return c;
+        return al16(HIST_WORDS * 4) + al16(cap * 4) + al16(cap * 2);
     }
 };
 
@@ -344,6 +320,56 @@ template <typename T> struct WqFly {
     }
 };
 
+// The exact test on the 32-bit weights, with its thresholds as whole weights:
+// S passes at a negative ratio when S >= tneg, at a ratio >= 0 when S >= tpos
+// (untruncated weights; the search steers by them, the test decides).
+struct Dec32 : Decide {
+    uint32_t tneg, tpos;
+    __device__ __forceinline__ void set(const ColInfo &ci, double lambda) {
+        init32(ci, lambda);
+        auto clamp = [](int64_t x) -> uint32_t {
+            return x < 0 ? 0u : (x > 0xFFFFFFFFll ? 0xFFFFFFFFu : (uint32_t)x);
+        };
+        tneg = clamp(((Q + Lf) >> 1) + 1);
+        tpos = clamp(((Q - Lc) >> 1) + 1);
+    }
+};
+
+// The lambdas of one launch (or of one instance of a batch).
+struct LamView {
+    const double *lam;
+    int tl_min, tl_max;  // positions of the smallest and largest lambda
+};
+
+// Everything one warp needs to solve the pairs of its CTA's column jhat.
+// The fast path's weights are the 32-bit q32 (both input types); s_dec and
+// decide_for use the same scale.
+template <typename T> struct WarpCtx {
+    const T *colb;
+    const float *inv;
+    const uint32_t *q32;
+    const uint16_t *samp;
+    uint32_t *hist;        // histogram of either selection
+    uint32_t *lk;          // 64-bit fallback's lists
+    uint16_t *li;
+    const Dec32 *s_dec;   // per-lambda thresholds for the first NDEC lambdas
+    int qt, n;
+    int d0;               // first-bracket half-width in sample positions
+    int srow;             // this lane's sample row and its 1/x_ijhat
+    float sinv;
+    ColInfo cinfo;
+};
+constexpr int NDEC = 32;
+
+// The coarse key of an exact key.
+template <typename T>
+__device__ __forceinline__ uint32_t coarse_of(typename Traits<T>::K k) {
+    if constexpr (sizeof(T) == 4)
+        return k;
+    else
+        return ckey(__double2float_rn(Traits<T>::value(k)));
+}
+
 }  // namespace l1l
 
 #include "select32.cuh"
@@ -421,7 +447,9 @@ __device__ int select_v2(const T *__restrict__ xk, const float *__restrict__ xf,
     P2 = min(sat_add(P2, 2 * G + 1), hi0);
     if (P1 > P2) P1 = P2;
     bool sampled = true;     // the bracket still comes from the sample
-    bool count_pass = false;  // next attempt: narrow by a histogram over all rows
+    // next attempt: narrow by a histogram over all rows (at once when the list
+    // is too short for a sample bracket)
+    bool count_pass = qt * 128 < n;
 
     int64_t L = 0;   // exact weight of rows with coarse key < lo
     uint32_t lo = 0, hi = CKMAX;
@@ -739,45 +767,14 @@ __device__ int select_v2(const T *__restrict__ xk, const float *__restrict__ xf,
     return SEL_OK;
 }
 
-// The lambdas of one launch (or of one instance of a batch).
-struct LamView {
-    const double *lam;
-    int tl_min, tl_max;  // positions of the smallest and largest lambda
-};
-
-// Everything one warp needs to solve the pairs of its CTA's column jhat.
-// The fast path's weights are the 32-bit q32 (both input types); s_dec and
-// decide_for use the same scale.
-template <typename T> struct WarpCtx {
-    const T *colb;
-    const float *inv;
-    const uint32_t *q32;
-    const uint16_t *samp;
-    uint32_t *lk;          // 64-bit fallback's lists and histogram
-    uint16_t *li;
-    uint32_t *hist;
-    uint2 *lst;            // 32-bit selection's list and histogram
-    uint32_t *hist32;
-    const Decide *s_dec;  // per-lambda thresholds for the first NDEC lambdas
-    int qt, n;
-    int d0;               // first-bracket half-width in sample positions
-    ColInfo cinfo;
-    __device__ __forceinline__ int64_t q(int i) const { return (int64_t)q32[i]; }
-};
-constexpr int NDEC = 32;
-
 // The exact test of lambda tl on the fast path's weight scale (q32).
 template <typename T>
-__device__ __forceinline__ void decide_init(Decide &dc, const ColInfo &ci, double lam) {
-    dc.init32(ci, lam);
-}
-template <typename T>
-__device__ __forceinline__ Decide decide_for(const WarpCtx<T> &w, const LamView &lp, int tl) {
-    Decide dc;
+__device__ __forceinline__ Dec32 decide_for(const WarpCtx<T> &w, const LamView &lp, int tl) {
+    Dec32 dc;
     if (tl < NDEC)
         dc = w.s_dec[tl];
     else
-        decide_init<T>(dc, w.cinfo, lp.lam[tl]);
+        dc.set(w.cinfo, lp.lam[tl]);
     return dc;
 }
 
@@ -807,10 +804,9 @@ template <typename T>
 __device__ __forceinline__ int select_pair(const T *xk, const float *xf, const WarpCtx<T> &w,
                                            const LamView &lp, int tl,
                                            typename Traits<T>::K &ts, int lane) {
-    const Decide dc = decide_for(w, lp, tl);
+    const Dec32 dc = decide_for(w, lp, tl);
     typename Traits<T>::K t32 = 0;
-    const int st = select_w32<T>(xf, xk, w.colb, w.inv, w.q32, w.samp, w.lst, w.hist32, w.qt,
-                                 w.n, w.d0, dc, t32, lane);
+    const int st = select_w32<T>(xf, xk, w, dc, t32, lane);
     if (st != SEL_W64) {
         ts = t32;
         return st;
@@ -1002,106 +998,39 @@ __device__ void solve_one(const ScanArgs<T> &a, const LamView &lp, int t0, int t
 
 // Lambda batch (step A7).  The weighted median moves monotonically toward 0
 // as lambda grows (the penalty point only gains weight), so every lambda's
-// median lies between those of the smallest and the largest lambda.  Solve
-// those two fully, collect the rows whose exact keys lie between them (one
-// pass, exact divisions only near the bounds) together with the exact weight
-// below, and decide every lambda from one sort and prefix scan of those rows.
-// Returns false (nothing written) when more than 31 rows lie between.
+// median lies between those of the smallest and the largest lambda: one
+// selection brackets both, and every lambda is decided from one sort and
+// prefix scan of the candidates between them.  Returns false (nothing
+// written) when more than 31 rows lie between.
 template <typename T, bool CS>
 __device__ bool lambda_path(const ScanArgs<T> &a, const LamView &lp, int t0, int nlc, int64_t j,
                             int64_t k, const T *__restrict__ xk, const float *__restrict__ xf,
                             const WarpCtx<T> &w, int lane) {
     using Tr = Traits<T>;
     using K = typename Tr::K;
-    using A = Approx<T>;
-    constexpr uint32_t G = A::G;
     const unsigned FULL = 0xFFFFFFFFu;
-    const int n = w.n;
-    K Ka = Tr::KEY0, Kb = Tr::KEY0;
-    if (select_pair<T>(xk, xf, w, lp, lp.tl_min, Ka, lane) != SEL_OK) return false;
-    if (select_pair<T>(xk, xf, w, lp, lp.tl_max, Kb, lane) != SEL_OK) return false;
-    const K Klo = min(Ka, Kb), Khi = max(Ka, Kb);
-    const uint32_t cl = ckey((float)Tr::value(Klo)), ch = ckey((float)Tr::value(Khi));
-    const uint32_t bt = sat_sub(cl, G), at = min(sat_add(ch, G), CKMAX);
-    int64_t Sb = 0;  // exact weight of rows with key < Klo
-    int cnt = 0;
-    uint16_t *stage = reinterpret_cast<uint16_t *>(w.hist);
-    int c = 0;
-    constexpr int U = 4;  // loads of the next batch in flight while this one is classified
-    float an[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const int i = u * 32 + lane;
-        an[u] = i < n ? xf[i] : 0.0f;
-    }
-    for (int i0 = 0; i0 < n; i0 += 32 * U) {
-        float ac[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) ac[u] = an[u];
-        if (i0 + 32 * U < n) {
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int i = i0 + 32 * U + u * 32 + lane;
-                an[u] = i < n ? xf[i] : 0.0f;
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * 32 + lane;
-            bool take = false;
-            if (i < n) {
-                const float iv = w.inv[i];
-                if (!isnan(iv)) {
-                    const uint32_t kk = akey(__fmul_rn(ac[u], iv));
-                    if (kk < bt) {
-                        Sb += w.q(i);
-                    } else if (kk <= at) {
-                        const K ke = Tr::key(Tr::div_rn(xk[i], w.colb[i]));
-                        if (ke < Klo)
-                            Sb += w.q(i);
-                        else if (ke <= Khi)
-                            take = true;
-                    }
-                }
-            }
-            const unsigned msk = __ballot_sync(FULL, take);
-            if (take) {
-                const int pos = c + __popc(msk & ((1u << lane) - 1u));
-                if (pos < 31) stage[pos] = (uint16_t)i;
-            }
-            c += __popc(msk);
-            cnt += take ? 1 : 0;
-        }
-    }
-    (void)cnt;
-    Sb = warp_sum_i64(Sb);
-    __syncwarp();
-    if (c > 31) return false;
-    K fk = Tr::NONE;
-    int64_t fq = 0;
-    if (lane < c) {
-        const int row = L1L_CHK((int)stage[lane], (n + ROW_PAD - 1) & ~(ROW_PAD - 1));
-        fk = Tr::key(Tr::div_rn(xk[row], w.colb[row]));
-        fq = w.q(row);
-    } else if (lane == c && Klo <= Tr::KEY0 && Tr::KEY0 <= Khi) {
-        fk = Tr::KEY0;
-    }
-    __syncwarp();
+    Cand32<T> f;
+    if (candidates32<T, true>(xf, xk, w, decide_for(w, lp, lp.tl_min), decide_for(w, lp, lp.tl_max),
+                              f, lane) != SEL_OK)
+        return false;
+    K fk = f.fk;
+    int64_t fq = (int64_t)f.fq;
     warp_sort32(fk, fq, lane);
     const int64_t P = warp_scan_add(fq, lane);
     const K nxt = __shfl_down_sync(FULL, fk, 1);
-    const bool last = (lane == 31) || (nxt != fk);
+    const bool last = fk != Tr::NONE && (lane == 31 || nxt != fk);
     K prev = Tr::NONE;
     T prev_res = T(0);
     for (int tl = 0; tl < nlc; ++tl) {
-        const Decide dc = decide_for(w, lp, tl);
+        const Dec32 dc = decide_for(w, lp, tl);
         int r = -2;
-        if (last && fk != Tr::NONE) r = dc.cond(Sb + P, fk >= Tr::KEY0);
+        if (last) r = dc.cond(f.L + P, fk >= Tr::KEY0);
         const unsigned okm = __ballot_sync(FULL, r == 1);
         const unsigned unm = __ballot_sync(FULL, r == -1);
         const unsigned any = okm | unm;
         const int first = any ? __ffs(any) - 1 : 0;
-        if (!any || ((unm >> first) & 1u)) {  // undecided here: full selection
+        // undecided here, or already passed below lo: full selection
+        if (!any || ((unm >> first) & 1u) || dc.cond(f.L, f.lo > CK0) != 0) {
             solve_one<T, CS>(a, lp, t0, tl, j, k, xk, xf, w, false, lane);
             prev = Tr::NONE;
             continue;
@@ -1109,7 +1038,7 @@ __device__ bool lambda_path(const ScanArgs<T> &a, const LamView &lp, int t0, int
         const K ts = __shfl_sync(FULL, fk, first);
         const T v = Tr::value(ts);
         if (ts != prev) {
-            prev_res = pair_residual<T, CS>(a, j, k, xk, w.colb, n, v, lane);
+            prev_res = pair_residual<T, CS>(a, j, k, xk, w.colb, w.n, v, lane);
             prev = ts;
         }
         if (lane == 0) {
@@ -1130,13 +1059,11 @@ __device__ bool lambda_path(const ScanArgs<T> &a, const LamView &lp, int t0, int
 template <typename T, bool MULTI, bool CS>
 __device__ void pairs_unit(const ScanArgs<T> &a, const LamView &lp, int t0, int nlc, int j,
                            int64_t k0, int64_t k1, int cap, int lay_npad, unsigned char *smem,
-                           Decide *s_dec) {
-    using Tr = Traits<T>;
-    using K = typename Tr::K;
+                           Dec32 *s_dec) {
     const int n = (int)a.n;
     const int64_t m = a.m, ldn = a.ldn;
     const int npad = lay_npad;  // shared-memory layout stride (>= n rounded up to 32)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
     const T *xj = a.Xt + (int64_t)j * ldn;
     T *colb_s = reinterpret_cast<T *>(smem);
@@ -1150,13 +1077,10 @@ __device__ void pairs_unit(const ScanArgs<T> &a, const LamView &lp, int t0, int 
     uint16_t *samp = reinterpret_cast<uint16_t *>(smem + off);
     unsigned char *wbase =
         smem + PairSmem<T>::col_bytes(npad, CS) + (size_t)warp * PairSmem<T>::warp_bytes(cap);
-    uint32_t *lk = reinterpret_cast<uint32_t *>(wbase);
-    uint16_t *li = reinterpret_cast<uint16_t *>(wbase + al16((size_t)cap * 4));
-    uint32_t *hist = reinterpret_cast<uint32_t *>(wbase + al16((size_t)cap * 4) +
-                                                  al16((size_t)cap * 2));
-    uint2 *lst = reinterpret_cast<uint2 *>(wbase);
-    uint32_t *hist32 = reinterpret_cast<uint32_t *>(wbase + al16((size_t)cap * 8));
-    // prologue scratch: the first 256 bytes of warp 0's candidate list
+    uint32_t *hist = reinterpret_cast<uint32_t *>(wbase);
+    uint32_t *lk = hist + HIST_WORDS;
+    uint16_t *li = reinterpret_cast<uint16_t *>(lk + cap);
+    // prologue scratch: the first 256 bytes of warp 0's histogram
     long long *s_wsum = reinterpret_cast<long long *>(smem + PairSmem<T>::col_bytes(npad, CS));
 
     const ColInfo cinfo = a.ci[j];
@@ -1203,11 +1127,9 @@ __device__ void pairs_unit(const ScanArgs<T> &a, const LamView &lp, int t0, int 
     }
     // per-lambda thresholds of the exact test depend on (jhat, lambda) only
     for (int tl = threadIdx.x; tl < min(nlc, NDEC); tl += blockDim.x)
-        decide_init<T>(s_dec[tl], cinfo, lp.lam[tl]);
-#if L1L_DYNAMIC_K
+        s_dec[tl].set(cinfo, lp.lam[tl]);
     __shared__ int s_knext;  // next k of this unit (offset from k0)
     if (threadIdx.x == 0) s_knext = 0;
-#endif
     __syncthreads();
     WarpCtx<T> wc;
     wc.colb = colb;
@@ -1217,8 +1139,8 @@ __device__ void pairs_unit(const ScanArgs<T> &a, const LamView &lp, int t0, int 
     wc.lk = lk;
     wc.li = li;
     wc.hist = hist;
-    wc.lst = lst;
-    wc.hist32 = hist32;
+    wc.srow = L1L_CHK((int)samp[2 * lane + 1], npad);
+    wc.sinv = inv[wc.srow];
     wc.s_dec = s_dec;
     wc.qt = cap / 32;
     wc.d0 = a.d0;
@@ -1226,19 +1148,14 @@ __device__ void pairs_unit(const ScanArgs<T> &a, const LamView &lp, int t0, int 
     wc.cinfo = cinfo;
 
     const bool jwide = (cinfo.flags & COL_WIDE) != 0;
-#if L1L_DYNAMIC_K
     // a warp takes the next k when it is done with its pair: pairs cost
     // different times (bracket misses, overflows), and a fixed share per warp
     // leaves the CTA waiting for its slowest warp
-    (void)nw;
     for (;;) {
         int idx = 0;
         if (lane == 0) idx = atomicAdd(&s_knext, 1);
         const int64_t k = k0 + __shfl_sync(0xFFFFFFFFu, idx, 0);
         if (k >= k1) break;
-#else
-    for (int64_t k = k0 + warp; k < k1; k += nw) {
-#endif
         if (k == j) {  // v_jhat = 1: zero residual, penalty lambda * 1
             for (int tl = lane; tl < nlc; tl += 32) {
                 int64_t o = L1L_CHK(((int64_t)(t0 + tl) * m + j) * m + k,
