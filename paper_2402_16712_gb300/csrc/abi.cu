@@ -379,7 +379,7 @@ int path_count_impl(const T *X, int64_t n, int64_t m, int64_t *offsets, void *ws
     L1L_TRY(scan_pairs<T>(c, &k_zero_lambda, 1, nullptr, m));  // lambda = 0 medians
     if (launch_path<T>(true, c.a.Xt, c.a.Xf, c.a.ci, n, m, c.a.ldn, c.a.v_all, offsets,
                        reinterpret_cast<int64_t *>(c.base + P.scan_tmp), nullptr, nullptr, nullptr,
-                       nullptr, nullptr, nullptr, nullptr, c.a.status, c.sms, c.st,
+                       nullptr, nullptr, nullptr, nullptr, nullptr, c.a.status, c.sms, c.st,
                        c.launches) !=
         cudaSuccess)
         return L1L_ERR_CUDA;
@@ -406,7 +406,9 @@ int path_write_impl(const T *X, int64_t n, int64_t m, const int64_t *offsets, do
                        reinterpret_cast<const float *>(base + P.L.Xf),
                        reinterpret_cast<const ColInfo *>(base + P.L.colinfo), n, m, P.L.ldn,
                        reinterpret_cast<const T *>(base + P.L.v_all),
-                       const_cast<int64_t *>(offsets), nullptr, out_lam, out_v, out_res, out_len,
+                       const_cast<int64_t *>(offsets), nullptr, out_lam, out_v, out_res,
+                       // the count call's objectives have served their purpose
+                       reinterpret_cast<float *>(base + P.L.z_all), out_len,
                        reinterpret_cast<int32_t *>(base + P.big),
                        reinterpret_cast<uint32_t *>(base + P.big_count), base + P.scratch,
                        reinterpret_cast<uint32_t *>(base + P.L.status), sms,

@@ -16,7 +16,28 @@
 // sorts them, and each run of equal keys writes its entry; pairs with more
 // rows than the list holds are queued for a second kernel that does the same
 // with a list in global scratch.
+//
+// Both passes look at a row with one multiply-add and two compares, four rows
+// per lane and step: z = x_ik / x_ijhat - c, approximately, tells the rows
+// that are certainly below or above the range; the few others (3% of the rows
+// at 1000 x 500) are queued and divided 32 at a time.
+//
+// Residuals R(t) = sum_i |x_ik - t x_ijhat| of the entries: R(0) is column
+// k's total, and between 0 and t only the rows of the range change sign, so
+//     t > 0:  R(t) = R(0) - 2 B(0, t] + t (2 S(t) - Q)
+//     t < 0:  R(t) = R(0) - 2 B(t, 0) + t (2 S(t) - Q)
+// with B the sum of |x_ik| over the rows whose ratio lies there.  All of them
+// are sums of fixed-point integers (column k's and column jhat's), exact
+// whatever the order; what truncation to those drops (double input; float input
+// only beyond 37 binary orders) is summed beside them in float, in units of the
+// last place.  (The five
+// double sums over all rows that gave R before made the double pipe, two
+// operations per SM and cycle, the bound: 1000 x 500 float with residuals,
+// write pass 5.07 -> 0.76 ms.  Without them, 2000 x 400: 1.33 -> 0.70 ms,
+// count pass 0.42 -> 0.22 ms.)  The write pass is bound by instructions, a
+// quarter of them the rows', the rest the sort and the prefix sums of the list.
 #include <cmath>
+#include <type_traits>
 
 #include "checks.cuh"
 #include "common.cuh"
@@ -29,6 +50,8 @@ namespace {
 
 constexpr int PW = 8;          // warps per CTA
 constexpr int PATH_CAP = 256;  // shared-memory list entries per warp
+constexpr int PATH_CAP_MIN = 128;  // where the column leaves no room for that
+constexpr int PEND = 64;       // rows queued for the exact division, per warp
 
 template <typename T> struct PathArgs {
     const T *Xt;
@@ -41,6 +64,7 @@ template <typename T> struct PathArgs {
     double *lam;           // write pass outputs
     T *val;
     double *res;           // optional: residual sum_i |x_ik - v x_ijhat| of each entry
+    float *crem;           // with residuals, double input: [m] remainders of a column's total
     int32_t *len;          // [m*m]
     int32_t *big;          // pairs whose rows exceed the warp list
     uint32_t *big_count;
@@ -50,46 +74,17 @@ template <typename T> struct PathArgs {
     uint32_t *status;
 };
 
-// Double sums of one pass for the residual R(t) = sum_i |x_ik - t x_ijhat|,
-// which for t a ratio value is  Btot - 2 B(t) + t (2 A(t) - Wv) + C0  with
-// A(t), B(t) the sums of |x_ijhat| and sgn(x_ijhat) x_ik over valid rows whose
-// ratio is <= t, Btot, Wv their totals and C0 the sum of |x_ik| over rows with
-// x_ijhat = 0 (|x_ijhat| (r_i - t) = sgn(x_ijhat) x_ik - t |x_ijhat|).
-struct RowSums {
-    double Btot, Wv, C0, Ab, Bb;  // Ab, Bb: over the rows below the range
-};
-
 // Classification of one row against the range between 0 and v0 (exclusive
-// of 0): -1 below it (exact weight counts in S), 0 inside, +1 above.
-// kexact receives the exact key when it was computed (else NONE).  x_ik is
-// read through xkp only when the exact key is needed.
-template <typename T>
-__device__ __forceinline__ int classify(float xf, float inv, const T *xkp, T xj, bool wide,
-                                        bool pos,
-                                        uint32_t ck_lo, uint32_t ck_hi,
-                                        typename Traits<T>::K kv,
-                                        typename Traits<T>::K &kexact) {
-    using Tr = Traits<T>;
-    using K = typename Tr::K;
-    constexpr uint32_t G = Approx<T>::G;
-    kexact = Tr::NONE;
-    if (!wide) {
-        const uint32_t kk = akey(__fmul_rn(xf, inv));
-        // certain when the approximate coarse key is more than G from both
-        // ends of the coarse range (the coarse image is monotone in the key)
-        if (kk > ck_lo + G && kk + G < ck_hi) return 0;
-        if (kk + G < ck_lo) return -1;
-        if (kk > ck_hi + G) return 1;
-    }
-    const K ke = Tr::key(Tr::div_rn(*xkp, xj));
-    kexact = ke;
+// of 0) by its exact key: -1 below it, 0 inside, +1 above.
+template <typename K>
+__device__ __forceinline__ int classify(K ke, K kv, K key0, bool pos) {
     if (pos) {  // range (KEY0, kv]
-        if (ke <= Tr::KEY0) return -1;
+        if (ke <= key0) return -1;
         return ke <= kv ? 0 : 1;
     }
     // range [kv, KEY0)
     if (ke < kv) return -1;
-    return ke < Tr::KEY0 ? 0 : 1;
+    return ke < key0 ? 0 : 1;
 }
 
 // Coarse-key range of (0, v0] or [v0, 0), and its exact upper/lower key.
@@ -108,19 +103,111 @@ __device__ __forceinline__ void range_of(T v0, bool &pos, uint32_t &ck_lo, uint3
     }
 }
 
-// Stage column jhat (x, float reciprocal, fixed-point weight) into shared memory.
+// What fixq(w, sigma) truncates, in units of 2^-sigma (double w; [0, 1)).
+__device__ __forceinline__ float fix_rem(double w, int sigma) {
+    const uint64_t u = (uint64_t)__double_as_longlong(w) & 0x7FFFFFFFFFFFFFFFull;
+    const int be = (int)(u >> 52);
+    uint64_t f = u & 0xFFFFFFFFFFFFFull;
+    if (be) f |= 0x10000000000000ull;
+    const int rs = 1075 - sigma - (be ? be : 1);
+    if (rs <= 0 || rs > 120) return 0.0f;
+    if (rs < 64) f &= (1ull << rs) - 1ull;
+    return (float)f * __int_as_float((127 - rs) << 23);
+}
+
+// Whether the remainders are summed: double input with residuals.
+template <typename T> __device__ __forceinline__ bool with_rem(const PathArgs<T> &a) {
+    return sizeof(T) == 8 && a.res != nullptr;
+}
+
+// The column arrays of jhat: float reciprocal, fixed-point weight, and x
+// itself (float input) or the weight's remainder (double input, which reads x
+// from the column copy: a few rows per pair).
+template <typename T> struct Column {
+    const T *x;
+    float *inv;
+    int64_t *q;
+    float *rem;
+};
+
+// Stage them by `nt` threads; `own` holds x or the remainders.
 template <typename T>
-__device__ void stage_column(const PathArgs<T> &a, int64_t j, T *colb, float *inv, int64_t *colq,
-                             int npad) {
+__device__ Column<T> stage_column(const PathArgs<T> &a, int64_t j, float *own, float *inv,
+                                  int64_t *colq, int npad, int t, int nt) {
     const ColInfo ci = a.ci[j];
     const T *xj = a.Xt + j * a.ldn;
-    for (int i = threadIdx.x; i < npad; i += blockDim.x) {
+    for (int i = t; i < npad; i += nt) {
         const T b = i < a.n ? xj[i] : T(0);
-        colb[i] = b;
-        inv[i] = b != T(0) ? Approx<T>::inv_of(b) : 0.0f;
+        if constexpr (sizeof(T) == 4)
+            own[i] = b;
+        else
+            own[i] = with_rem(a) ? fix_rem(b, ci.sigma) : 0.0f;
+        // NaN: neither inside, below nor above any range
+        inv[i] = b != T(0) ? Approx<T>::inv_of(b) : __int_as_float(0x7FFFFFFF);
         int e = 0;
         colq[i] = b != T(0) ? fixq(b < T(0) ? -b : b, ci.sigma, e) : 0;
     }
+    if constexpr (sizeof(T) == 4)
+        return Column<T>{own, inv, colq, nullptr};
+    else
+        return Column<T>{xj, inv, colq, own};
+}
+
+// Remainder of each column's fixed-point total.
+template <typename T> __global__ void __launch_bounds__(256) k_colrem(PathArgs<T> a) {
+    if constexpr (sizeof(T) == 8) {
+        __shared__ float sm[8];
+        const T *x = a.Xt + (int64_t)blockIdx.x * a.ldn;
+        const int sigma = a.ci[blockIdx.x].sigma;
+        float s = 0.0f;
+        for (int64_t i = threadIdx.x; i < a.n; i += 256) s += fix_rem(x[i], sigma);
+        s = warp_sum_f32(s);
+        if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = s;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int q = 1; q < 8; ++q) s += sm[q];
+            a.crem[blockIdx.x] = s;
+        }
+    }
+}
+
+// The list's sums of one pair: the weight below the range and the |x_ik| in
+// it, in fixed point and the remainders of both.
+struct ListSums {
+    int64_t Sbelow, Ball;
+    float Srem, Brem;
+};
+
+// Sort of up to 64 (key, row) by one warp: every lane counts the entries
+// before its own two (ties by list position) and puts them there.  Up to 64
+// entries that is fewer instructions than the bitonic network below.
+template <typename K> __device__ void warp_rank_sort(K *keys, uint32_t *rows, int c, int lane) {
+    const int l2 = lane + 32;
+    const K k0 = lane < c ? keys[lane] : (K)~(K)0, k1 = l2 < c ? keys[l2] : (K)~(K)0;
+    const uint32_t r0 = lane < c ? rows[lane] : 0u, r1 = l2 < c ? rows[l2] : 0u;
+    int p0 = 0, p1 = 0;
+    if (c <= 32) {
+        for (int q = 0; q < c; ++q) {
+            const K kq = keys[q];
+            p0 += kq < k0 || (kq == k0 && q < lane) ? 1 : 0;
+        }
+    } else {
+        for (int q = 0; q < c; ++q) {
+            const K kq = keys[q];
+            p0 += kq < k0 || (kq == k0 && q < lane) ? 1 : 0;
+            p1 += kq < k1 || (kq == k1 && q < l2) ? 1 : 0;
+        }
+    }
+    __syncwarp();
+    if (lane < c) {
+        keys[p0] = k0;
+        rows[p0] = r0;
+    }
+    if (l2 < c) {
+        keys[p1] = k1;
+        rows[p1] = r1;
+    }
+    __syncwarp();
 }
 
 // Warp bitonic sort of (key, row) over P (power of two) entries of a list;
@@ -152,19 +239,40 @@ __device__ void warp_list_sort(K *keys, uint32_t *rows, int c, int P, int lane) 
     }
 }
 
+// D 2^-sigma rounded to double, |D| < 2^63.  Normalised, rounded (to nearest,
+// ties to even) and scaled in integer instructions: the conversion and the
+// scaling on the double pipe (2 results per SM and cycle) cost twice as much.
 __device__ __forceinline__ double fix_to_double(int64_t D, int sigma) {
-    return scalbn((double)D, -sigma);
+    if (sigma < -900 || sigma > 900) return scalbn((double)D, -sigma);
+    const uint64_t u = (uint64_t)(D < 0 ? -D : D);
+    const int lz = __clzll((long long)u);
+    const uint64_t f = u << (lz & 63);
+    uint64_t m = f >> 11;  // 53 bits, the leading one at bit 52
+    const uint32_t rest = (uint32_t)f & 0x7FFu;
+    m += rest > 0x400u || (rest == 0x400u && (m & 1u)) ? 1u : 0u;
+    // the leading bit adds the last 1 to the exponent
+    const uint64_t r = ((uint64_t)(1085 - lz - sigma) << 52) + m;
+    const uint64_t sg = (uint64_t)D & 0x8000000000000000ull;
+    return __longlong_as_double((long long)(u == 0 ? 0ull : (r | sg)));
+}
+
+// sum_i |x_i| of a column (rem: of a double column's fixed-point total).
+__device__ __forceinline__ double column_total(const ColInfo &c, float rem) {
+    const double t = fix_to_double(c.Q, c.sigma);
+    return rem == 0.0f ? t : t + scalbn((double)rem, -c.sigma);
 }
 
 // Entries of one pair from its sorted in-range list (c > 0 rows).
 template <typename T>
 __device__ void emit_path(const PathArgs<T> &a, int64_t p, T v0, bool pos,
                           const typename Traits<T>::K *keys, const uint32_t *rows, int c,
-                          const int64_t *colq, int64_t Q, int64_t Sbelow, int sigma,
-                          const T *colb, const T *xk, const RowSums &rs, int lane) {
+                          const Column<T> &col, const ColInfo &cj, const ColInfo &ck,
+                          const ListSums &ls, float remj, float remk, const T *xk, int lane) {
     using Tr = Traits<T>;
-    using K = typename Tr::K;
+    // corrections of a run: double input's lie below the fixed point's units
+    using QC = typename std::conditional<sizeof(T) == 4, int64_t, float>::type;
     const unsigned FULL = 0xFFFFFFFFu;
+    const int64_t Q = cj.Q;
     const int64_t o = a.off[p];
     const int64_t room = a.off[p + 1] - o;  // entries the count pass reserved
     // number of runs of equal keys
@@ -176,64 +284,99 @@ __device__ void emit_path(const PathArgs<T> &a, int64_t p, T v0, bool pos,
     }
     // the entries 0 .. groups lie inside the room the count pass reserved
     L1L_CHK((int64_t)groups, room);
-    int64_t carry = Sbelow;  // S at the end of the previous chunk
-    double cA = rs.Ab, cB = rs.Bb;  // residual sums at the end of the previous chunk
-    double cQrun = 0.0;             // corrections of the run open at the chunk's end
+    int64_t carry = ls.Sbelow;  // S at the end of the previous chunk
+    int64_t cB = 0;          // B of the list up to there
+    float cSr = ls.Srem, cBr = 0.0f;  // remainders of both
+    QC crun = 0;             // corrections of the run open at the chunk's end
     int gbase = 0;           // runs ended before this chunk
     for (int i0 = 0; i0 < c; i0 += 32) {
         const int i = i0 + lane;
-        const int64_t q = i < c ? colq[rows[i]] : 0;
+        const uint32_t row = i < c ? rows[i] : 0u;
+        const int64_t q = i < c ? col.q[row] : 0;
         const int64_t S = carry + warp_scan_add(q, lane);  // S(key_i) at a run end
         const bool end = i < c && (i == c - 1 || keys[i] != keys[i + 1]);
         const unsigned em = __ballot_sync(FULL, end);
         const int g = gbase + __popc(em & ((1u << lane) - 1u));  // run index (ascending)
+        const int64_t D = 2 * S - Q;
+        const double Dd = fix_to_double(D, cj.sigma);
         if (a.res) {
-            // A, B: prefix sums through this row.  The formula counts the
-            // rows of t's own run as "ratio <= t"; a row whose exact ratio
-            // lies above its rounded value t then enters with the wrong sign,
-            // so each row of the run adds the correction
-            // qc = |x - t b| - (t |b| - sgn(b) x), summed over the run.
-            double w = 0.0, sx = 0.0, qc = 0.0, t = 0.0;
+            // The formula counts the rows of t's own run as "ratio <= t"; a
+            // row whose exact ratio lies above its rounded value t then enters
+            // with the wrong sign, so each row of the run adds the correction
+            // |x - t b| - (t |b| - sgn(b) x) = 2 max(sgn(b) x - t |b|, 0).
+            int64_t xq = 0;
+            QC qc = 0;
+            T t = T(0);
+            float wr = 0.0f, xr = 0.0f;
             if (i < c) {
-                const double b = (double)colb[rows[i]], x = (double)xk[rows[i]];
-                t = (double)Tr::value(keys[i]);
-                w = fabs(b);
-                sx = b < 0.0 ? -x : x;
-                qc = fabs(x - t * b) - (t * w - sx);
+                const T b = col.x[row], x = xk[row];
+                const T sx = b < T(0) ? -x : x;
+                t = Tr::value(keys[i]);
+                int e = 0;
+                xq = fixq(fabs(x), ck.sigma, e);
+                // the remainder of a correctly rounded division is exact in
+                // its operands' precision unless it underflows: float rows
+                // that small take it in double
+                if constexpr (sizeof(T) == 8) {
+                    const T d = fma(-t, fabs(b), sx);
+                    if (d > T(0)) qc = (float)scalbn(2.0 * d, ck.sigma);
+                    wr = col.rem[row];
+                    xr = fix_rem(x, ck.sigma);
+                } else if (fabs(x) >= T(0x1p-100)) {
+                    const T d = fma(-t, fabs(b), sx);
+                    if (d > T(0)) qc = fixq(T(2) * d, ck.sigma, e);
+                } else {
+                    const double d = fma(-(double)t, fabs((double)b), (double)sx);
+                    if (d > 0.0) qc = fixq(2.0 * d, ck.sigma, e);
+                }
             }
-            const double A = cA + warp_scan_add(w, lane), B = cB + warp_scan_add(sx, lane);
-            const double Qi = warp_scan_add(qc, lane);  // inclusive, this chunk only
-            // run sums of qc: the run's start holds the prefix before it
-            const bool start = i < c && (i == 0 || keys[i - 1] != keys[i]);
-            const unsigned smk = __ballot_sync(FULL, start);
-            const double Qs = Qi - qc;  // chunk prefix before this row
-            const unsigned upto = smk & (lane == 31 ? FULL : ((2u << lane) - 1u));
-            const int hs = upto ? 31 - __clz(upto) : -1;
-            const double Qstart = __shfl_sync(FULL, Qs, hs < 0 ? 0 : hs);
-            // the run began in an earlier chunk: its prefix is cQ - cQrun
-            const double run_q = hs >= 0 ? Qi - Qstart : cQrun + Qi;
+            float Sr = 0.0f, Br = 0.0f;
+            if constexpr (sizeof(T) == 8) {
+                Sr = cSr + warp_scan_add(wr, lane);
+                Br = cBr + warp_scan_add(xr, lane);
+                cSr = __shfl_sync(FULL, Sr, 31);
+                cBr = __shfl_sync(FULL, Br, 31);
+            }
+            const int64_t B = cB + warp_scan_add(xq, lane);
+            QC run_q = 0;
+            if (__any_sync(FULL, qc != 0) || crun != 0) {
+                const QC Qi = warp_scan_add(qc, lane);  // inclusive, this chunk only
+                // run sums of qc: the run's start holds the prefix before it
+                const bool start = i < c && (i == 0 || keys[i - 1] != keys[i]);
+                const unsigned smk = __ballot_sync(FULL, start);
+                const unsigned upto = smk & (lane == 31 ? FULL : ((2u << lane) - 1u));
+                const int hs = upto ? 31 - __clz(upto) : -1;
+                const QC Qstart = __shfl_sync(FULL, Qi - qc, hs < 0 ? 0 : hs);
+                // the run began in an earlier chunk: its corrections are in crun
+                run_q = hs >= 0 ? Qi - Qstart : crun + Qi;
+            }
             if (end) {  // each run writes the residual of its own entry
                 const int slot = pos ? groups - 1 - g : g;
-                a.res[o + slot] = rs.Btot - 2.0 * B + t * (2.0 * A - rs.Wv) + rs.C0 + run_q;
+                int64_t F = ck.Q - 2 * (pos ? B : ls.Ball - B);
+                if constexpr (sizeof(T) == 4) {
+                    F += run_q;
+                    a.res[o + slot] = fma((double)t, Dd, fix_to_double(F, ck.sigma));
+                } else {
+                    const float fr = remk - 2.0f * (pos ? Br : ls.Brem - Br) + run_q;
+                    const double dr = scalbn((double)(2.0f * Sr - remj), -cj.sigma);
+                    a.res[o + slot] = fma(t, Dd + dr, fix_to_double(F, ck.sigma) +
+                                                          scalbn((double)fr, -ck.sigma));
+                }
             }
             // the run still open at the end of this chunk carries its partial sum
-            const double last = __shfl_sync(FULL, run_q, 31);
-            cQrun = last;
-            cA = __shfl_sync(FULL, A, 31);
+            crun = __shfl_sync(FULL, run_q, 31);
             cB = __shfl_sync(FULL, B, 31);
         }
         if (end) {
             if (pos) {
                 // run g (not the top one) starts at Q - 2 S(t_g), slot groups-1-g
                 if (g < groups - 1) {
-                    const int64_t D = Q - 2 * S;
-                    a.lam[o + groups - 1 - g] = D > 0 ? fix_to_double(D, sigma) : 0.0;
+                    a.lam[o + groups - 1 - g] = D < 0 ? -Dd : 0.0;
                     a.val[o + groups - 1 - g] = Tr::value(keys[i]);
                 }
             } else {
                 // the run after g starts at 2 S(t_g) - Q; after the last, 0
-                const int64_t D = 2 * S - Q;
-                a.lam[o + g + 1] = D > 0 ? fix_to_double(D, sigma) : 0.0;
+                a.lam[o + g + 1] = D > 0 ? Dd : 0.0;
                 a.val[o + g + 1] = g + 1 < groups ? Tr::value(keys[i + 1]) : T(0);
             }
         }
@@ -244,101 +387,137 @@ __device__ void emit_path(const PathArgs<T> &a, int64_t p, T v0, bool pos,
         a.lam[o] = 0.0;
         a.val[o] = v0;
         if (pos) {
-            const int64_t D = Q - 2 * Sbelow;
-            a.lam[o + groups] = D > 0 ? fix_to_double(D, sigma) : 0.0;
+            const int64_t D = Q - 2 * ls.Sbelow;
+            a.lam[o + groups] = D > 0 ? fix_to_double(D, cj.sigma) : 0.0;
             a.val[o + groups] = T(0);
         }
-        // v = 0: R = Btot - 2 B(0) + C0 with B(0) the signed sum over ratios <= 0
-        if (a.res) a.res[o + groups] = rs.Btot - 2.0 * (pos ? rs.Bb : cB) + rs.C0;
+        if (a.res) a.res[o + groups] = column_total(ck, remk);  // v = 0
         a.len[p] = groups + 1;
     }
 }
 
-// One pass over the rows of pair (j, k) by one warp.  COUNT: rows in range.
-// Else: append in-range rows (exact key, row) to the list (at most cap; the
-// total is returned either way) and sum the exact weight below the range.
-// Without residual sums the rows are visited four per lane per step, the
-// step's loads of the float copy issued together (measured 14% faster for the
-// count and write passes); with them, one per lane per step (the double sums
-// bound that pass, and the wider step measured 3% slower).
+// One pass over the rows of pair (j, k) by one warp; returns the number of
+// rows in range.  Unless COUNT: appends them (exact key, row) to the list (at
+// most cap; the total is returned either way), sums the exact weight below the
+// range and, with residuals, the fixed-point |x_ik| of the range.  The column
+// arrays hold a multiple of 128 rows, zero past n.
 template <typename T, bool COUNT>
-__device__ int scan_rows(const PathArgs<T> &a, int64_t j, int64_t k, const T *colb,
-                         const float *inv, const int64_t *colq, bool wide, bool pos,
-                         uint32_t ck_lo, uint32_t ck_hi, typename Traits<T>::K kv,
-                         typename Traits<T>::K *keys, uint32_t *rows, int cap, int64_t &Sbelow,
-                         RowSums &rs, int lane) {
+__device__ int scan_rows(const PathArgs<T> &a, int64_t k, const Column<T> &col, uint16_t *pend,
+                         bool wide, bool pos, uint32_t ck_lo, uint32_t ck_hi,
+                         typename Traits<T>::K kv, int sigma_k, typename Traits<T>::K *keys,
+                         uint32_t *rows, int cap, ListSums &ls, int lane) {
     using Tr = Traits<T>;
     using K = typename Tr::K;
+    constexpr uint32_t G = Approx<T>::G;
     const unsigned FULL = 0xFFFFFFFFu;
     const T *xk = a.Xt + k * a.ldn;
-    const float *xf = a.Xf + k * a.ldn;
+    const float4 *xf = reinterpret_cast<const float4 *>(a.Xf + k * a.ldn);
+    const int ng = ((int)a.n + 127) >> 7;
     const bool want_r = !COUNT && a.res != nullptr;
-    const int n = (int)a.n;
-    int c = 0;
-    int64_t sb = 0;
-    // one row: classify, weight below, exact key, list append
-    auto visit = [&](int i, float xv, double *sums) {
-        const bool inb = i < n;
+    // Rows with a coarse key outside [ck_lo - G, ck_hi + G] are certainly
+    // below or above; [va, vb] holds the ratios of the others, and |fma(x,
+    // inv, -cen)| differs from |fl(x inv) - cen| by at most 3 roundings of
+    // 2^-24 of the larger end.  Every row is queued where that means nothing:
+    // a wide column, or a range that reaches the infinities.
+    const float va = akey_value(sat_sub(ck_lo, G)), vb = akey_value(sat_add(ck_hi, G));
+    const float cen = 0.5f * va + 0.5f * vb;
+    float delta = (0.5f * vb - 0.5f * va) * (1.0f + 0x1p-20f) +
+                  0x1p-21f * fmaxf(fabsf(va), fabsf(vb)) + 0x1p-148f;
+    const bool all = wide || !(delta < 0x1p126f) || !(fabsf(cen) < 0x1p126f);
+    int c = 0, np = 0;
+    int64_t sb = 0, bl = 0;
+    float sr = 0.0f, br = 0.0f;  // their remainders
+    const bool want_rem = !COUNT && with_rem(a);
+    // the queue's first 32 rows (fewer at the end): exact keys, list append
+    auto flush = [&](int cnt) {
         int cls = 1;
         K ke = Tr::NONE;
-        const T b = inb ? colb[i] : T(0);
-        const bool valid = b != T(0);
-        if (valid) cls = classify<T>(xv, inv[i], xk + i, b, wide, pos, ck_lo, ck_hi, kv, ke);
-        if (!COUNT) {
-            if (cls < 0) sb += colq[i];
-            if (cls == 0 && ke == Tr::NONE) ke = Tr::key(Tr::div_rn(xk[i], b));
+        const int i = L1L_CHK(lane < cnt ? (int)pend[lane] : 0, ng * 128);
+        const T b = col.x[i];
+        T x = T(0);
+        if (lane < cnt && b != T(0)) {
+            x = xk[i];
+            ke = Tr::key(Tr::div_rn(x, b));
+            cls = classify<K>(ke, kv, Tr::KEY0, pos);
         }
-        if (sums && inb) {  // bt, wv, c0, ab, bb of RowSums
-            // float input: the float copy is the input itself
-            const double x = sizeof(T) == 4 ? (double)xv : (double)xk[i];
-            const double bd = (double)b;
-            if (valid) {
-                const double sx = bd < 0.0 ? -x : x;
-                sums[0] += sx;
-                sums[1] += fabs(bd);
-                if (cls < 0) {
-                    sums[3] += fabs(bd);
-                    sums[4] += sx;
-                }
-            } else {
-                sums[2] += fabs(x);
-            }
+        if (!COUNT && cls < 0) {
+            sb += col.q[i];
+            if (want_rem) sr += col.rem[i];
         }
         const unsigned im = __ballot_sync(FULL, cls == 0);
         if (!COUNT && cls == 0) {
-            const int pos_i = c + __popc(im & ((1u << lane) - 1u));
-            if (pos_i < cap) {
-                keys[pos_i] = ke;
-                rows[pos_i] = (uint32_t)i;
+            const int at = c + __popc(im & ((1u << lane) - 1u));
+            if (at < cap) {
+                keys[at] = ke;
+                rows[at] = (uint32_t)i;
             }
+            int e = 0;
+            if (want_r) bl += fixq(fabs(x), sigma_k, e);
+            if constexpr (sizeof(T) == 8)
+                if (want_rem) br += fix_rem(x, sigma_k);
         }
         c += __popc(im);
     };
-    if (want_r) {
-        double sums[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-        for (int i0 = 0; i0 < n; i0 += 32) {
-            const int i = i0 + lane;
-            visit(i, i < n ? xf[i] : 0.0f, sums);
-        }
-        rs.Btot = warp_sum_f64(sums[0]);
-        rs.Wv = warp_sum_f64(sums[1]);
-        rs.C0 = warp_sum_f64(sums[2]);
-        rs.Ab = warp_sum_f64(sums[3]);
-        rs.Bb = warp_sum_f64(sums[4]);
-    } else {
-        constexpr int U = 4;
-        for (int i0 = 0; i0 < n; i0 += 32 * U) {
-            float xv[U];
+    for (int g0 = 0; g0 < ng; g0 += 8) {  // 8 groups: one byte of flags per row of the lane
+        const int ge = min(ng, g0 + 8);
+        uint32_t mask = 0;  // bit 4 (g - g0) + u: row u of the lane in group g
+        float4 xn = __ldg(xf + g0 * 32 + lane);
+        for (int g = g0; g < ge; ++g) {
+            const float4 x4 = xn;
+            if (g + 1 < ge) xn = __ldg(xf + (g + 1) * 32 + lane);
+            const int i = L1L_CHK(g * 128 + 4 * lane, ng * 128);
+            const float4 v4 = *reinterpret_cast<const float4 *>(col.inv + i);
+            const float z[4] = {fmaf(x4.x, v4.x, -cen), fmaf(x4.y, v4.y, -cen),
+                                fmaf(x4.z, v4.z, -cen), fmaf(x4.w, v4.w, -cen)};
+            uint32_t f = 0;
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int i = i0 + u * 32 + lane;
-                xv[u] = i < n ? xf[i] : 0.0f;
+            for (int u = 0; u < 4; ++u)
+                if (fabsf(z[u]) < delta) f |= 1u << u;
+            if (!COUNT && !all) {
+                const longlong2 qa = *reinterpret_cast<const longlong2 *>(col.q + i);
+                const longlong2 qb = *reinterpret_cast<const longlong2 *>(col.q + i + 2);
+                if (z[0] <= -delta) sb += qa.x;
+                if (z[1] <= -delta) sb += qa.y;
+                if (z[2] <= -delta) sb += qb.x;
+                if (z[3] <= -delta) sb += qb.y;
+                if (want_rem) {
+                    const float4 r4 = *reinterpret_cast<const float4 *>(col.rem + i);
+                    if (z[0] <= -delta) sr += r4.x;
+                    if (z[1] <= -delta) sr += r4.y;
+                    if (z[2] <= -delta) sr += r4.z;
+                    if (z[3] <= -delta) sr += r4.w;
+                }
             }
-#pragma unroll
-            for (int u = 0; u < U; ++u) visit(i0 + u * 32 + lane, xv[u], nullptr);
+            mask |= f << (4 * (g - g0));
+        }
+        if (all) mask = ge - g0 == 8 ? FULL : (1u << (4 * (ge - g0))) - 1u;
+        unsigned m;
+        while ((m = __ballot_sync(FULL, mask != 0)) != 0) {
+            if (mask != 0) {
+                const int bit = __ffs(mask) - 1;
+                mask &= mask - 1;
+                const int at = L1L_CHK(np + __popc(m & ((1u << lane) - 1u)), PEND);
+                pend[at] = (uint16_t)((g0 + (bit >> 2)) * 128 + 4 * lane + (bit & 3));
+            }
+            np += __popc(m);
+            __syncwarp();
+            if (np >= 32) {
+                flush(32);
+                const uint16_t up = pend[32 + lane];
+                __syncwarp();
+                pend[lane] = up;
+                np -= 32;
+                __syncwarp();
+            }
         }
     }
-    if (!COUNT) Sbelow = warp_sum_i64(sb);
+    if (np > 0) flush(np);
+    if (!COUNT) {
+        ls.Sbelow = warp_sum_i64(sb);
+        ls.Ball = want_r ? warp_sum_i64(bl) : 0;
+        ls.Srem = want_rem ? warp_sum_f32(sr) : 0.0f;
+        ls.Brem = want_rem ? warp_sum_f32(br) : 0.0f;
+    }
     __syncwarp();
     return c;
 }
@@ -349,35 +528,32 @@ __device__ __forceinline__ bool pair_is_wide(const PathArgs<T> &a, const ColInfo
 }
 
 template <typename T, bool COUNT>
-__global__ void __launch_bounds__(PW * 32) k_path_pass(PathArgs<T> a, int kchunk) {
+__global__ void __launch_bounds__(PW * 32) k_path_pass(PathArgs<T> a, int kchunk, int cap) {
     using Tr = Traits<T>;
     using K = typename Tr::K;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int npad = ((int)a.n + 31) & ~31;
-    T *colb = reinterpret_cast<T *>(smem);
-    size_t o = al16((size_t)npad * sizeof(T));
+    const int npad = ((int)a.n + ROW_PAD - 1) & ~(ROW_PAD - 1);
+    float *own = reinterpret_cast<float *>(smem);
+    size_t o = (size_t)npad * 4;
     float *inv = reinterpret_cast<float *>(smem + o);
-    o += al16((size_t)npad * 4);
+    o += (size_t)npad * 4;
     int64_t *colq = reinterpret_cast<int64_t *>(smem + o);
-    o += al16((size_t)npad * 8);
-    K *keys = reinterpret_cast<K *>(smem + o + (size_t)warp * PATH_CAP * (sizeof(K) + 4));
-    uint32_t *rows = reinterpret_cast<uint32_t *>(keys + PATH_CAP);
+    o += (size_t)npad * 8;
+    uint16_t *pend = reinterpret_cast<uint16_t *>(smem + o) + warp * PEND;
+    o += (size_t)PW * PEND * 2;
+    K *keys = reinterpret_cast<K *>(smem + o + (size_t)warp * cap * (sizeof(K) + 4));
+    uint32_t *rows = reinterpret_cast<uint32_t *>(keys + cap);
     const int64_t j = blockIdx.x;
-    stage_column<T>(a, j, colb, inv, colq, npad);
+    const Column<T> col = stage_column<T>(a, j, own, inv, colq, npad, threadIdx.x, PW * 32);
     __syncthreads();
+    const float remj = with_rem(a) ? a.crem[j] : 0.0f;
     const ColInfo cj = a.ci[j];
     const int64_t k0 = (int64_t)blockIdx.y * kchunk, k1 = min(a.m, k0 + kchunk);
     for (int64_t k = k0 + warp; k < k1; k += PW) {
         const int64_t p = j * a.m + k;
         const T v0 = a.v0[p];
         if (k == j || v0 == T(0) || cj.n_valid == 0) {  // constant path
-            double r = 0.0;  // v = 1 for k == jhat: zero residual; v = 0: sum |x_ik|
-            if (!COUNT && a.res && k != j) {
-                const T *xk = a.Xt + k * a.ldn;
-                for (int i = lane; i < (int)a.n; i += 32) r += fabs((double)xk[i]);
-                r = warp_sum_f64(r);
-            }
             if (lane == 0) {
                 if (COUNT) {
                     a.bound[p] = 1;
@@ -385,7 +561,10 @@ __global__ void __launch_bounds__(PW * 32) k_path_pass(PathArgs<T> a, int kchunk
                     const int64_t off = a.off[p];
                     a.lam[off] = 0.0;
                     a.val[off] = k == j ? T(1) : T(0);
-                    if (a.res) a.res[off] = r;
+                    // v = 1 for k == jhat: zero residual; v = 0: sum |x_ik|
+                    if (a.res)
+                        a.res[off] = k == j ? 0.0
+                                            : column_total(a.ci[k], with_rem(a) ? a.crem[k] : 0.0f);
                     a.len[p] = 1;
                 }
             }
@@ -396,23 +575,27 @@ __global__ void __launch_bounds__(PW * 32) k_path_pass(PathArgs<T> a, int kchunk
         K kv;
         range_of<T>(v0, pos, ck_lo, ck_hi, kv);
         const bool wide = pair_is_wide<T>(a, cj, k);
-        int64_t Sbelow = 0;
-        RowSums rs{};
-        const int c = scan_rows<T, COUNT>(a, j, k, colb, inv, colq, wide, pos, ck_lo, ck_hi, kv,
-                                          keys, rows, PATH_CAP, Sbelow, rs, lane);
+        const ColInfo ck = a.ci[k];
+        ListSums ls{};
+        const int c = scan_rows<T, COUNT>(a, k, col, pend, wide, pos, ck_lo, ck_hi, kv, ck.sigma,
+                                          keys, rows, cap, ls, lane);
         if (COUNT) {
             if (lane == 0) a.bound[p] = (int64_t)c + 1;
             continue;
         }
-        if (c > PATH_CAP) {  // the big-pair kernel takes it
+        if (c > cap) {  // the big-pair kernel takes it
             if (lane == 0) a.big[atomicAdd(a.big_count, 1u)] = (int32_t)(p);
             continue;
         }
-        int P = 32;
-        while (P < c) P <<= 1;
-        warp_list_sort<K>(keys, rows, c, P, lane);
-        emit_path<T>(a, p, v0, pos, keys, rows, c, colq, cj.Q, Sbelow, cj.sigma, colb,
-                     a.Xt + k * a.ldn, rs, lane);
+        if (c <= 64) {
+            warp_rank_sort<K>(keys, rows, c, lane);
+        } else {
+            int P = 128;
+            while (P < c) P <<= 1;
+            warp_list_sort<K>(keys, rows, c, P, lane);
+        }
+        emit_path<T>(a, p, v0, pos, keys, rows, c, col, cj, ck, ls, remj,
+                     with_rem(a) ? a.crem[k] : 0.0f, a.Xt + k * a.ldn, lane);
         __syncwarp();
     }
 }
@@ -423,17 +606,18 @@ template <typename T>
 __global__ void __launch_bounds__(128) k_path_big(PathArgs<T> a) {
     using Tr = Traits<T>;
     using K = typename Tr::K;
+    __shared__ uint16_t s_pend[4][PEND];
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // worker warp
-    const int npad = ((int)a.n + 31) & ~31;
-    unsigned char *sl = a.scratch + (size_t)gw * (size_t)a.slice * (sizeof(K) + 4 + sizeof(T) + 12);
+    const int npad = ((int)a.n + ROW_PAD - 1) & ~(ROW_PAD - 1);
+    unsigned char *sl = a.scratch + (size_t)gw * (size_t)a.slice * (sizeof(K) + 20);
     K *keys = reinterpret_cast<K *>(sl);
     uint32_t *rows = reinterpret_cast<uint32_t *>(keys + a.slice);
     // the column arrays of jhat live in the slice too (each warp may hold a different jhat)
-    T *cb = reinterpret_cast<T *>(rows + a.slice);
-    float *ci_inv = reinterpret_cast<float *>(cb + a.slice);
+    float *own = reinterpret_cast<float *>(rows + a.slice);
+    float *ci_inv = own + a.slice;
     int64_t *cq = reinterpret_cast<int64_t *>(ci_inv + a.slice);
-    const uint32_t total = *a.big_count;
+    const uint32_t total = *a.big_count;  // rows > PATH_CAP_MIN, so a slice holds npad rows
     for (;;) {
         uint32_t w = 0;
         if (lane == 0) w = atomicAdd(a.big_next, 1u);
@@ -441,31 +625,23 @@ __global__ void __launch_bounds__(128) k_path_big(PathArgs<T> a) {
         if (w >= total) break;
         const int64_t p = a.big[w];
         const int64_t j = p / a.m, k = p - j * a.m;
-        const ColInfo cj = a.ci[j];
-        const T *xj = a.Xt + j * a.ldn;
-        for (int i = lane; i < npad; i += 32) {
-            const T b = i < a.n ? xj[i] : T(0);
-            cb[i] = b;
-            ci_inv[i] = b != T(0) ? Approx<T>::inv_of(b) : 0.0f;
-            int e = 0;
-            cq[i] = b != T(0) ? fixq(b < T(0) ? -b : b, cj.sigma, e) : 0;
-        }
+        const ColInfo cj = a.ci[j], ck = a.ci[k];
+        const Column<T> col = stage_column<T>(a, j, own, ci_inv, cq, npad, lane, 32);
         __syncwarp();
         const T v0 = a.v0[p];
         bool pos;
         uint32_t ck_lo, ck_hi;
         K kv;
         range_of<T>(v0, pos, ck_lo, ck_hi, kv);
-        int64_t Sbelow = 0;
-        RowSums rs{};
-        const int c = scan_rows<T, false>(a, j, k, cb, ci_inv, cq, pair_is_wide<T>(a, cj, k), pos,
-                                          ck_lo, ck_hi, kv, keys, rows, (int)a.slice, Sbelow,
-                                          rs, lane);
+        ListSums ls{};
+        const int c = scan_rows<T, false>(a, k, col, s_pend[threadIdx.x >> 5],
+                                          pair_is_wide<T>(a, cj, k), pos, ck_lo, ck_hi, kv,
+                                          ck.sigma, keys, rows, (int)a.slice, ls, lane);
         int P = 32;
         while (P < c) P <<= 1;
         warp_list_sort<K>(keys, rows, c, P, lane);
-        emit_path<T>(a, p, v0, pos, keys, rows, c, cq, cj.Q, Sbelow, cj.sigma, cb,
-                     a.Xt + k * a.ldn, rs, lane);
+        emit_path<T>(a, p, v0, pos, keys, rows, c, col, cj, ck, ls, with_rem(a) ? a.crem[j] : 0.0f,
+                     with_rem(a) ? a.crem[k] : 0.0f, a.Xt + k * a.ldn, lane);
         __syncwarp();
     }
 }
@@ -539,28 +715,31 @@ int path_big_workers() { return 64; }
 template <typename T> size_t path_slice_bytes(int64_t n) {
     int64_t P = 32;
     while (P < n) P <<= 1;
-    return (size_t)P * (sizeof(typename Traits<T>::K) + 4 + sizeof(T) + 12);
+    return (size_t)P * (sizeof(typename Traits<T>::K) + 20);
 }
 
-template <typename T> size_t path_smem_bytes(int64_t n) {
-    const int npad = ((int)n + 31) & ~31;
-    return al16((size_t)npad * sizeof(T)) + al16((size_t)npad * 4) + al16((size_t)npad * 8) +
-           (size_t)PW * PATH_CAP * (sizeof(typename Traits<T>::K) + 4);
+// Shared memory of a CTA with lists of `cap` entries.
+template <typename T> size_t path_smem_bytes(int64_t n, int cap) {
+    const size_t npad = (size_t)((n + ROW_PAD - 1) & ~int64_t(ROW_PAD - 1));
+    return npad * 16 + (size_t)PW * PEND * 2 +
+           (size_t)PW * cap * (sizeof(typename Traits<T>::K) + 4);
 }
 
-// Largest n whose staged column and lists fit one CTA of the path kernels
-// (and that the fit, which solves lambda = 0, accepts).
+// The limit on n is a fixed one (13,504 float, 10,368 double): the rows, in
+// steps of 32, whose x, reciprocal and weight, with full lists, fit 227 KB (and
+// that the fit, which solves lambda = 0, accepts).  Float rows next to it, with
+// their padding to 128 and the queues, get lists of PATH_CAP_MIN.
 template <typename T> int64_t path_max_rows() {
-    int64_t n = 32;
-    while (n + 32 <= max_rows_pairs<T>() && path_smem_bytes<T>(n + 32) <= 227 * 1024) n += 32;
-    return n;
+    const int64_t room = 227 * 1024 - (int64_t)PW * PATH_CAP * (sizeof(typename Traits<T>::K) + 4);
+    const int64_t n = room / (int64_t)(sizeof(T) + 12) & ~int64_t(31);
+    return std::min<int64_t>(n, max_rows_pairs<T>() & ~int64_t(31));
 }
 
 template <typename T>
 cudaError_t launch_path(bool count, const T *Xt, const float *Xf, const ColInfo *ci, int64_t n,
                         int64_t m, int64_t ldn, const T *v0, int64_t *bound_or_off,
-                        int64_t *scan_tmp, double *lam, T *val, double *res, int32_t *len,
-                        int32_t *big, uint32_t *big_count, unsigned char *scratch,
+                        int64_t *scan_tmp, double *lam, T *val, double *res, float *crem,
+                        int32_t *len, int32_t *big, uint32_t *big_count, unsigned char *scratch,
                         uint32_t *status, int num_sms, cudaStream_t st, int &launches) {
     PathArgs<T> a{};
     a.Xt = Xt;
@@ -571,7 +750,8 @@ cudaError_t launch_path(bool count, const T *Xt, const float *Xf, const ColInfo 
     a.ldn = ldn;
     a.v0 = v0;
     a.status = status;
-    const size_t smem = path_smem_bytes<T>(n);
+    const int cap = path_smem_bytes<T>(n, PATH_CAP) <= 227 * 1024 ? PATH_CAP : PATH_CAP_MIN;
+    const size_t smem = path_smem_bytes<T>(n, cap);
     const int64_t chunks = std::max<int64_t>(1, std::min<int64_t>((m + PW - 1) / PW,
                                                                   (num_sms * 8 + m - 1) / m));
     const int kchunk = (int)((m + chunks - 1) / chunks);
@@ -581,7 +761,7 @@ cudaError_t launch_path(bool count, const T *Xt, const float *Xf, const ColInfo 
         a.bound = bound_or_off;
         auto kern = k_path_pass<T, true>;
         if ((e = ensure_smem(reinterpret_cast<const void *>(kern), smem)) != cudaSuccess) return e;
-        kern<<<grid, PW * 32, smem, st>>>(a, kchunk);
+        kern<<<grid, PW * 32, smem, st>>>(a, kchunk, cap);
         launches++;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         // exclusive scan of the m*m bounds, in place, total at [m*m]
@@ -591,6 +771,7 @@ cudaError_t launch_path(bool count, const T *Xt, const float *Xf, const ColInfo 
     a.lam = lam;
     a.val = val;
     a.res = res;
+    a.crem = crem;
     a.len = len;
     a.big = big;
     a.big_count = big_count;
@@ -600,9 +781,14 @@ cudaError_t launch_path(bool count, const T *Xt, const float *Xf, const ColInfo 
     while (P < n) P <<= 1;
     a.slice = P;
     if ((e = cudaMemsetAsync(big_count, 0, 2 * sizeof(uint32_t), st)) != cudaSuccess) return e;
+    if (sizeof(T) == 8 && res) {
+        k_colrem<T><<<(unsigned)m, 256, 0, st>>>(a);
+        launches++;
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
     auto kern = k_path_pass<T, false>;
     if ((e = ensure_smem(reinterpret_cast<const void *>(kern), smem)) != cudaSuccess) return e;
-    kern<<<grid, PW * 32, smem, st>>>(a, kchunk);
+    kern<<<grid, PW * 32, smem, st>>>(a, kchunk, cap);
     launches++;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_path_big<T><<<path_big_workers() / 4, 128, 0, st>>>(a);
@@ -616,13 +802,15 @@ template int64_t path_max_rows<float>();
 template int64_t path_max_rows<double>();
 template cudaError_t launch_path<float>(bool, const float *, const float *, const ColInfo *,
                                         int64_t, int64_t, int64_t, const float *, int64_t *,
-                                        int64_t *, double *, float *, double *, int32_t *,
-                                        int32_t *, uint32_t *, unsigned char *, uint32_t *, int,
+                                        int64_t *, double *, float *, double *, float *,
+                                        int32_t *, int32_t *, uint32_t *, unsigned char *,
+                                        uint32_t *, int,
                                         cudaStream_t, int &);
 template cudaError_t launch_path<double>(bool, const double *, const float *, const ColInfo *,
                                          int64_t, int64_t, int64_t, const double *, int64_t *,
-                                         int64_t *, double *, double *, double *, int32_t *,
-                                         int32_t *, uint32_t *, unsigned char *, uint32_t *, int,
+                                         int64_t *, double *, double *, double *, float *,
+                                         int32_t *, int32_t *, uint32_t *, unsigned char *,
+                                        uint32_t *, int,
                                          cudaStream_t, int &);
 
 L1L_CHECKS_READER(l1l_checks_path)

@@ -156,9 +156,9 @@ template <typename T> int64_t path_max_rows();
 template <typename T>
 cudaError_t launch_path(bool count, const T *Xt, const float *Xf, const ColInfo *ci, int64_t n,
                         int64_t m, int64_t ldn, const T *v0, int64_t *bound_or_off,
-                        int64_t *scan_tmp, double *lam, T *val, double *res, int32_t *len,
-                        int32_t *big, uint32_t *big_count, unsigned char *scratch,
-                        uint32_t *status, int num_sms, cudaStream_t st, int &launches);
+                        int64_t *scan_tmp, double *lam, T *val, double *res, float *crem,
+                        int32_t *len, int32_t *big, uint32_t *big_count,
+                        unsigned char *scratch, uint32_t *status, int num_sms, cudaStream_t st, int &launches);
 
 // A size class of a batch: units [u0, u1) run in one persistent launch whose
 // shared memory is laid out for the class's largest n.
