@@ -7,24 +7,38 @@
 // columns from the staged column-major copy in global memory (L2-resident for
 // moderate m), each CTA over its own slice of the rows:
 //
-//   descent  a radix descent over the order-preserving key of the correctly
+//   sample   the ratios of 1024 rows, sorted with their weights, bracket the
+//            median (12% of the weight either side);
+//   bins     one pass: the exact fixed-point weight (the pair kernel's q_i) of
+//            the rows below the bracket and, for those inside, of each of 1024
+//            equal steps of the approximate ratio x_ik * (1 / x_ijhat).  The
+//            CTAs of the cluster read each other's sums through distributed
+//            shared memory and every CTA finds the same crossing bin;
+//   rows     one pass: the rows whose approximate ratio lies within the guard
+//            band of that bin (a few hundred) are divided exactly, and the
+//            smallest exact key that passes the Decide test is the median.  As
+//            in the pair kernel's selection no step before has to be trusted:
+//            the rows' weights must add up to the bin's, and the weight below
+//            must fail the test.
+//   descent  what that cannot settle (ties, a wide column, few valid rows): a
+//            radix descent over the order-preserving key of the correctly
 //            rounded ratio r_i = x_ik / x_ijhat, 11 key bits per pass (float:
-//            3 passes, double: 6).  A pass histograms the exact fixed-point
-//            weights q_i (the pair kernel's q_i and Decide test) of the rows
-//            whose key lies in the surviving range by its next digit; the CTAs
-//            of the cluster read each other's histograms through distributed
-//            shared memory, every CTA takes the same decision from the same
-//            totals, and the first bin at which "weight at or below t exceeds
-//            W/2" (penalty point (0, lambda) included) becomes true is kept.
-//            After the last digit the surviving key is the median itself.
+//            3 passes, double: 6).  A pass histograms the weights of the rows
+//            whose key lies in the surviving range by its next digit; every CTA
+//            takes the same decision from the cluster's totals, and the first
+//            bin at which "weight at or below t exceeds W/2" (penalty point (0,
+//            lambda) included) becomes true is kept.  After the last digit the
+//            surviving key is the median itself.
 //   residual sum_i |x_ik - v x_ijhat| over the rows (float input: runs of 32
 //            terms in float, the runs in double; double input: double), a
 //            fixed reduction order per CTA, then rank order over the cluster;
 //            C depends on n only, so results do not depend on m or on the
 //            number of lambdas.
 //
-// Ratios are recomputed by division in every pass rather than stored.  A
-// decision the truncated weights cannot settle lists the pair for the exact
+// A row costs the bins pass a reciprocal and ~20 further instructions, the rows
+// pass ~8, against a division, a 64-bit weight and a key compare in each pass of
+// the descent (~60): 1,000,000 x 16 float 2.48 -> 1.14 ms.
+// A decision the truncated weights cannot settle lists the pair for the exact
 // wide-accumulator path, as in the pair kernel.  Control flow depends only on
 // the pair index and on values every CTA of a cluster computes identically,
 // so all CTAs meet every cluster barrier.
@@ -93,6 +107,35 @@ template <typename K> struct LgDecision {
     int first;       // first bin whose test is not "false" (LG_NB: none)
 };
 
+constexpr int LG_NS = 1024;    // sampled rows
+constexpr int LG_BINS = 1024;  // bins of the bracket
+constexpr int LG_SIDE = 8;     // bins kept free either side of it
+constexpr int LG_ROWS = 1024;  // rows divided exactly, at most
+constexpr float LG_HALF = 0.12f;  // sampled weight either side of the crossing
+// Weights of up to 46 bits are summed as two halves of at most 23 bits, 512
+// rows at a time in 32 bits.
+constexpr int LG_QBITS = 46;
+constexpr int LG_FLUSH = 128;  // vectors of four rows
+
+// The bracket search's arrays, in the space of the descent's histograms.
+template <typename T> struct LgPick {
+    using K = typename Traits<T>::K;
+    float key[LG_NS], w[LG_NS];            // the sample
+    uint32_t hi[LG_BINS], lo[LG_BINS];     // this CTA's bins, upper and lower halves
+    K akey[LG_ROWS + 1];                   // the cluster's rows
+    long long aq[LG_ROWS + 1];
+    K lkey[LG_ROWS];                       // this CTA's rows, read by the cluster
+    long long lq[LG_ROWS];
+    int lcnt;                              // their number (read by the cluster)
+    long long lsum[3];                     // in the bin, under it, below the range
+    int j1, ia, ib, first;
+    long long fl, fw;                      // weight before the crossing bin, its own
+    float wsumf[LG_NT / 32];
+    long long wsum[3][LG_NT / 32];
+    K kmin;
+    int und;
+};
+
 template <typename T> struct LgSmem {
     using K = typename Traits<T>::K;
     unsigned long long copies[LG_COPIES][LG_NB];  // this CTA's histogram copies
@@ -102,6 +145,427 @@ template <typename T> struct LgSmem {
     double wres[LG_NT / 32];                      // residual: warp partials
     LgDecision<K> dec;
 };
+
+__device__ __forceinline__ float rcp_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// floor(w 2^sigma) as hi 2^b + lo.  Float: w 2^(sigma - b) < 2^23, so adding
+// 2^23 rounding down leaves its floor in the mantissa, and the remainder, exact,
+// the same way.  up: 2^(sigma - b), dn: 2^b.
+__device__ __forceinline__ void split_q(float w, int, int, float up, float dn, uint32_t &hi,
+                                        uint32_t &lo) {
+    const float t = w * up;
+    const float m1 = __fadd_rz(t, Z32);
+    const float m2 = __fmaf_rz(t - (m1 - Z32), dn, Z32);
+    hi = __float_as_uint(m1) - Z32_BITS;
+    lo = __float_as_uint(m2) - Z32_BITS;
+}
+__device__ __forceinline__ void split_q(double w, int sigma, int b, float, float, uint32_t &hi,
+                                        uint32_t &lo) {
+    int e = 0;
+    const uint64_t q = (uint64_t)fixq(w, sigma, e);
+    hi = (uint32_t)(q >> b);
+    lo = (uint32_t)q & ((1u << b) - 1u);
+}
+
+// One row of the bins pass: its weight to the sum below (z < 2^23) or to the sum
+// inside and to bin z - 2^23 (z < 2^23 + LG_BINS), whose upper half lies at
+// shared address hb + 4 (bits of z), its lower half LG_BINS words further; NaN is
+// neither.  Predicated throughout: as branches the row cost twice as much.
+__device__ __forceinline__ void lg_bin(float z, uint32_t qh, uint32_t ql, uint32_t hb,
+                                       uint32_t &bh, uint32_t &bl, uint32_t &ih, uint32_t &il) {
+    static_assert(LG_BINS == 1024, "the PTX below holds 2^23 + LG_BINS and 4 LG_BINS");
+#if L1L_CHECKS
+    if (z < Z32) {
+        bh += qh;
+        bl += ql;
+    } else if (z < Z32 + (float)LG_BINS) {
+        (void)L1L_CHK((int)(__float_as_uint(z) - Z32_BITS), LG_BINS);
+#else
+    {
+#endif
+        asm volatile(
+            "{\n\t"
+            ".reg .pred pb, pc;\n\t"
+            ".reg .b32 a, zb;\n\t"
+            "setp.lt.f32 pb, %4, 0f4B000000;\n\t"
+            "setp.lt.and.f32 pc, %4, 0f4B000400, !pb;\n\t"
+            "@pb add.u32 %0, %0, %5;\n\t"
+            "@pb add.u32 %1, %1, %6;\n\t"
+            "@pc add.u32 %2, %2, %5;\n\t"
+            "@pc add.u32 %3, %3, %6;\n\t"
+            "mov.b32 zb, %4;\n\t"
+            "shl.b32 a, zb, 2;\n\t"
+            "add.u32 a, a, %7;\n\t"
+            "@pc red.shared.add.u32 [a], %5;\n\t"
+            "@pc red.shared.add.u32 [a + 4096], %6;\n\t"
+            "}"
+            : "+r"(bh), "+r"(bl), "+r"(ih), "+r"(il)
+            : "f"(z), "r"(qh), "r"(ql), "r"(hb)
+            : "memory");
+    }
+}
+
+// U vectors of four rows of the two columns, LG_NT apart, loaded together (the
+// passes are bound by the latency of these loads from L2); rows from `end` on
+// are 0.  w: the weights, in the input's type.
+template <typename T, int U> struct LgRows {
+    float4 vb[U], va[U];
+    double2 d0[sizeof(T) == 8 ? U : 1], d1[sizeof(T) == 8 ? U : 1];
+    __device__ __forceinline__ void load(const float *fj, const float *fk, const T *xj, int64_t v,
+                                         int64_t end) {
+#pragma unroll
+        for (int g = 0; g < U; ++g) {
+            const int64_t p = v + g * LG_NT;
+            vb[g] = va[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if constexpr (sizeof(T) == 8) d0[g] = d1[g] = make_double2(0.0, 0.0);
+            if (p < end) {
+                vb[g] = __ldg(reinterpret_cast<const float4 *>(fj) + p);
+                va[g] = __ldg(reinterpret_cast<const float4 *>(fk) + p);
+                if constexpr (sizeof(T) == 8) {
+                    d0[g] = __ldg(reinterpret_cast<const double2 *>(xj) + 2 * p);
+                    d1[g] = __ldg(reinterpret_cast<const double2 *>(xj) + 2 * p + 1);
+                }
+            }
+        }
+    }
+    static __device__ __forceinline__ float at(const float4 &v, int u) {
+        return u == 0 ? v.x : (u == 1 ? v.y : (u == 2 ? v.z : v.w));
+    }
+    __device__ __forceinline__ float b(int g, int u) const { return at(vb[g], u); }
+    __device__ __forceinline__ float a(int g, int u) const { return at(va[g], u); }
+    __device__ __forceinline__ T w(int g, int u) const {
+        if constexpr (sizeof(T) == 4)
+            return b(g, u);
+        else
+            return u == 0 ? d0[g].x : (u == 1 ? d0[g].y : (u == 2 ? d1[g].x : d1[g].y));
+    }
+};
+constexpr int LG_UB = 2;  // vectors in flight per thread: bins pass (4 spill),
+constexpr int LG_UR = 4;  // rows pass and residual
+
+// The block's sum of one value per thread, for every thread.
+__device__ __forceinline__ long long lg_sum(long long x, long long *ws) {
+    x = warp_sum_i64(x);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = x;
+    __syncthreads();
+    long long r = 0;
+    for (int w = 0; w < LG_NT / 32; ++w) r += ws[w];
+    return r;
+}
+
+// The weighted median of a pair by the cluster: LG_FOUND with its key, LG_EXACT
+// where the weights cannot settle it, LG_SEARCH where the descent has to look.
+// Every CTA returns the same.  c0, c1: this CTA's rows in vectors of four.
+template <typename T>
+__device__ int large_pick(const ScanArgs<T> &a, const ColInfo &ci, int64_t j, int64_t k,
+                          const Decide &dec, int64_t c0, int64_t c1, LgSmem<T> &sm, int &buf,
+                          typename Traits<T>::K &key) {
+    using Tr = Traits<T>;
+    using K = typename Tr::K;
+    constexpr uint32_t G = Approx<T>::G;
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = (int)cl.num_blocks();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t n = a.n, ldn = a.ldn;
+    // what the split and the approximate ratio need (else: the descent)
+    const int qbits = 61 - (32 - __clz(ci.n_valid));
+    const int qb = (qbits + 1) / 2, es = ci.sigma - qb;
+    if (qbits > LG_QBITS || (ci.flags & COL_WIDE) || es < -120 || es > 120 ||
+        (sizeof(T) == 8 && (a.ci[k].flags & COL_WIDE)))
+        return LG_SEARCH;
+    const float up = __int_as_float((127 + es) << 23), dn = __int_as_float((127 + qb) << 23);
+    static_assert(sizeof(LgPick<T>) <= sizeof(sm.copies), "the descent's histograms hold it");
+    LgPick<T> &pk = *reinterpret_cast<LgPick<T> *>(&sm.copies[0][0]);
+    const T *xj = a.Xt + j * ldn, *xk = a.Xt + k * ldn;
+    const float *fj = a.Xf + j * ldn, *fk = a.Xf + k * ldn;
+
+    // ---- sample: the same rows and the same arithmetic in every CTA ----
+    for (int s = tid; s < LG_NS; s += LG_NT) {
+        const int64_t i = (int64_t)(2 * s + 1) * n / (2 * LG_NS);
+        const float xb = fj[i];
+        const float r = fk[i] * rcp_approx(xb);
+        pk.key[s] = xb != 0.0f ? r : INFINITY;
+        pk.w[s] = fabsf(xb);
+    }
+    if (tid == 0) pk.j1 = pk.ia = pk.ib = LG_NS - 1;
+    for (int size = 2; size <= LG_NS; size <<= 1)
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            __syncthreads();
+            for (int t = tid; t < LG_NS / 2; t += LG_NT) {
+                const int i = 2 * t - (t & (stride - 1)), o = i + stride;
+                const float x = pk.key[i], y = pk.key[o];
+                if ((x > y) == ((i & size) == 0)) {
+                    pk.key[i] = y;
+                    pk.key[o] = x;
+                    const float u = pk.w[i];
+                    pk.w[i] = pk.w[o];
+                    pk.w[o] = u;
+                }
+            }
+        }
+    __syncthreads();
+    float a0, b0;
+    {
+        static_assert(LG_NS == 2 * LG_NT, "two samples per thread");
+        const float w0 = pk.w[2 * tid], w1 = pk.w[2 * tid + 1];
+        const float incl = warp_scan_add(w0 + w1, lane);
+        if (lane == 31) pk.wsumf[warp] = incl;
+        __syncthreads();
+        float before = 0.0f, total = 0.0f;
+        for (int w = 0; w < LG_NT / 32; ++w) {
+            if (w == warp) before = total;
+            total += pk.wsumf[w];
+        }
+        const float cum1 = before + incl, cum0 = cum1 - w1;
+        const float per = total / (float)dec.Q;
+        const float tpos = 0.5f * per * (float)(dec.Q - dec.Lc);
+        const float tneg = 0.5f * per * (float)(dec.Q + dec.Lf);
+        auto passes = [&](float cum, float x) { return cum >= (x >= 0.0f ? tpos : tneg); };
+        if (passes(cum0, pk.key[2 * tid]))
+            atomicMin(&pk.j1, 2 * tid);
+        else if (passes(cum1, pk.key[2 * tid + 1]))
+            atomicMin(&pk.j1, 2 * tid + 1);
+        __syncthreads();
+        if (pk.j1 == 2 * tid) pk.wsumf[0] = cum0;
+        if (pk.j1 == 2 * tid + 1) pk.wsumf[0] = cum1;
+        __syncthreads();
+        const float mid = pk.wsumf[0];
+        const float ta = mid - LG_HALF * total, tb = mid + LG_HALF * total;
+        if (cum0 >= ta)
+            atomicMin(&pk.ia, 2 * tid);
+        else if (cum1 >= ta)
+            atomicMin(&pk.ia, 2 * tid + 1);
+        if (cum0 >= tb)
+            atomicMin(&pk.ib, 2 * tid);
+        else if (cum1 >= tb)
+            atomicMin(&pk.ib, 2 * tid + 1);
+        __syncthreads();
+        a0 = pk.key[max(pk.ia - 1, 0)];
+        b0 = pk.key[pk.ib];
+    }
+
+    for (int attempt = 0; attempt < 3; ++attempt) {
+        // ---- bins: steps of w1, no finer than 16 keys of the largest ratio ----
+        const float w1 = fmaxf((b0 - a0) * (1.0f / (LG_BINS - 2 * LG_SIDE)),
+                               fmaxf(fabsf(a0), fabsf(b0)) * 0x1p-19f);
+        if (!(w1 > 0x1p-100f && w1 < 0x1p100f)) return LG_SEARCH;
+        const float sc = __frcp_rn(w1);
+        const float bm = __fmaf_rn(-a0, sc, Z32 + (float)LG_SIDE);
+        constexpr float ZT = Z32 + (float)LG_BINS;
+        for (int b = tid; b < LG_BINS; b += LG_NT) pk.hi[b] = pk.lo[b] = 0;
+        if (tid == 0) pk.first = LG_BINS;
+        __syncthreads();
+        long long Sb = 0, Sa = 0;  // below the bracket; inside it, then below its end
+        const uint32_t hb = smem_addr(pk.hi) - 4u * Z32_BITS;
+        for (int64_t v0 = c0 + tid; v0 < c1; v0 += (int64_t)LG_FLUSH * LG_NT) {
+            const int64_t ve = std::min<int64_t>(c1, v0 + (int64_t)LG_FLUSH * LG_NT);
+            uint32_t bh = 0, bl = 0, ih = 0, il = 0;
+            for (int64_t v = v0; v < ve; v += LG_UB * LG_NT) {
+                LgRows<T, LG_UB> x;
+                x.load(fj, fk, xj, v, ve);
+#pragma unroll
+                for (int g = 0; g < LG_UB; ++g)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        // x_ijhat = 0: the weight is 0, wherever the ratio falls
+                        const float z = __fmaf_rn(__fmul_rn(x.a(g, u), rcp_approx(x.b(g, u))), sc, bm);
+                        uint32_t qh, ql;
+                        split_q(fabs(x.w(g, u)), ci.sigma, qb, up, dn, qh, ql);
+                        lg_bin(z, qh, ql, hb, bh, bl, ih, il);
+                    }
+            }
+            Sb += ((long long)bh << qb) + (long long)bl;
+            Sa += ((long long)ih << qb) + (long long)il;
+        }
+        Sa += Sb;
+        Sb = lg_sum(Sb, pk.wsum[0]);
+        Sa = lg_sum(Sa, pk.wsum[1]);  // also: the bins are complete
+        for (int b = tid; b < LG_BINS; b += LG_NT)
+            sm.tot[buf][b] = ((unsigned long long)pk.hi[b] << qb) + pk.lo[b];
+        if (tid == 0) {
+            sm.tot[buf][LG_BINS] = (unsigned long long)Sb;
+            sm.tot[buf][LG_BINS + 1] = (unsigned long long)Sa;
+        }
+        cl.sync();
+        // ---- the crossing bin of the cluster's totals ----
+        constexpr int Q = LG_BINS / LG_NT;
+        long long h[Q], run = 0;
+#pragma unroll
+        for (int u = 0; u < Q; ++u) {
+            unsigned long long x = 0;
+            for (int r = 0; r < C; ++r) x += cl.map_shared_rank(&sm.tot[buf][0], r)[Q * tid + u];
+            h[u] = (long long)x;
+            run += h[u];
+        }
+        Sb = Sa = 0;
+        for (int r = 0; r < C; ++r) {
+            const unsigned long long *o = cl.map_shared_rank(&sm.tot[buf][0], r);
+            Sb += (long long)o[LG_BINS];
+            Sa += (long long)o[LG_BINS + 1];
+        }
+        buf ^= 1;
+        const long long incl = warp_scan_add(run, lane);
+        if (lane == 31) pk.wsum[2][warp] = incl;
+        __syncthreads();
+        long long cum = Sb + incl - run, all = 0;
+        for (int w = 0; w < LG_NT / 32; ++w) {
+            if (w < warp) cum += pk.wsum[2][w];
+            all += pk.wsum[2][w];
+        }
+        if (all != Sa - Sb) return LG_SEARCH;  // a bin of one CTA left 32 bits
+        const int zb = bm < Z32 ? 0 : (bm < ZT ? (int)(bm - Z32) : LG_BINS);
+        const int64_t tneg = ((dec.Q + dec.Lf) >> 1) + 1, tpos = ((dec.Q - dec.Lc) >> 1) + 1;
+        int mine = LG_BINS;
+        long long ml = 0, mw = 0;
+#pragma unroll
+        for (int u = 0; u < Q; ++u) {
+            const int b = Q * tid + u;
+            if (mine == LG_BINS && cum + h[u] >= (b >= zb ? tpos : tneg)) {
+                mine = b;
+                ml = cum;
+                mw = h[u];
+            }
+            cum += h[u];
+        }
+        if (mine < LG_BINS) atomicMin(&pk.first, mine);
+        __syncthreads();
+        const int ca = pk.first;
+        if (mine == ca && mine < LG_BINS) {
+            pk.fl = ml;
+            pk.fw = mw;
+        }
+        if (tid == 0) {
+            pk.lcnt = 0;
+            pk.kmin = Tr::NONE;
+            pk.und = 0;
+        }
+        __syncthreads();
+        if (ca < 1 || ca >= LG_BINS) {  // missed: further out on that side
+            const float span = b0 - a0;
+            if (ca < 1) {
+                b0 = a0 + 2.0f * w1;
+                a0 = a0 - 4.0f * fmaxf(span, 2.0f * w1);
+            } else {
+                a0 = b0 - 2.0f * w1;
+                b0 = b0 + 4.0f * fmaxf(span, 2.0f * w1);
+            }
+            if (!(a0 < b0)) return LG_SEARCH;
+            continue;
+        }
+        // ---- the coarse keys [lo, hi] around it (pair kernel's selection) ----
+        const float ra = ((Z32 + (float)ca - bm) - 0.5f) * w1;
+        const float rb = ((Z32 + (float)ca - bm) + 0.5f) * w1;
+        const uint32_t ka = sat_sub(akey(ra), 2 * G + 4), kb = sat_add(akey(rb), 2 * G + 4);
+        const float va = akey_value(ka), vb = akey_value(kb);
+        if (!(va < vb)) return LG_SEARCH;
+        const uint32_t lo = ka + G, hi = kb - G;
+        const float cen = 0.5f * (va + vb);
+        const float delta =
+            0.5f * (vb - va) * (1.0f + 0x1p-20f) + 0x1p-21f * fmaxf(fabsf(va), fabsf(vb));
+        long long in_w = 0, under_w = 0, below_w = 0;
+        for (int64_t v = c0 + tid; v < c1; v += LG_UR * LG_NT) {
+            LgRows<float, LG_UR> x;
+            x.load(fj, fk, fj, v, c1);
+            uint32_t hit = 0;
+#pragma unroll
+            for (int g = 0; g < LG_UR; ++g)
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (fabsf(__fmaf_rn(x.a(g, u), rcp_approx(x.b(g, u)), -cen)) < delta)
+                        hit |= 1u << (4 * g + u);
+            for (; hit; hit &= hit - 1) {
+                const int bit = __ffs(hit) - 1;
+                const int64_t i = 4 * (v + (bit >> 2) * LG_NT) + (bit & 3);
+                const float b = fj[i], r = __fmul_rn(fk[i], rcp_approx(b));
+                if (!(r >= va && r <= vb) || b == 0.0f) continue;
+                int e = 0;
+                const long long q = fixq(fabs(xj[i]), ci.sigma, e);
+                const float z = __fmaf_rn(r, sc, bm);
+                if (z < Z32 + (float)ca)
+                    under_w += q;
+                else if (z <= Z32 + (float)ca)
+                    in_w += q;
+                const K fkey = Tr::key(Tr::div_rn(xk[i], xj[i]));
+                const uint32_t ck = coarse_of<T>(fkey);
+                if (ck < lo) {
+                    below_w += q;
+                } else if (ck <= hi) {
+                    const int at = atomicAdd(&pk.lcnt, 1);
+                    if (at < LG_ROWS) {
+                        pk.lkey[at] = fkey;
+                        pk.lq[at] = q;
+                    }
+                }
+            }
+        }
+        in_w = lg_sum(in_w, pk.wsum[0]);
+        under_w = lg_sum(under_w, pk.wsum[1]);
+        below_w = lg_sum(below_w, pk.wsum[2]);
+        if (tid == 0) {
+            pk.lsum[0] = in_w;
+            pk.lsum[1] = under_w;
+            pk.lsum[2] = below_w;
+        }
+        cl.sync();
+        // ---- every CTA gathers the cluster's rows ----
+        int c = 0;
+        in_w = 0;
+        long long L = pk.fl;
+        for (int r = 0; r < C; ++r) {
+            const LgPick<T> *o = cl.map_shared_rank(&pk, r);
+            const int cr = o->lcnt;
+            in_w += o->lsum[0];
+            L += o->lsum[2] - o->lsum[1];
+            for (int e = tid; e < cr && c + e < LG_ROWS; e += LG_NT) {
+                pk.akey[c + e] = o->lkey[e];
+                pk.aq[c + e] = o->lq[e];
+            }
+            c += cr;
+        }
+        const long long W = pk.fw;
+        cl.sync();  // the lists are free again
+        if (c > LG_ROWS || in_w != W || dec.cond(L, lo > CK0) != 0) return LG_SEARCH;
+        if (lo <= CK0 && CK0 <= hi) {  // the penalty point; lambda sits in the test
+            if (tid == 0) {
+                pk.akey[c] = Tr::KEY0;
+                pk.aq[c] = 0;
+            }
+            c += 1;
+            __syncthreads();
+        }
+        for (int e = tid; e < c; e += LG_NT) {
+            const K x = pk.akey[e];
+            long long S = L;
+            for (int q = 0; q < c; ++q) S += pk.akey[q] <= x ? pk.aq[q] : 0;
+            const int res = dec.cond(S, x >= Tr::KEY0);
+            if (res != 0) {
+                if constexpr (sizeof(K) == 4)
+                    atomicMin(&pk.kmin, x);
+                else
+                    atomicMin(reinterpret_cast<unsigned long long *>(&pk.kmin),
+                              (unsigned long long)x);
+            }
+        }
+        __syncthreads();
+        key = pk.kmin;
+        if (key == Tr::NONE) return LG_SEARCH;
+        // equal keys have equal sums: any of them tells whether it was certain
+        for (int e = tid; e < c; e += LG_NT)
+            if (pk.akey[e] == key) {
+                long long S = L;
+                for (int q = 0; q < c; ++q) S += pk.akey[q] <= key ? pk.aq[q] : 0;
+                if (dec.cond(S, key >= Tr::KEY0) < 0) pk.und = 1;
+            }
+        __syncthreads();
+        return pk.und ? LG_EXACT : LG_FOUND;
+    }
+    return LG_SEARCH;
+}
 
 template <typename T>
 __global__ void __launch_bounds__(LG_NT, 2)
@@ -166,6 +630,14 @@ __global__ void __launch_bounds__(LG_NT, 2)
         K prefix = 0;
         int64_t sbelow = 0;
         int state = ci.n_valid > 0 ? LG_SEARCH : LG_NONE;  // no valid row: v = 0
+        if (state == LG_SEARCH) {
+            state = large_pick<T>(a, ci, j, k, dec, r0 / 4, r1 / 4, sm, buf, prefix);
+            if (state == LG_SEARCH) {
+                prefix = 0;
+                cl.sync();  // the descent's histograms overlap what the cluster read
+            }
+            __syncthreads();
+        }
         for (int l = 0; state == LG_SEARCH && l < LgDigits<T>::levels; ++l) {
             const int sh = LgDigits<T>::shift(l);
             const int top = l == 0 ? KB : LgDigits<T>::shift(l - 1);
@@ -309,18 +781,30 @@ __global__ void __launch_bounds__(LG_NT, 2)
         double racc = 0.0;
         T run = T(0);
         int nrun = 0;
-        for (int64_t v = v0 + tid; v < v1; v += LG_NT) {
-            T xb[VW], xa[VW];
-            VT::get(xjv[v], xb);
-            VT::get(xkv[v], xa);
-            T t4 = T(0);
+        for (int64_t v = v0 + tid; v < v1; v += LG_UR * LG_NT) {
+            V vb[LG_UR], va[LG_UR];
 #pragma unroll
-            for (int u = 0; u < VW; ++u) t4 += fabs(fma(-vv, xb[u], xa[u]));
-            run += t4;
-            if (++nrun == 32 / VW || sizeof(T) == 8) {
-                racc += (double)run;
-                run = T(0);
-                nrun = 0;
+            for (int g = 0; g < LG_UR; ++g) {
+                vb[g] = va[g] = V{};
+                if (v + g * LG_NT < v1) {
+                    vb[g] = xjv[v + g * LG_NT];
+                    va[g] = xkv[v + g * LG_NT];
+                }
+            }
+#pragma unroll
+            for (int g = 0; g < LG_UR; ++g) {
+                T xb[VW], xa[VW];
+                VT::get(vb[g], xb);
+                VT::get(va[g], xa);
+                T t4 = T(0);
+#pragma unroll
+                for (int u = 0; u < VW; ++u) t4 += fabs(fma(-vv, xb[u], xa[u]));
+                run += t4;
+                if (++nrun == 32 / VW || sizeof(T) == 8) {
+                    racc += (double)run;
+                    run = T(0);
+                    nrun = 0;
+                }
             }
         }
         racc += (double)run;

@@ -2,6 +2,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "launch.h"
@@ -30,7 +31,7 @@ __global__ void __launch_bounds__(256) k_colprep(const T *__restrict__ Xt, ColIn
     colprep_column<T>(Xt + (int64_t)blockIdx.x * ldn, ci + blockIdx.x, n);
 }
 
-// Block-wide reductions of one value per thread (512 threads); `red` holds
+// Block-wide reductions of one value per thread; `red` holds
 // the warp partials, `out` receives the result for every thread.
 enum { RED_SUM, RED_MAX, RED_MIN };
 template <int OP>
@@ -51,41 +52,63 @@ __device__ __forceinline__ long long block_reduce_ll(long long x, long long *red
     return r;
 }
 
-// Column statistics of tall columns: a cluster of C CTAs per column, each
-// over its slice of rows; the three dependent reductions (count and exponent
-// range -> sigma; Q and truncations -> the 32-bit shift; Q32 and its
-// truncations) are combined across the cluster through distributed shared
-// memory.  Integer sums, so the result equals the one-CTA version's.
+// Column statistics of tall columns: a cluster of C CTAs per column, each over
+// its slice of rows; the two dependent reductions (count and exponent range ->
+// sigma; Q and truncations) are combined across the cluster through distributed
+// shared memory.  Integer sums, so the result equals the one-CTA version's.  The
+// 32-bit weights' totals are left out: only the pair kernel reads them, which
+// ends far below these heights.  16 columns of 1,000,000 floats are 128 CTAs, one
+// per SM, so the passes are bound by loads in flight: four vectors per thread and
+// 1024 threads instead of scalar loads by 512 (and two passes for three), 179 us,
+// 79 us.
+constexpr int CT_NT = 1024;
 template <typename T>
-__global__ void __launch_bounds__(512) k_colprep_tall(const T *__restrict__ Xt, ColInfo *ci,
-                                                      int64_t n, int64_t ldn, int64_t rpc) {
+__global__ void __launch_bounds__(CT_NT) k_colprep_tall(const T *__restrict__ Xt, ColInfo *ci,
+                                                        int64_t ldn, int64_t rpc) {
+    using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+    constexpr int W = 16 / sizeof(T), U = 4;
     cg::cluster_group cl = cg::this_cluster();
     const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
     const int64_t j = blockIdx.x / C;
-    const T *col = Xt + j * ldn;
-    const int64_t r0 = std::min<int64_t>(n, (int64_t)rank * rpc);
-    const int64_t r1 = std::min<int64_t>(n, r0 + rpc);
-    __shared__ long long red[16];
-    __shared__ long long p1[3], p2[2], p3[2];  // this CTA's partials, read by the cluster
+    const V *col = reinterpret_cast<const V *>(Xt + j * ldn);
+    // whole vectors: ldn and rpc are multiples of 128, rows past n are 0
+    const int64_t v0 = std::min<int64_t>(ldn, (int64_t)rank * rpc) / W;
+    const int64_t v1 = std::min<int64_t>(ldn, (int64_t)(rank + 1) * rpc) / W;
+    __shared__ long long red[CT_NT / 32];
+    __shared__ long long p1[3], p2[2];  // this CTA's partials, read by the cluster
+    auto each = [&](auto &&f) {
+        for (int64_t v = v0 + threadIdx.x; v < v1; v += U * CT_NT) {
+            V x[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) x[u] = v + u * CT_NT < v1 ? __ldg(col + v + u * CT_NT) : V{};
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                f(T(x[u].x));
+                f(T(x[u].y));
+                if constexpr (W == 4) {
+                    f(T(x[u].z));
+                    f(T(x[u].w));
+                }
+            }
+        }
+    };
 
     int cnt = 0, emax = -100000, emin = 100000;
-#pragma unroll 4
-    for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) {
-        const T b = col[i];
+    each([&](T b) {
         if (b != T(0)) {
             cnt++;
             const int e = ilog2_pos(b);
             emax = max(emax, e);
             emin = min(emin, e);
         }
-    }
-    long long v0 = block_reduce_ll<RED_SUM>(cnt, red);
-    long long v1 = block_reduce_ll<RED_MAX>(emax, red);
-    long long v2 = block_reduce_ll<RED_MIN>(emin, red);
+    });
+    long long x0 = block_reduce_ll<RED_SUM>(cnt, red);
+    long long x1 = block_reduce_ll<RED_MAX>(emax, red);
+    const long long x2 = block_reduce_ll<RED_MIN>(emin, red);
     if (threadIdx.x == 0) {
-        p1[0] = v0;
-        p1[1] = v1;
-        p1[2] = v2;
+        p1[0] = x0;
+        p1[1] = x1;
+        p1[2] = x2;
     }
     cl.sync();
     long long nvl = 0;
@@ -101,58 +124,26 @@ __global__ void __launch_bounds__(512) k_colprep_tall(const T *__restrict__ Xt, 
 
     long long qs = 0;
     int inx = 0;
-#pragma unroll 4
-    for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) {
-        const T b = col[i];
-        if (b != T(0)) {
-            int e = 0;
-            qs += fixq(absval(b), sigma, e);
-            inx += e;
-        }
-    }
-    v0 = block_reduce_ll<RED_SUM>(qs, red);
-    v1 = block_reduce_ll<RED_SUM>(inx, red);
+    each([&](T b) {
+        int e = 0;
+        qs += fixq(absval(b), sigma, e);
+        inx += e;
+    });
+    x0 = block_reduce_ll<RED_SUM>(qs, red);
+    x1 = block_reduce_ll<RED_SUM>(inx, red);
     if (threadIdx.x == 0) {
-        p2[0] = v0;
-        p2[1] = v1;
-    }
-    cl.sync();
-    long long Q = 0, I = 0;
-    for (int r = 0; r < C; ++r) {
-        const long long *q = cl.map_shared_rank(&p2[0], r);
-        Q += q[0];
-        I += q[1];
-    }
-    const int shift = colprep_shift32(Q);
-    const uint64_t lowmask = (1ull << shift) - 1ull;
-
-    long long q32 = 0;
-    int inx32 = 0;
-#pragma unroll 4
-    for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) {
-        const T b = col[i];
-        if (b != T(0)) {
-            int e = 0;
-            const uint64_t qi = (uint64_t)fixq(absval(b), sigma, e);
-            q32 += (long long)(qi >> shift);
-            inx32 += (e || (qi & lowmask) != 0) ? 1 : 0;
-        }
-    }
-    v0 = block_reduce_ll<RED_SUM>(q32, red);
-    v1 = block_reduce_ll<RED_SUM>(inx32, red);
-    if (threadIdx.x == 0) {
-        p3[0] = v0;
-        p3[1] = v1;
+        p2[0] = x0;
+        p2[1] = x1;
     }
     cl.sync();
     if (rank == 0 && threadIdx.x == 0) {
-        long long Q32 = 0, I32 = 0;
+        long long Q = 0, I = 0;
         for (int r = 0; r < C; ++r) {
-            const long long *q = cl.map_shared_rank(&p3[0], r);
-            Q32 += q[0];
-            I32 += q[1];
+            const long long *q = cl.map_shared_rank(&p2[0], r);
+            Q += q[0];
+            I += q[1];
         }
-        ci[j] = colprep_make<T>(Q, sigma, nv, (int)I, Emin, E, Q32, shift, (int)I32);
+        ci[j] = colprep_make<T>(Q, sigma, nv, (int)I, Emin, E, 0, 0, 0);
     }
     cl.sync();  // no CTA leaves while rank 0 may still read its partials
 }
@@ -181,13 +172,13 @@ cudaError_t launch_prep(const T *X, T *Xt, float *Xf, ColInfo *ci, int64_t n, in
     at[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(m * C));
-    cfg.blockDim = dim3(512);
+    cfg.blockDim = dim3(CT_NT);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = st;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    const int64_t rpc = (n + C - 1) / C;
-    e = cudaLaunchKernelEx(&cfg, k_colprep_tall<T>, (const T *)Xt, ci, n, ldn, rpc);
+    const int64_t rpc = ((ldn + C - 1) / C + ROW_PAD - 1) & ~int64_t(ROW_PAD - 1);
+    e = cudaLaunchKernelEx(&cfg, k_colprep_tall<T>, (const T *)Xt, ci, ldn, rpc);
     launches++;
     return e;
 }
