@@ -28,14 +28,13 @@
 //     t < 0:  R(t) = R(0) - 2 B(t, 0) + t (2 S(t) - Q)
 // with B the sum of |x_ik| over the rows whose ratio lies there.  All of them
 // are sums of fixed-point integers (column k's and column jhat's), exact
-// whatever the order; what truncation to those drops (double input; float input
-// only beyond 37 binary orders) is summed beside them in float, in units of the
-// last place.  (The five
-// double sums over all rows that gave R before made the double pipe, two
-// operations per SM and cycle, the bound: 1000 x 500 float with residuals,
-// write pass 5.07 -> 0.76 ms.  Without them, 2000 x 400: 1.33 -> 0.70 ms,
-// count pass 0.42 -> 0.22 ms.)  The write pass is bound by instructions, a
-// quarter of them the rows', the rest the sort and the prefix sums of the list.
+// whatever the order; what truncation to those drops (double input, and float
+// columns that span many binary orders) is summed beside them in float, in units
+// of the last place.  (The five double sums over all rows that gave R before made
+// the double pipe, two operations per SM and cycle, the bound: 1000 x 500 float
+// with residuals, write pass 5.07 -> 0.61 ms.  Without them, 2000 x 400: 1.33 ->
+// 0.56 ms; count pass 0.42 -> 0.22 ms.)  The write pass is bound by instructions,
+// a quarter of them the rows', the rest the order and the prefix sums of the list.
 #include <cmath>
 #include <type_traits>
 
@@ -52,6 +51,8 @@ constexpr int PW = 8;          // warps per CTA
 constexpr int PATH_CAP = 256;  // shared-memory list entries per warp
 constexpr int PATH_CAP_MIN = 128;  // where the column leaves no room for that
 constexpr int PEND = 64;       // rows queued for the exact division, per warp
+constexpr int PBUCK = 64;      // buckets of the list's sort
+constexpr uint32_t BUCK_MAX = 48;
 
 template <typename T> struct PathArgs {
     const T *Xt;
@@ -64,11 +65,12 @@ template <typename T> struct PathArgs {
     double *lam;           // write pass outputs
     T *val;
     double *res;           // optional: residual sum_i |x_ik - v x_ijhat| of each entry
-    float *crem;           // with residuals, double input: [m] remainders of a column's total
+    float *crem;           // with residuals: [m] remainder of a column's fixed-point total
     int32_t *len;          // [m*m]
     int32_t *big;          // pairs whose rows exceed the warp list
     uint32_t *big_count;
     uint32_t *big_next;    // work counter of the big-pair kernel
+    uint32_t *inexact;     // whether any column's remainders are needed
     unsigned char *scratch;  // big-pair lists, one slice per worker warp
     int64_t slice;         // entries per slice (power of two >= n)
     uint32_t *status;
@@ -115,19 +117,33 @@ __device__ __forceinline__ float fix_rem(double w, int sigma) {
     return (float)f * __int_as_float((127 - rs) << 23);
 }
 
-// Whether the remainders are summed: double input with residuals.
-template <typename T> __device__ __forceinline__ bool with_rem(const PathArgs<T> &a) {
-    return sizeof(T) == 8 && a.res != nullptr;
+// Whether a column's truncated weights may together lack more than 2^-54 of its
+// total, and whether a pair's remainders are summed (the same for the warp).
+__device__ __forceinline__ bool lacks(const ColInfo &c) {
+    return (int64_t)c.n_inexact > (c.Q >> 54);
+}
+template <typename T>
+__device__ __forceinline__ bool with_rem(const PathArgs<T> &a, const ColInfo &cj,
+                                         const ColInfo &ck) {
+    return a.res != nullptr && (lacks(cj) || lacks(ck));
 }
 
 // The column arrays of jhat: float reciprocal, fixed-point weight, and x
-// itself (float input) or the weight's remainder (double input, which reads x
-// from the column copy: a few rows per pair).
+// itself (float input, whose remainders are computed where there are any) or
+// the weight's remainder (double input, which reads x from the column copy: a
+// few rows per pair).
 template <typename T> struct Column {
     const T *x;
     float *inv;
     int64_t *q;
     float *rem;
+    int sigma;
+    __device__ __forceinline__ float rem_of(int i) const {
+        if constexpr (sizeof(T) == 8)
+            return rem[i];
+        else
+            return fix_rem(x[i], sigma);
+    }
 };
 
 // Stage them by `nt` threads; `own` holds x or the remainders.
@@ -141,73 +157,101 @@ __device__ Column<T> stage_column(const PathArgs<T> &a, int64_t j, float *own, f
         if constexpr (sizeof(T) == 4)
             own[i] = b;
         else
-            own[i] = with_rem(a) ? fix_rem(b, ci.sigma) : 0.0f;
+            own[i] = a.res ? fix_rem(b, ci.sigma) : 0.0f;
         // NaN: neither inside, below nor above any range
         inv[i] = b != T(0) ? Approx<T>::inv_of(b) : __int_as_float(0x7FFFFFFF);
         int e = 0;
         colq[i] = b != T(0) ? fixq(b < T(0) ? -b : b, ci.sigma, e) : 0;
     }
     if constexpr (sizeof(T) == 4)
-        return Column<T>{own, inv, colq, nullptr};
+        return Column<T>{own, inv, colq, nullptr, ci.sigma};
     else
-        return Column<T>{xj, inv, colq, own};
+        return Column<T>{xj, inv, colq, own, ci.sigma};
 }
 
 // Remainder of each column's fixed-point total.
 template <typename T> __global__ void __launch_bounds__(256) k_colrem(PathArgs<T> a) {
-    if constexpr (sizeof(T) == 8) {
-        __shared__ float sm[8];
-        const T *x = a.Xt + (int64_t)blockIdx.x * a.ldn;
-        const int sigma = a.ci[blockIdx.x].sigma;
-        float s = 0.0f;
-        for (int64_t i = threadIdx.x; i < a.n; i += 256) s += fix_rem(x[i], sigma);
-        s = warp_sum_f32(s);
-        if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = s;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int q = 1; q < 8; ++q) s += sm[q];
-            a.crem[blockIdx.x] = s;
-        }
+    __shared__ float sm[8];
+    const T *x = a.Xt + (int64_t)blockIdx.x * a.ldn;
+    const ColInfo ci = a.ci[blockIdx.x];
+    float s = 0.0f;
+    if (ci.n_inexact > 0)
+        for (int64_t i = threadIdx.x; i < a.n; i += 256) s += fix_rem(x[i], ci.sigma);
+    s = warp_sum_f32(s);
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int q = 1; q < 8; ++q) s += sm[q];
+        a.crem[blockIdx.x] = s;
+        if (lacks(ci)) atomicOr(a.inexact, 1u);
     }
 }
 
-// The list's sums of one pair: the weight below the range and the |x_ik| in
-// it, in fixed point and the remainders of both.
+// The list's sums of one pair: the weight below the range and (negative ranges)
+// the |x_ik| in it, in fixed point and the remainders of both.
 struct ListSums {
     int64_t Sbelow, Ball;
     float Srem, Brem;
 };
 
-// Sort of up to 64 (key, row) by one warp: every lane counts the entries
-// before its own two (ties by list position) and puts them there.  Up to 64
-// entries that is fewer instructions than the bitonic network below.
-template <typename K> __device__ void warp_rank_sort(K *keys, uint32_t *rows, int c, int lane) {
-    const int l2 = lane + 32;
-    const K k0 = lane < c ? keys[lane] : (K)~(K)0, k1 = l2 < c ? keys[l2] : (K)~(K)0;
-    const uint32_t r0 = lane < c ? rows[lane] : 0u, r1 = l2 < c ? rows[l2] : 0u;
-    int p0 = 0, p1 = 0;
-    if (c <= 32) {
-        for (int q = 0; q < c; ++q) {
-            const K kq = keys[q];
-            p0 += kq < k0 || (kq == k0 && q < lane) ? 1 : 0;
+// A warp's sort of its list, as an order: bucket counts and two index arrays
+// (the first is the queue while the rows are scanned).
+struct SortBuf {
+    uint32_t *cnt;      // [PBUCK]
+    uint16_t *part, *ord;  // [cap]
+};
+__host__ __device__ constexpr size_t sort_bytes(int cap) { return PBUCK * 4 + (size_t)cap * 4; }
+
+// ord[i] = list position of the i-th smallest (key, position) of c, by one
+// warp: the ratios of a list spread evenly between 0 and v0, so 64 equal steps
+// hold a few each, and an entry is ranked within its own.  Returns whether two
+// keys are equal, or -1, with no order, when a bucket holds over BUCK_MAX (many
+// ties, a range with most ratios in one place): ranking within it would take
+// longer than the network.  (A bitonic network: 28 steps of 20 instructions and their
+// latencies at 65 to 128 entries; 2000 x 400 write pass 0.70 -> 0.61 ms.
+// Ranking up to 64 entries among all instead: 0.87 -> 0.91 ms at 1000 x 500.)
+template <typename T>
+__device__ int warp_bucket_sort(const typename Traits<T>::K *keys, int c, T v0,
+                                 const SortBuf &sb, int lane) {
+    using Tr = Traits<T>;
+    using K = typename Tr::K;
+    const bool pos = v0 > T(0);
+    const float scale = (float)PBUCK / fabsf((float)v0);
+    auto bucket = [&](K k) -> int {  // monotone in the key
+        const int b = min(PBUCK - 1, (int)(fabsf((float)Tr::value(k)) * scale));
+        return pos ? b : PBUCK - 1 - b;
+    };
+    static_assert(PBUCK == 64, "two buckets per lane");
+    sb.cnt[lane] = sb.cnt[lane + 32] = 0u;
+    __syncwarp();
+    for (int e = lane; e < c; e += 32) atomicAdd(&sb.cnt[bucket(keys[e])], 1u);
+    __syncwarp();
+    const uint32_t c0 = sb.cnt[2 * lane], c1 = sb.cnt[2 * lane + 1];
+    if (__reduce_max_sync(0xFFFFFFFFu, max(c0, c1)) > BUCK_MAX) return -1;
+    const uint32_t ex = warp_scan_add(c0 + c1, lane) - c0 - c1;
+    sb.cnt[2 * lane] = ex;
+    sb.cnt[2 * lane + 1] = ex + c0;
+    __syncwarp();
+    for (int e = lane; e < c; e += 32)
+        sb.part[atomicAdd(&sb.cnt[bucket(keys[e])], 1u)] = (uint16_t)e;
+    __syncwarp();
+    bool ties = false;
+    for (int p = lane; p < c; p += 32) {
+        const int e = sb.part[p];
+        const K k = keys[e];
+        const int b = bucket(k);
+        const int q0 = b ? (int)sb.cnt[b - 1] : 0, q1 = (int)sb.cnt[b];
+        int r = q0;
+        for (int q = q0; q < q1; ++q) {
+            const int f = sb.part[q];
+            const K kf = keys[f];
+            r += kf < k || (kf == k && f < e) ? 1 : 0;
+            ties |= kf == k && f != e;
         }
-    } else {
-        for (int q = 0; q < c; ++q) {
-            const K kq = keys[q];
-            p0 += kq < k0 || (kq == k0 && q < lane) ? 1 : 0;
-            p1 += kq < k1 || (kq == k1 && q < l2) ? 1 : 0;
-        }
+        sb.ord[r] = (uint16_t)e;
     }
     __syncwarp();
-    if (lane < c) {
-        keys[p0] = k0;
-        rows[p0] = r0;
-    }
-    if (l2 < c) {
-        keys[p1] = k1;
-        rows[p1] = r1;
-    }
-    __syncwarp();
+    return __any_sync(0xFFFFFFFFu, ties) ? 1 : 0;
 }
 
 // Warp bitonic sort of (key, row) over P (power of two) entries of a list;
@@ -262,25 +306,35 @@ __device__ __forceinline__ double column_total(const ColInfo &c, float rem) {
     return rem == 0.0f ? t : t + scalbn((double)rem, -c.sigma);
 }
 
-// Entries of one pair from its sorted in-range list (c > 0 rows).
-template <typename T>
+// Entries of one pair from its in-range list (c > 0 rows); ord: its order, or
+// null for a sorted list; ties: whether keys may be equal.
+template <typename T, bool REM>
 __device__ void emit_path(const PathArgs<T> &a, int64_t p, T v0, bool pos,
-                          const typename Traits<T>::K *keys, const uint32_t *rows, int c,
-                          const Column<T> &col, const ColInfo &cj, const ColInfo &ck,
-                          const ListSums &ls, float remj, float remk, const T *xk, int lane) {
+                          const typename Traits<T>::K *keys, const uint32_t *rows,
+                          const uint16_t *ord, bool ties, int c, const Column<T> &col, const ColInfo &cj, const ColInfo &ck,
+                          const ListSums &ls, bool rem_, const T *xk, int lane) {
     using Tr = Traits<T>;
+    using K = typename Tr::K;
     // corrections of a run: double input's lie below the fixed point's units
     using QC = typename std::conditional<sizeof(T) == 4, int64_t, float>::type;
     const unsigned FULL = 0xFFFFFFFFu;
     const int64_t Q = cj.Q;
+    const bool rem = REM && rem_;
+    const float remj = rem ? a.crem[p / a.m] : 0.0f, remk = rem ? a.crem[p % a.m] : 0.0f;
     const int64_t o = a.off[p];
     const int64_t room = a.off[p + 1] - o;  // entries the count pass reserved
+    auto at = [&](int i) -> int { return ord ? (int)ord[i] : i; };
+    // whether run ends (starts) lie at place i, whose key is ki
+    auto ends = [&](int i, K ki) { return i == c - 1 || !ties || ki != keys[at(i + 1)]; };
+    auto starts = [&](int i, K ki) { return i == 0 || !ties || ki != keys[at(i - 1)]; };
     // number of runs of equal keys
-    int groups = 0;
-    for (int i0 = 0; i0 < c; i0 += 32) {
-        const int i = i0 + lane;
-        const bool end = i < c && (i == c - 1 || keys[i] != keys[i + 1]);
-        groups += __popc(__ballot_sync(FULL, end));
+    int groups = c;
+    if (ties) {
+        groups = 0;
+        for (int i0 = 0; i0 < c; i0 += 32) {
+            const int i = i0 + lane;
+            groups += __popc(__ballot_sync(FULL, i < c && ends(i, keys[at(i)])));
+        }
     }
     // the entries 0 .. groups lie inside the room the count pass reserved
     L1L_CHK((int64_t)groups, room);
@@ -291,10 +345,12 @@ __device__ void emit_path(const PathArgs<T> &a, int64_t p, T v0, bool pos,
     int gbase = 0;           // runs ended before this chunk
     for (int i0 = 0; i0 < c; i0 += 32) {
         const int i = i0 + lane;
-        const uint32_t row = i < c ? rows[i] : 0u;
+        const int e0 = i < c ? at(i) : 0;
+        const uint32_t row = i < c ? rows[e0] : 0u;
+        const K ki = keys[e0];
         const int64_t q = i < c ? col.q[row] : 0;
         const int64_t S = carry + warp_scan_add(q, lane);  // S(key_i) at a run end
-        const bool end = i < c && (i == c - 1 || keys[i] != keys[i + 1]);
+        const bool end = i < c && ends(i, ki);
         const unsigned em = __ballot_sync(FULL, end);
         const int g = gbase + __popc(em & ((1u << lane) - 1u));  // run index (ascending)
         const int64_t D = 2 * S - Q;
@@ -311,7 +367,7 @@ __device__ void emit_path(const PathArgs<T> &a, int64_t p, T v0, bool pos,
             if (i < c) {
                 const T b = col.x[row], x = xk[row];
                 const T sx = b < T(0) ? -x : x;
-                t = Tr::value(keys[i]);
+                t = Tr::value(ki);
                 int e = 0;
                 xq = fixq(fabs(x), ck.sigma, e);
                 // the remainder of a correctly rounded division is exact in
@@ -320,8 +376,6 @@ __device__ void emit_path(const PathArgs<T> &a, int64_t p, T v0, bool pos,
                 if constexpr (sizeof(T) == 8) {
                     const T d = fma(-t, fabs(b), sx);
                     if (d > T(0)) qc = (float)scalbn(2.0 * d, ck.sigma);
-                    wr = col.rem[row];
-                    xr = fix_rem(x, ck.sigma);
                 } else if (fabs(x) >= T(0x1p-100)) {
                     const T d = fma(-t, fabs(b), sx);
                     if (d > T(0)) qc = fixq(T(2) * d, ck.sigma, e);
@@ -329,9 +383,13 @@ __device__ void emit_path(const PathArgs<T> &a, int64_t p, T v0, bool pos,
                     const double d = fma(-(double)t, fabs((double)b), (double)sx);
                     if (d > 0.0) qc = fixq(2.0 * d, ck.sigma, e);
                 }
+                if (rem) {
+                    wr = col.rem_of(row);
+                    xr = fix_rem(x, ck.sigma);
+                }
             }
             float Sr = 0.0f, Br = 0.0f;
-            if constexpr (sizeof(T) == 8) {
+            if (rem) {
                 Sr = cSr + warp_scan_add(wr, lane);
                 Br = cBr + warp_scan_add(xr, lane);
                 cSr = __shfl_sync(FULL, Sr, 31);
@@ -339,10 +397,12 @@ __device__ void emit_path(const PathArgs<T> &a, int64_t p, T v0, bool pos,
             }
             const int64_t B = cB + warp_scan_add(xq, lane);
             QC run_q = 0;
-            if (__any_sync(FULL, qc != 0) || crun != 0) {
+            if (!ties) {  // every row is a run
+                run_q = qc;
+            } else if (__any_sync(FULL, qc != 0) || crun != 0) {
                 const QC Qi = warp_scan_add(qc, lane);  // inclusive, this chunk only
                 // run sums of qc: the run's start holds the prefix before it
-                const bool start = i < c && (i == 0 || keys[i - 1] != keys[i]);
+                const bool start = i < c && starts(i, ki);
                 const unsigned smk = __ballot_sync(FULL, start);
                 const unsigned upto = smk & (lane == 31 ? FULL : ((2u << lane) - 1u));
                 const int hs = upto ? 31 - __clz(upto) : -1;
@@ -353,15 +413,15 @@ __device__ void emit_path(const PathArgs<T> &a, int64_t p, T v0, bool pos,
             if (end) {  // each run writes the residual of its own entry
                 const int slot = pos ? groups - 1 - g : g;
                 int64_t F = ck.Q - 2 * (pos ? B : ls.Ball - B);
-                if constexpr (sizeof(T) == 4) {
-                    F += run_q;
-                    a.res[o + slot] = fma((double)t, Dd, fix_to_double(F, ck.sigma));
-                } else {
-                    const float fr = remk - 2.0f * (pos ? Br : ls.Brem - Br) + run_q;
-                    const double dr = scalbn((double)(2.0f * Sr - remj), -cj.sigma);
-                    a.res[o + slot] = fma(t, Dd + dr, fix_to_double(F, ck.sigma) +
-                                                          scalbn((double)fr, -ck.sigma));
+                if constexpr (sizeof(T) == 4) F += run_q;
+                double Ft = fix_to_double(F, ck.sigma), Dt = Dd;
+                if (rem) {
+                    float fr = remk - 2.0f * (pos ? Br : ls.Brem - Br);
+                    if constexpr (sizeof(T) == 8) fr += run_q;
+                    Ft += scalbn((double)fr, -ck.sigma);
+                    Dt += scalbn((double)(2.0f * Sr - remj), -cj.sigma);
                 }
+                a.res[o + slot] = fma((double)t, Dt, Ft);
             }
             // the run still open at the end of this chunk carries its partial sum
             crun = __shfl_sync(FULL, run_q, 31);
@@ -372,12 +432,12 @@ __device__ void emit_path(const PathArgs<T> &a, int64_t p, T v0, bool pos,
                 // run g (not the top one) starts at Q - 2 S(t_g), slot groups-1-g
                 if (g < groups - 1) {
                     a.lam[o + groups - 1 - g] = D < 0 ? -Dd : 0.0;
-                    a.val[o + groups - 1 - g] = Tr::value(keys[i]);
+                    a.val[o + groups - 1 - g] = Tr::value(ki);
                 }
             } else {
                 // the run after g starts at 2 S(t_g) - Q; after the last, 0
                 a.lam[o + g + 1] = D > 0 ? Dd : 0.0;
-                a.val[o + g + 1] = g + 1 < groups ? Tr::value(keys[i + 1]) : T(0);
+                if (g > 0) a.val[o + g] = Tr::value(ki);
             }
         }
         carry = __shfl_sync(FULL, S, 31);
@@ -389,8 +449,8 @@ __device__ void emit_path(const PathArgs<T> &a, int64_t p, T v0, bool pos,
         if (pos) {
             const int64_t D = Q - 2 * ls.Sbelow;
             a.lam[o + groups] = D > 0 ? fix_to_double(D, cj.sigma) : 0.0;
-            a.val[o + groups] = T(0);
         }
+        a.val[o + groups] = T(0);
         if (a.res) a.res[o + groups] = column_total(ck, remk);  // v = 0
         a.len[p] = groups + 1;
     }
@@ -401,9 +461,9 @@ __device__ void emit_path(const PathArgs<T> &a, int64_t p, T v0, bool pos,
 // most cap; the total is returned either way), sums the exact weight below the
 // range and, with residuals, the fixed-point |x_ik| of the range.  The column
 // arrays hold a multiple of 128 rows, zero past n.
-template <typename T, bool COUNT>
+template <typename T, bool COUNT, bool REM>
 __device__ int scan_rows(const PathArgs<T> &a, int64_t k, const Column<T> &col, uint16_t *pend,
-                         bool wide, bool pos, uint32_t ck_lo, uint32_t ck_hi,
+                         bool wide, bool rem_, bool pos, uint32_t ck_lo, uint32_t ck_hi,
                          typename Traits<T>::K kv, int sigma_k, typename Traits<T>::K *keys,
                          uint32_t *rows, int cap, ListSums &ls, int lane) {
     using Tr = Traits<T>;
@@ -413,7 +473,7 @@ __device__ int scan_rows(const PathArgs<T> &a, int64_t k, const Column<T> &col, 
     const T *xk = a.Xt + k * a.ldn;
     const float4 *xf = reinterpret_cast<const float4 *>(a.Xf + k * a.ldn);
     const int ng = ((int)a.n + 127) >> 7;
-    const bool want_r = !COUNT && a.res != nullptr;
+    const bool want_r = !COUNT && a.res != nullptr, rem = REM && rem_;
     // Rows with a coarse key outside [ck_lo - G, ck_hi + G] are certainly
     // below or above; [va, vb] holds the ratios of the others, and |fma(x,
     // inv, -cen)| differs from |fl(x inv) - cen| by at most 3 roundings of
@@ -427,7 +487,6 @@ __device__ int scan_rows(const PathArgs<T> &a, int64_t k, const Column<T> &col, 
     int c = 0, np = 0;
     int64_t sb = 0, bl = 0;
     float sr = 0.0f, br = 0.0f;  // their remainders
-    const bool want_rem = !COUNT && with_rem(a);
     // the queue's first 32 rows (fewer at the end): exact keys, list append
     auto flush = [&](int cnt) {
         int cls = 1;
@@ -442,7 +501,7 @@ __device__ int scan_rows(const PathArgs<T> &a, int64_t k, const Column<T> &col, 
         }
         if (!COUNT && cls < 0) {
             sb += col.q[i];
-            if (want_rem) sr += col.rem[i];
+            if (rem) sr += col.rem_of(i);
         }
         const unsigned im = __ballot_sync(FULL, cls == 0);
         if (!COUNT && cls == 0) {
@@ -452,9 +511,8 @@ __device__ int scan_rows(const PathArgs<T> &a, int64_t k, const Column<T> &col, 
                 rows[at] = (uint32_t)i;
             }
             int e = 0;
-            if (want_r) bl += fixq(fabs(x), sigma_k, e);
-            if constexpr (sizeof(T) == 8)
-                if (want_rem) br += fix_rem(x, sigma_k);
+            if (want_r && !pos) bl += fixq(fabs(x), sigma_k, e);
+            if (rem && !pos) br += fix_rem(x, sigma_k);
         }
         c += __popc(im);
     };
@@ -480,12 +538,19 @@ __device__ int scan_rows(const PathArgs<T> &a, int64_t k, const Column<T> &col, 
                 if (z[1] <= -delta) sb += qa.y;
                 if (z[2] <= -delta) sb += qb.x;
                 if (z[3] <= -delta) sb += qb.y;
-                if (want_rem) {
-                    const float4 r4 = *reinterpret_cast<const float4 *>(col.rem + i);
-                    if (z[0] <= -delta) sr += r4.x;
-                    if (z[1] <= -delta) sr += r4.y;
-                    if (z[2] <= -delta) sr += r4.z;
-                    if (z[3] <= -delta) sr += r4.w;
+                if (rem) {
+                    if constexpr (sizeof(T) == 8) {
+                        const float4 r4 = *reinterpret_cast<const float4 *>(col.rem + i);
+                        if (z[0] <= -delta) sr += r4.x;
+                        if (z[1] <= -delta) sr += r4.y;
+                        if (z[2] <= -delta) sr += r4.z;
+                        if (z[3] <= -delta) sr += r4.w;
+                    } else {
+#pragma unroll 1
+                        for (int u = 0; u < 4; ++u)
+                            if (fmaf(a.Xf[k * a.ldn + i + u], col.inv[i + u], -cen) <= -delta)
+                                sr += col.rem_of(i + u);
+                    }
                 }
             }
             mask |= f << (4 * (g - g0));
@@ -515,8 +580,8 @@ __device__ int scan_rows(const PathArgs<T> &a, int64_t k, const Column<T> &col, 
     if (!COUNT) {
         ls.Sbelow = warp_sum_i64(sb);
         ls.Ball = want_r ? warp_sum_i64(bl) : 0;
-        ls.Srem = want_rem ? warp_sum_f32(sr) : 0.0f;
-        ls.Brem = want_rem ? warp_sum_f32(br) : 0.0f;
+        ls.Srem = rem ? warp_sum_f32(sr) : 0.0f;
+        ls.Brem = rem ? warp_sum_f32(br) : 0.0f;
     }
     __syncwarp();
     return c;
@@ -527,8 +592,12 @@ __device__ __forceinline__ bool pair_is_wide(const PathArgs<T> &a, const ColInfo
     return (cj.flags & COL_WIDE) != 0 || (sizeof(T) == 8 && (a.ci[k].flags & COL_WIDE));
 }
 
-template <typename T, bool COUNT>
-__global__ void __launch_bounds__(PW * 32) k_path_pass(PathArgs<T> a, int kchunk, int cap) {
+// REM: with remainders.  They cost a fifth of the write pass in registers even
+// where there are none, so with residuals of float input both are launched and
+// `inexact` says which of them has the work (USE_FLAG).
+template <typename T, bool COUNT, bool REM, bool USE_FLAG>
+__global__ void __launch_bounds__(PW * 32, 4) k_path_pass(PathArgs<T> a, int kchunk, int cap) {
+    if (USE_FLAG && (*a.inexact != 0) != REM) return;
     using Tr = Traits<T>;
     using K = typename Tr::K;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -540,14 +609,17 @@ __global__ void __launch_bounds__(PW * 32) k_path_pass(PathArgs<T> a, int kchunk
     o += (size_t)npad * 4;
     int64_t *colq = reinterpret_cast<int64_t *>(smem + o);
     o += (size_t)npad * 8;
-    uint16_t *pend = reinterpret_cast<uint16_t *>(smem + o) + warp * PEND;
-    o += (size_t)PW * PEND * 2;
     K *keys = reinterpret_cast<K *>(smem + o + (size_t)warp * cap * (sizeof(K) + 4));
     uint32_t *rows = reinterpret_cast<uint32_t *>(keys + cap);
+    o += (size_t)PW * cap * (sizeof(K) + 4) + (size_t)warp * sort_bytes(cap);
+    SortBuf sb;
+    sb.cnt = reinterpret_cast<uint32_t *>(smem + o);
+    sb.part = reinterpret_cast<uint16_t *>(smem + o + PBUCK * 4);
+    sb.ord = sb.part + cap;
+    static_assert(PEND <= PATH_CAP_MIN, "the queue lies in the first index array");
     const int64_t j = blockIdx.x;
     const Column<T> col = stage_column<T>(a, j, own, inv, colq, npad, threadIdx.x, PW * 32);
     __syncthreads();
-    const float remj = with_rem(a) ? a.crem[j] : 0.0f;
     const ColInfo cj = a.ci[j];
     const int64_t k0 = (int64_t)blockIdx.y * kchunk, k1 = min(a.m, k0 + kchunk);
     for (int64_t k = k0 + warp; k < k1; k += PW) {
@@ -564,7 +636,7 @@ __global__ void __launch_bounds__(PW * 32) k_path_pass(PathArgs<T> a, int kchunk
                     // v = 1 for k == jhat: zero residual; v = 0: sum |x_ik|
                     if (a.res)
                         a.res[off] = k == j ? 0.0
-                                            : column_total(a.ci[k], with_rem(a) ? a.crem[k] : 0.0f);
+                                            : column_total(a.ci[k], a.crem[k]);
                     a.len[p] = 1;
                 }
             }
@@ -576,9 +648,10 @@ __global__ void __launch_bounds__(PW * 32) k_path_pass(PathArgs<T> a, int kchunk
         range_of<T>(v0, pos, ck_lo, ck_hi, kv);
         const bool wide = pair_is_wide<T>(a, cj, k);
         const ColInfo ck = a.ci[k];
+        const bool rem = REM && with_rem(a, cj, ck);
         ListSums ls{};
-        const int c = scan_rows<T, COUNT>(a, k, col, pend, wide, pos, ck_lo, ck_hi, kv, ck.sigma,
-                                          keys, rows, cap, ls, lane);
+        const int c = scan_rows<T, COUNT, REM>(a, k, col, sb.part, wide, rem, pos, ck_lo, ck_hi, kv,
+                                          ck.sigma, keys, rows, cap, ls, lane);
         if (COUNT) {
             if (lane == 0) a.bound[p] = (int64_t)c + 1;
             continue;
@@ -587,15 +660,14 @@ __global__ void __launch_bounds__(PW * 32) k_path_pass(PathArgs<T> a, int kchunk
             if (lane == 0) a.big[atomicAdd(a.big_count, 1u)] = (int32_t)(p);
             continue;
         }
-        if (c <= 64) {
-            warp_rank_sort<K>(keys, rows, c, lane);
-        } else {
-            int P = 128;
-            while (P < c) P <<= 1;
+        const int ties = warp_bucket_sort<T>(keys, c, v0, sb, lane);
+        if (ties < 0) {
+            int P = 32;
+            while (P < c) P <<= 1;  // at most cap, a power of two
             warp_list_sort<K>(keys, rows, c, P, lane);
         }
-        emit_path<T>(a, p, v0, pos, keys, rows, c, col, cj, ck, ls, remj,
-                     with_rem(a) ? a.crem[k] : 0.0f, a.Xt + k * a.ldn, lane);
+        emit_path<T, REM>(a, p, v0, pos, keys, rows, ties < 0 ? nullptr : sb.ord, ties != 0, c,
+                          col, cj, ck, ls, rem, a.Xt + k * a.ldn, lane);
         __syncwarp();
     }
 }
@@ -633,15 +705,16 @@ __global__ void __launch_bounds__(128) k_path_big(PathArgs<T> a) {
         uint32_t ck_lo, ck_hi;
         K kv;
         range_of<T>(v0, pos, ck_lo, ck_hi, kv);
+        const bool rem = with_rem(a, cj, ck);
         ListSums ls{};
-        const int c = scan_rows<T, false>(a, k, col, s_pend[threadIdx.x >> 5],
-                                          pair_is_wide<T>(a, cj, k), pos, ck_lo, ck_hi, kv,
+        const int c = scan_rows<T, false, true>(a, k, col, s_pend[threadIdx.x >> 5],
+                                          pair_is_wide<T>(a, cj, k), rem, pos, ck_lo, ck_hi, kv,
                                           ck.sigma, keys, rows, (int)a.slice, ls, lane);
         int P = 32;
         while (P < c) P <<= 1;
         warp_list_sort<K>(keys, rows, c, P, lane);
-        emit_path<T>(a, p, v0, pos, keys, rows, c, col, cj, ck, ls, with_rem(a) ? a.crem[j] : 0.0f,
-                     with_rem(a) ? a.crem[k] : 0.0f, a.Xt + k * a.ldn, lane);
+        emit_path<T, true>(a, p, v0, pos, keys, rows, nullptr, true, c, col, cj, ck, ls, rem,
+                     a.Xt + k * a.ldn, lane);
         __syncwarp();
     }
 }
@@ -721,8 +794,7 @@ template <typename T> size_t path_slice_bytes(int64_t n) {
 // Shared memory of a CTA with lists of `cap` entries.
 template <typename T> size_t path_smem_bytes(int64_t n, int cap) {
     const size_t npad = (size_t)((n + ROW_PAD - 1) & ~int64_t(ROW_PAD - 1));
-    return npad * 16 + (size_t)PW * PEND * 2 +
-           (size_t)PW * cap * (sizeof(typename Traits<T>::K) + 4);
+    return npad * 16 + (size_t)PW * (cap * (sizeof(typename Traits<T>::K) + 4) + sort_bytes(cap));
 }
 
 // The limit on n is a fixed one (13,504 float, 10,368 double): the rows, in
@@ -750,7 +822,8 @@ cudaError_t launch_path(bool count, const T *Xt, const float *Xf, const ColInfo 
     a.ldn = ldn;
     a.v0 = v0;
     a.status = status;
-    const int cap = path_smem_bytes<T>(n, PATH_CAP) <= 227 * 1024 ? PATH_CAP : PATH_CAP_MIN;
+    // the count pass keeps no list, only the queue
+    const int cap = count ? PEND : path_smem_bytes<T>(n, PATH_CAP) <= 227 * 1024 ? PATH_CAP : PATH_CAP_MIN;
     const size_t smem = path_smem_bytes<T>(n, cap);
     const int64_t chunks = std::max<int64_t>(1, std::min<int64_t>((m + PW - 1) / PW,
                                                                   (num_sms * 8 + m - 1) / m));
@@ -759,7 +832,7 @@ cudaError_t launch_path(bool count, const T *Xt, const float *Xf, const ColInfo 
     cudaError_t e;
     if (count) {
         a.bound = bound_or_off;
-        auto kern = k_path_pass<T, true>;
+        auto kern = k_path_pass<T, true, false, false>;
         if ((e = ensure_smem(reinterpret_cast<const void *>(kern), smem)) != cudaSuccess) return e;
         kern<<<grid, PW * 32, smem, st>>>(a, kchunk, cap);
         launches++;
@@ -776,21 +849,33 @@ cudaError_t launch_path(bool count, const T *Xt, const float *Xf, const ColInfo 
     a.big = big;
     a.big_count = big_count;
     a.big_next = big_count + 1;
+    a.inexact = big_count + 2;
     a.scratch = scratch;
     int64_t P = 32;
     while (P < n) P <<= 1;
     a.slice = P;
-    if ((e = cudaMemsetAsync(big_count, 0, 2 * sizeof(uint32_t), st)) != cudaSuccess) return e;
-    if (sizeof(T) == 8 && res) {
+    if ((e = cudaMemsetAsync(big_count, 0, 3 * sizeof(uint32_t), st)) != cudaSuccess) return e;
+    auto pass = [&](auto kern) -> cudaError_t {
+        cudaError_t r = ensure_smem(reinterpret_cast<const void *>(kern), smem);
+        if (r != cudaSuccess) return r;
+        kern<<<grid, PW * 32, smem, st>>>(a, kchunk, cap);
+        launches++;
+        return cudaGetLastError();
+    };
+    if (!res) {
+        e = pass(k_path_pass<T, false, false, false>);
+    } else {
         k_colrem<T><<<(unsigned)m, 256, 0, st>>>(a);
         launches++;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if constexpr (sizeof(T) == 8) {
+            e = pass(k_path_pass<T, false, true, false>);
+        } else {
+            e = pass(k_path_pass<T, false, false, true>);
+            if (e == cudaSuccess) e = pass(k_path_pass<T, false, true, true>);
+        }
     }
-    auto kern = k_path_pass<T, false>;
-    if ((e = ensure_smem(reinterpret_cast<const void *>(kern), smem)) != cudaSuccess) return e;
-    kern<<<grid, PW * 32, smem, st>>>(a, kchunk, cap);
-    launches++;
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (e != cudaSuccess) return e;
     k_path_big<T><<<path_big_workers() / 4, 128, 0, st>>>(a);
     launches++;
     return cudaGetLastError();

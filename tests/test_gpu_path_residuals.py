@@ -66,3 +66,12 @@ def test_residuals_of_magnitudes_beyond_the_approximate_keys(scale):
     rng = np.random.default_rng(4)
     X = rng.uniform(-1, 1, size=(200, 4)) * np.array(scale)
     _check(np.ascontiguousarray(X.astype(np.float32)))
+
+
+def test_residuals_of_a_column_beyond_the_fixed_point():
+    # one row 2^40 or 2^28 above the others: the fixed point drops the others' low bits
+    rng = np.random.default_rng(5)
+    X = rng.uniform(-1, 1, size=(1030, 4))
+    X[17, 1] = 2.0 ** 40
+    X[19, 2] = -2.0 ** 28
+    _check(np.ascontiguousarray(X.astype(np.float32)))
