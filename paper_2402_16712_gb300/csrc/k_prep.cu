@@ -25,6 +25,54 @@ __global__ void __launch_bounds__(256) k_transpose(const T *__restrict__ X, T *_
     }
 }
 
+// The same for up to NARROW columns and many rows: a CTA's NR_ROWS rows are one
+// contiguous run of X, read 16 bytes a thread (where X is aligned) and written a
+// column at a time.  Half or more of a 32 x 32 tile is empty there: 1,000,000 x
+// 16 float 73 us (1.8 TB/s), 21 us here.
+constexpr int NARROW = 16, NR_ROWS = 256;
+template <typename T>
+__global__ void __launch_bounds__(256) k_transpose_narrow(const T *__restrict__ X,
+                                                          T *__restrict__ Xt,
+                                                          float *__restrict__ Xf, int64_t n,
+                                                          int m, int64_t ldn, uint32_t *status) {
+    using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+    constexpr int W = 16 / sizeof(T);
+    __shared__ T tile[NR_ROWS * (NARROW + 1)];
+    const int64_t r0 = (int64_t)blockIdx.x * NR_ROWS;
+    const int rows = (int)std::max<int64_t>(0, std::min<int64_t>(NR_ROWS, n - r0));
+    const int total = rows * m, ms = m | 1;  // odd row stride: no bank conflicts
+    const T *x = X + r0 * m;
+    bool bad = false;
+    const bool vec = (reinterpret_cast<uintptr_t>(X) & 15) == 0;  // r0 m is a multiple of W
+    for (int e = threadIdx.x * W; e < total; e += 256 * W) {
+        T v[W];
+        if (vec && e + W <= total) {
+            const V q = __ldg(reinterpret_cast<const V *>(x + e));
+            v[0] = q.x, v[1] = q.y;
+            if constexpr (W == 4) v[2] = q.z, v[3] = q.w;
+        } else {
+#pragma unroll
+            for (int u = 0; u < W; ++u) v[u] = e + u < total ? x[e + u] : T(0);
+        }
+        int r = e / m, c = e - r * m;
+#pragma unroll
+        for (int u = 0; u < W; ++u) {
+            if (e + u < total) tile[r * ms + c] = v[u];
+            bad |= !isfinite(v[u]);
+            if (++c == m) {
+                c = 0;
+                ++r;
+            }
+        }
+    }
+    if (__any_sync(0xFFFFFFFFu, bad) && (threadIdx.x & 31) == 0) atomicOr(status, ST_NONFINITE);
+    __syncthreads();
+    const int r = threadIdx.x;
+    if (r0 + r < ldn)
+        for (int c = 0; c < m; ++c)
+            put_column<T>(Xt, Xf, m, ldn, c, r0 + r, r < rows ? tile[r * ms + c] : T(0));
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256) k_colprep(const T *__restrict__ Xt, ColInfo *ci,
                                                  int64_t n, int64_t ldn) {
@@ -154,7 +202,12 @@ cudaError_t launch_prep(const T *X, T *Xt, float *Xf, ColInfo *ci, int64_t n, in
     dim3 tb(32, 8);
     const int64_t tiles_r = (ldn + 31) / 32;
     dim3 tg((unsigned)((m + 31) / 32), (unsigned)std::min<int64_t>(tiles_r, 65535));
-    k_transpose<T><<<tg, tb, 0, st>>>(X, Xt, Xf, n, m, ldn, status, tiles_r);
+    // fewer rows than that leave SMs without a CTA of NR_ROWS
+    if (m <= NARROW && n >= 152 * NR_ROWS)
+        k_transpose_narrow<T><<<(unsigned)((ldn + NR_ROWS - 1) / NR_ROWS), 256, 0, st>>>(
+            X, Xt, Xf, n, (int)m, ldn, status);
+    else
+        k_transpose<T><<<tg, tb, 0, st>>>(X, Xt, Xf, n, m, ldn, status, tiles_r);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     launches++;

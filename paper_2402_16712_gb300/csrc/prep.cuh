@@ -6,6 +6,20 @@
 
 namespace l1l {
 
+// x_rc into the column-major copies.
+template <typename T>
+__device__ __forceinline__ void put_column(T *__restrict__ Xt, float *__restrict__ Xf, int64_t m,
+                                           int64_t ldn, int64_t c, int64_t r, T v) {
+    Xt[c * ldn + r] = v;
+    if constexpr (sizeof(T) == 8) {
+        // the float pair of the double residual: hi, then (at m ldn further)
+        // lo = fl(v - hi), where v - hi is exact in double
+        const float hi = (float)v;
+        Xf[c * ldn + r] = hi;
+        Xf[(m + c) * ldn + r] = (float)(v - (double)hi);
+    }
+}
+
 // X (n x m, row-major, rows = points) -> Xt (m x ldn, column-major, rows
 // n..ldn-1 zero), and for double input also Xf, the same copy rounded to float
 // (the pair kernel's approximate keys read it, so they need no conversion on
@@ -37,17 +51,7 @@ __device__ __forceinline__ void transpose_tile(const T *__restrict__ X, T *__res
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         int64_t c = c0 + ty + 8 * q, r = r0 + tx;
-        if (c < m && r < ldn) {
-            const T v = tile[tx][ty + 8 * q];
-            Xt[c * ldn + r] = v;
-            if constexpr (sizeof(T) == 8) {
-                // the float pair of the double residual: hi, then (at m ldn
-                // further) lo = fl(v - hi), where v - hi is exact in double
-                const float hi = (float)v;
-                Xf[c * ldn + r] = hi;
-                Xf[(m + c) * ldn + r] = (float)(v - (double)hi);
-            }
-        }
+        if (c < m && r < ldn) put_column<T>(Xt, Xf, m, ldn, c, r, tile[tx][ty + 8 * q]);
     }
 }
 
