@@ -113,8 +113,9 @@ cudaError_t launch_featstd(const float *raw, int64_t m, float *stdz, cudaStream_
 // The R rows of largest l1 norm of the row-major X (rho: row norms [n],
 // rows: their indices in ascending order [R]) copied into Y (R x m).
 template <typename T>
-cudaError_t launch_heavy_rows(const T *X, int64_t n, int64_t m, int64_t R, float *rho,
-                              int32_t *rows, T *Y, cudaStream_t st, int &launches);
+cudaError_t launch_heavy_rows(const T *X, const T *Xt, int64_t ldn, int64_t n, int64_t m,
+                              int64_t R, float *rho, int32_t *rows, T *Y, cudaStream_t st,
+                              int &launches);
 // *dst |= *src (device status words), one thread.
 cudaError_t launch_status_or(uint32_t *dst, const uint32_t *src, cudaStream_t st, int &launches);
 // raw[j][c] = z[j] for j < m.
