@@ -177,6 +177,8 @@ template <typename T> struct Scan {
     unsigned char *base = nullptr;
     cudaStream_t st = nullptr;
     int launches = 0;
+    bool counter_zero = false;  // the prep has zeroed slow_count too
+    bool reduced = true;        // z is summed (else scan_argmin does it)
 };
 
 template <typename T>
@@ -223,7 +225,10 @@ int scan_setup(const T *X, int64_t n, int64_t m, const double *lambdas, int64_t 
 template <typename T> int scan_prep(const T *X, Scan<T> &c) {
     L1L_RANGE("l1l::stage");
     ScanArgs<T> &a = c.a;
-    if (cudaMemsetAsync(a.status, 0, sizeof(uint32_t), c.st) != cudaSuccess) return L1L_ERR_CUDA;
+    // status and slow_count are the first two 256-byte slots
+    if (cudaMemsetAsync(a.status, 0, c.L.slow_count + sizeof(uint32_t), c.st) != cudaSuccess)
+        return L1L_ERR_CUDA;
+    c.counter_zero = true;
     if (launch_prep<T>(X, const_cast<T *>(a.Xt), const_cast<float *>(a.Xf),
                        const_cast<ColInfo *>(a.ci), a.n, a.m, a.ldn,
                        a.status, c.st, c.launches) != cudaSuccess)
@@ -242,8 +247,10 @@ int scan_pairs_large(Scan<T> &c, const double *lambdas, int64_t nl, const int32_
     for (int64_t t0 = 0; t0 < nl; t0 += MAX_LAMBDA_PER_LAUNCH) {
         const int nlc = (int)((nl - t0) < MAX_LAMBDA_PER_LAUNCH ? (nl - t0) : MAX_LAMBDA_PER_LAUNCH);
         const bool last = t0 + MAX_LAMBDA_PER_LAUNCH >= nl;
-        if (cudaMemsetAsync(a.slow_count, 0, sizeof(uint32_t), c.st) != cudaSuccess)
+        if (!c.counter_zero &&
+            cudaMemsetAsync(a.slow_count, 0, sizeof(uint32_t), c.st) != cudaSuccess)
             return L1L_ERR_CUDA;
+        c.counter_zero = false;
         if (prof && t0 == 0 && cudaEventRecord(g_ev_start, c.st) != cudaSuccess)
             return L1L_ERR_CUDA;
         if (launch_large<T>(a, lambdas, (int)t0, nlc, c.st, c.launches) != cudaSuccess)
@@ -252,7 +259,8 @@ int scan_pairs_large(Scan<T> &c, const double *lambdas, int64_t nl, const int32_
         if (launch_exact<T>(a, lambdas, (int)t0, nlc, c.sms, c.st, c.launches) != cudaSuccess)
             return L1L_ERR_CUDA;
     }
-    if (launch_zreduce(a.s_all, c.z, a.m, nl, jlist, nj, c.st, c.launches) != cudaSuccess)
+    if (c.reduced &&
+        launch_zreduce(a.s_all, c.z, a.m, nl, jlist, nj, c.st, c.launches) != cudaSuccess)
         return L1L_ERR_CUDA;
     return L1L_OK;
 }
@@ -272,8 +280,10 @@ int scan_pairs(Scan<T> &c, const double *lambdas, int64_t nl, const int32_t *jli
     for (int64_t t0 = 0; t0 < nl; t0 += MAX_LAMBDA_PER_LAUNCH) {
         const int nlc = (int)((nl - t0) < MAX_LAMBDA_PER_LAUNCH ? (nl - t0) : MAX_LAMBDA_PER_LAUNCH);
         const bool last = t0 + MAX_LAMBDA_PER_LAUNCH >= nl;
-        if (cudaMemsetAsync(a.slow_count, 0, sizeof(uint32_t), c.st) != cudaSuccess)
+        if (!c.counter_zero &&
+            cudaMemsetAsync(a.slow_count, 0, sizeof(uint32_t), c.st) != cudaSuccess)
             return L1L_ERR_CUDA;
+        c.counter_zero = false;
         if (prof && t0 == 0 && cudaEventRecord(g_ev_start, c.st) != cudaSuccess)
             return L1L_ERR_CUDA;
         if (launch_pairs<T>(a, lambdas, (int)t0, nlc, plan, c.st, c.launches) != cudaSuccess)
@@ -282,7 +292,8 @@ int scan_pairs(Scan<T> &c, const double *lambdas, int64_t nl, const int32_t *jli
         if (launch_exact<T>(a, lambdas, (int)t0, nlc, c.sms, c.st, c.launches) != cudaSuccess)
             return L1L_ERR_CUDA;
     }
-    if (launch_zreduce(a.s_all, c.z, a.m, nl, jlist, nj, c.st, c.launches) != cudaSuccess)
+    if (c.reduced &&
+        launch_zreduce(a.s_all, c.z, a.m, nl, jlist, nj, c.st, c.launches) != cudaSuccess)
         return L1L_ERR_CUDA;
     return L1L_OK;
 }
@@ -290,6 +301,12 @@ int scan_pairs(Scan<T> &c, const double *lambdas, int64_t nl, const int32_t *jli
 template <typename T>
 int scan_argmin(Scan<T> &c, int64_t nl, T *out_v, double *out_obj, int32_t *out_jstar) {
     L1L_RANGE("l1l::argmin");
+    if (!c.reduced)
+        return launch_reduce_argmin<T>(c.a.s_all, c.z, c.a.v_all, c.a.m, nl, c.a.jlist, c.a.nj,
+                                       out_v, out_obj, out_jstar, c.st,
+                                       c.launches) == cudaSuccess
+                   ? L1L_OK
+                   : L1L_ERR_CUDA;
     if (launch_argmin<T>(c.z, c.a.v_all, c.a.m, nl, c.a.jlist, c.a.nj, out_v, out_obj, out_jstar,
                          c.st, c.launches) != cudaSuccess)
         return L1L_ERR_CUDA;
@@ -328,6 +345,7 @@ int fit_impl(const T *X, int64_t n, int64_t m, const double *lambdas, int64_t nl
     L1L_TRY(scan_setup<T>(X, n, m, lambdas, nl, nullptr, nullptr, nullptr, ws, ws_bytes, stream,
                           0u, c));
     L1L_TRY(scan_prep<T>(X, c));
+    c.reduced = (jlist ? nj : m) * m > REDUCE_ONE;
     L1L_TRY(scan_pairs<T>(c, lambdas, nl, jlist, jlist ? nj : m));
     L1L_TRY(scan_argmin<T>(c, nl, out_v, out_obj, out_jstar));
     g_last_launches = c.launches;

@@ -264,6 +264,18 @@ constexpr int D0_DEFAULT = 6;
 
 constexpr int MAX_LAMBDA_PER_LAUNCH = 256;
 
+// Programmatic dependent launch (launch_after): a kernel lets the next one of
+// the stream be placed while its own last CTAs run (next_may_start, first
+// thing), and waits for the end of the one before it, whose writes it then
+// sees, before it touches memory (wait_for_previous; no wait where it was
+// launched without the attribute).
+__device__ __forceinline__ void next_may_start() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void wait_for_previous() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Rows of the staged column-major copy (and of the pair kernel's shared
 // column arrays) are padded with zeros to a multiple of ROW_PAD, so that the
 // selection's unrolled passes (4 loads of 32 rows per lane group) never need

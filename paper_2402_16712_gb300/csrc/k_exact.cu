@@ -18,6 +18,8 @@ namespace l1l {
 template <typename T>
 __global__ void __launch_bounds__(128) k_exact(ScanArgs<T> a, const __grid_constant__ LambdaPack lp,
                                                int t0) {
+    next_may_start();
+    wait_for_previous();
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -36,9 +38,8 @@ cudaError_t launch_exact(const ScanArgs<T> &a, const double *lambdas, int t0, in
     LambdaPack lp;
     lp.tl_min = lp.tl_max = 0;
     for (int q = 0; q < nlc; ++q) lp.lam[q] = lambdas[t0 + q];
-    k_exact<T><<<num_sms * 2, 128, 0, st>>>(a, lp, t0);
     launches++;
-    return cudaGetLastError();
+    return launch_after(k_exact<T>, dim3(num_sms * 2), dim3(128), 0, st, a, lp, t0);
 }
 
 template cudaError_t launch_exact<float>(const ScanArgs<float> &, const double *, int, int, int,

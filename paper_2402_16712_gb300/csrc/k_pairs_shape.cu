@@ -39,6 +39,8 @@ __global__ void __launch_bounds__(ShapeBounds<S>::threads, ShapeBounds<S>::block
             int cap) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ Dec32 s_dec[NDEC];
+    next_may_start();
+    wait_for_previous();
     const int64_t k0 = (int64_t)blockIdx.y * kchunk;
     const int64_t k1 = min(a.m, k0 + kchunk);
     const LamView lv{lp.lam, lp.tl_min, lp.tl_max};
@@ -61,8 +63,8 @@ cudaError_t launch_pairs_sh(const ScanArgs<T> &a, const LambdaPack &lp, int t0, 
     cudaError_t e = ensure_smem(reinterpret_cast<const void *>(kern), plan.smem);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)a.nj, (unsigned)plan.kchunks);
-    kern<<<grid, plan.warps * 32, plan.smem, st>>>(a, lp, t0, nlc, plan.kchunk, plan.cap);
-    return cudaGetLastError();
+    return launch_after(kern, grid, dim3(plan.warps * 32), plan.smem, st, a, lp, t0, nlc,
+                        plan.kchunk, plan.cap);
 }
 
 template cudaError_t launch_pairs_sh<float, SH>(const ScanArgs<float> &, const LambdaPack &, int,

@@ -19,6 +19,7 @@ __global__ void __launch_bounds__(256) k_transpose(const T *__restrict__ X, T *_
                                                    float *__restrict__ Xf,
                                                    int64_t n, int64_t m, int64_t ldn,
                                                    uint32_t *status, int64_t tiles_r) {
+    next_may_start();
     for (int64_t tr = blockIdx.y; tr < tiles_r; tr += gridDim.y) {
         transpose_tile<T>(X, Xt, Xf, n, m, ldn, status, blockIdx.x, tr);
         __syncthreads();  // the next row tile refills the shared tile
@@ -76,6 +77,8 @@ __global__ void __launch_bounds__(256) k_transpose_narrow(const T *__restrict__ 
 template <typename T>
 __global__ void __launch_bounds__(256) k_colprep(const T *__restrict__ Xt, ColInfo *ci,
                                                  int64_t n, int64_t ldn) {
+    next_may_start();
+    wait_for_previous();
     colprep_column<T>(Xt + (int64_t)blockIdx.x * ldn, ci + blockIdx.x, n);
 }
 
@@ -213,9 +216,9 @@ cudaError_t launch_prep(const T *X, T *Xt, float *Xf, ColInfo *ci, int64_t n, in
     launches++;
     const int C = large_cluster_size(ldn);
     if (C == 1) {
-        k_colprep<T><<<(unsigned)m, 256, 0, st>>>(Xt, ci, n, ldn);
         launches++;
-        return cudaGetLastError();
+        return launch_after(k_colprep<T>, dim3((unsigned)m), dim3(256), 0, st, (const T *)Xt, ci,
+                            n, ldn);
     }
     // tall columns: one cluster of C CTAs per column
     cudaLaunchAttribute at[1];

@@ -12,6 +12,8 @@ namespace l1l {
 __global__ void __launch_bounds__(32) k_zreduce(const double *__restrict__ s_all,
                                                 double *__restrict__ z_all, int64_t m,
                                                 const int32_t *__restrict__ jlist) {
+    next_may_start();
+    wait_for_previous();
     const int64_t t = blockIdx.y;
     const int64_t j = jlist ? (int64_t)jlist[blockIdx.x] : (int64_t)blockIdx.x;
     if (j < 0 || j >= m) return;  // flagged by the pair kernel
@@ -25,10 +27,9 @@ __global__ void __launch_bounds__(32) k_zreduce(const double *__restrict__ s_all
 // Per lambda: jhat* = smallest index attaining min z (Algorithm 1 keeps the
 // first strict improvement in increasing jhat); copy v^{jhat*} out.
 template <typename T>
-__global__ void __launch_bounds__(256) k_argmin(const double *__restrict__ z_all,
-                                                const T *__restrict__ v_all, int64_t m,
-                                                const int32_t *__restrict__ jlist, int64_t nj,
-                                                T *out_v, double *out_obj, int32_t *out_jstar) {
+__device__ __forceinline__ void argmin_of(const double *z_all, const T *__restrict__ v_all,
+                                          int64_t m, const int32_t *__restrict__ jlist, int64_t nj,
+                                          T *out_v, double *out_obj, int32_t *out_jstar) {
     const int64_t t = blockIdx.x;
     const double *z = z_all + t * m;
     double bz = 0.0;
@@ -70,22 +71,65 @@ __global__ void __launch_bounds__(256) k_argmin(const double *__restrict__ z_all
         out_v[t * m + k] = js >= 0 ? v_all[(t * m + js) * m + k] : T(NAN);
 }
 
+template <typename T>
+__global__ void __launch_bounds__(256) k_argmin(const double *__restrict__ z_all,
+                                                const T *__restrict__ v_all, int64_t m,
+                                                const int32_t *__restrict__ jlist, int64_t nj,
+                                                T *out_v, double *out_obj, int32_t *out_jstar) {
+    wait_for_previous();
+    argmin_of<T>(z_all, v_all, m, jlist, nj, out_v, out_obj, out_jstar);
+}
+
+// Both steps of a small fit in one launch, a CTA per lambda: its warps take the
+// jhat in turn (z summed as above), then the argmin.  A CTA reads nj m values
+// that would be spread over nj SMs otherwise, so only up to REDUCE_ONE of them,
+// which take about as long as a launch.
+template <typename T>
+__global__ void __launch_bounds__(256) k_reduce_argmin(const double *__restrict__ s_all,
+                                                       double *z_all,
+                                                       const T *__restrict__ v_all, int64_t m,
+                                                       const int32_t *__restrict__ jlist,
+                                                       int64_t nj, T *out_v, double *out_obj,
+                                                       int32_t *out_jstar) {
+    wait_for_previous();
+    const int64_t t = blockIdx.x;
+    for (int64_t p = threadIdx.x >> 5; p < nj; p += 8) {
+        const int64_t j = jlist ? (int64_t)jlist[p] : p;
+        if (j < 0 || j >= m) continue;  // flagged by the pair kernel
+        const double *s = s_all + (t * m + j) * m;
+        double acc = 0.0;
+        for (int64_t k = threadIdx.x & 31; k < m; k += 32) acc += s[k];
+        acc = warp_sum_f64(acc);
+        if ((threadIdx.x & 31) == 0) z_all[t * m + j] = acc;
+    }
+    __syncthreads();
+    argmin_of<T>(z_all, v_all, m, jlist, nj, out_v, out_obj, out_jstar);
+}
+
 cudaError_t launch_zreduce(const double *s_all, double *z_all, int64_t m, int64_t n_lambda,
                            const int32_t *jlist, int64_t nj, cudaStream_t st, int &launches) {
     dim3 grid((unsigned)nj, (unsigned)n_lambda);
-    k_zreduce<<<grid, 32, 0, st>>>(s_all, z_all, m, jlist);
     launches++;
-    return cudaGetLastError();
+    return launch_after(k_zreduce, grid, dim3(32), 0, st, s_all, z_all, m, jlist);
 }
 
 template <typename T>
 cudaError_t launch_argmin(const double *z_all, const T *v_all, int64_t m, int64_t n_lambda,
                           const int32_t *jlist, int64_t nj, T *out_v, double *out_obj,
                           int32_t *out_jstar, cudaStream_t st, int &launches) {
-    k_argmin<T><<<(unsigned)n_lambda, 256, 0, st>>>(z_all, v_all, m, jlist, nj, out_v, out_obj,
-                                                    out_jstar);
     launches++;
-    return cudaGetLastError();
+    return launch_after(k_argmin<T>, dim3((unsigned)n_lambda), dim3(256), 0, st, z_all, v_all, m,
+                        jlist, nj, out_v, out_obj, out_jstar);
+}
+
+template <typename T>
+cudaError_t launch_reduce_argmin(const double *s_all, double *z_all, const T *v_all, int64_t m,
+                                 int64_t n_lambda, const int32_t *jlist, int64_t nj, T *out_v,
+                                 double *out_obj, int32_t *out_jstar, cudaStream_t st,
+                                 int &launches) {
+    launches++;
+    return launch_after(k_reduce_argmin<T>, dim3((unsigned)n_lambda), dim3(256), 0, st, s_all,
+                        z_all, v_all, m, jlist, nj, out_v, out_obj, out_jstar);
 }
 
 // Successive components: x'_ik = fl(x_ik - fl(v_k x_ijhat)) (no fused
@@ -124,6 +168,13 @@ template cudaError_t launch_deflate<double>(const double *, double *, int64_t, i
                                             const int32_t *, const double *, int, cudaStream_t,
                                             int &);
 
+template cudaError_t launch_reduce_argmin<float>(const double *, double *, const float *, int64_t,
+                                                 int64_t, const int32_t *, int64_t, float *,
+                                                 double *, int32_t *, cudaStream_t, int &);
+template cudaError_t launch_reduce_argmin<double>(const double *, double *, const double *,
+                                                  int64_t, int64_t, const int32_t *, int64_t,
+                                                  double *, double *, int32_t *, cudaStream_t,
+                                                  int &);
 template cudaError_t launch_argmin<float>(const double *, const float *, int64_t, int64_t,
                                           const int32_t *, int64_t, float *, double *, int32_t *,
                                           cudaStream_t, int &);
