@@ -325,6 +325,7 @@ template <typename T> struct WqFly {
 // (untruncated weights; the search steers by them, the test decides).
 struct Dec32 : Decide {
     uint32_t tneg, tpos;
+    float fneg, fpos, Qf;  // for the sample: the same, and Q / 32
     __device__ __forceinline__ void set(const ColInfo &ci, double lambda) {
         init32(ci, lambda);
         auto clamp = [](int64_t x) -> uint32_t {
@@ -332,6 +333,9 @@ struct Dec32 : Decide {
         };
         tneg = clamp(((Q + Lf) >> 1) + 1);
         tpos = clamp(((Q - Lc) >> 1) + 1);
+        fneg = (float)tneg;
+        fpos = (float)tpos;
+        Qf = (float)Q * (1.0f / 32.0f);
     }
 };
 

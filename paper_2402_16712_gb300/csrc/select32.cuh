@@ -41,11 +41,13 @@
 // Bound (2000 x 2000 float, 32 resident warps): the L1/shared data pipe, ~730
 // wavefronts of 128 bytes per pair at 70% of its rate (pass 1: x, 1/x_ijhat,
 // q and ~2.5 per histogram atomic; pass 2: x and 1/x_ijhat; residual: x and
-// x_ijhat), and ~2600 instructions per pair at 62% of the issue slots.  Against
-// the selection that kept every row of the bracket in a per-lane list: 13.66
-// -> 11.14 ms there; 1000 x 500 with 32 lambdas 5.62 -> 2.61 ms (one selection
-// instead of two and a pass); and without the lists 5000 rows keep 32 warps
-// resident instead of 16, 5000 x 1000 10.23 -> 7.61 ms.
+// x_ijhat), and ~2600 instructions per pair at 62% of the issue slots, ~900 of
+// them whatever the rows.  Against the selection that kept every row of the
+// bracket in a per-lane list: 13.66 -> 11.14 ms there; 1000 x 500 with 32 lambdas
+// 5.62 -> 2.61 ms (one selection instead of two and a pass); and without the lists
+// 5000 rows keep 32 warps resident instead of 16, 5000 x 1000 10.23 -> 7.61 ms.
+// Finding the crossing lane before the bin in it, instead of every bin's prefix
+// sum and test: 11.14 -> 11.06 ms, double 19.36 -> 19.19 ms.
 #pragma once
 #include <cstdint>
 
@@ -228,9 +230,9 @@ __device__ __forceinline__ int candidates32(const float *__restrict__ xf, const 
     // one, cost more to gather and sort than their narrower bracket saved
     // (2000 x 2000 float: 11.4 -> 11.7 ms).
     const float s = warp_sort32f(__fmul_rn(__ldg(xf + w.srow), w.sinv), lane);
-    const float cum = (float)(lane + 1) * ((float)d1.Q * (1.0f / 32.0f));
+    const float cum = (float)(lane + 1) * d1.Qf;
     auto crossing = [&](const Dec32 &d) -> int {
-        const unsigned b = __ballot_sync(FULL, cum >= (float)(s >= 0.0f ? d.tpos : d.tneg));
+        const unsigned b = __ballot_sync(FULL, cum >= (s >= 0.0f ? d.fpos : d.fneg));
         return b ? __ffs(b) - 1 : 31;
     };
     const int j1 = crossing(d1), j2 = TWO ? crossing(d2) : j1;
@@ -289,46 +291,48 @@ __device__ __forceinline__ int candidates32(const float *__restrict__ xf, const 
         }
         Sb = __reduce_add_sync(FULL, Sb);  // <= Q32 < 2^32
         __syncwarp();
-        // ---- the crossing bin(s): lane l scans bins 8l .. 8l+7 -------------
-        uint32_t h[BPL];
+        // ---- the crossing bin(s): first the lane (bins 8l .. 8l+7), then the
+        // bin among its eight.  Whether a bin passes is monotone in the bin.
+        uint32_t tot = 0;
         {
 #pragma unroll
             for (int e = 0; e < BPL; e += 4) {
-                const uint4 h0 = reinterpret_cast<const uint4 *>(hist)[(BPL / 4) * lane + e / 4];
-                h[e] = h0.x, h[e + 1] = h0.y, h[e + 2] = h0.z, h[e + 3] = h0.w;
+                const uint4 h = reinterpret_cast<const uint4 *>(hist)[(BPL / 4) * lane + e / 4];
+                tot += (h.x + h.y) + (h.z + h.w);
             }
-#pragma unroll
-            for (int e = 1; e < BPL; ++e) h[e] += h[e - 1];
-            uint32_t inc = h[BPL - 1];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(FULL, inc, o);
-                if (lane >= o) inc += y;
-            }
-            const uint32_t before = Sb + inc - h[BPL - 1];
-#pragma unroll
-            for (int e = 0; e < BPL; ++e) h[e] += before;
-#pragma unroll
-            for (int e = 0; e < BPL; e += 4)
-                reinterpret_cast<uint4 *>(hist)[(BPL / 4) * lane + e / 4] =
-                    make_uint4(h[e], h[e + 1], h[e + 2], h[e + 3]);
         }
+        uint32_t end = tot;  // weight up to this lane's last bin
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL, end, o);
+            if (lane >= o) end += y;
+        }
+        end += Sb;
         // bins from that of 0 on end at ratios >= 0
         const int zb = bm < Z32 ? 0 : (bm < Z32 + (float)NB32 ? (int)(bm - Z32) : NB32);
-        auto cross_bin = [&](const Dec32 &d) -> int {
-            int fails = 0;
-#pragma unroll
-            for (int e = 0; e < BPL; ++e)
-                fails += h[e] >= (BPL * lane + e >= zb ? d.tpos : d.tneg) ? 0 : 1;
-            const unsigned any = __ballot_sync(FULL, fails < BPL);
+        auto cross_bin = [&](const Dec32 &d, uint32_t &before, uint32_t &through) -> int {
+            const unsigned any =
+                __ballot_sync(FULL, end >= (BPL * lane + BPL - 1 >= zb ? d.tpos : d.tneg));
             if (!any) return NB32;
-            const int ln = __ffs(any) - 1;
-            return BPL * ln + __shfl_sync(FULL, fails, ln);
+            const int ln = __ffs(any) - 1, e = lane & (BPL - 1);
+            const uint32_t q = hist[BPL * ln + e];
+            uint32_t c = q;
+#pragma unroll
+            for (int o = 1; o < BPL; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(FULL, c, o, BPL);
+                if (e >= o) c += y;
+            }
+            c += __shfl_sync(FULL, end - tot, ln);
+            const int at =
+                __ffs(__ballot_sync(FULL, c >= (BPL * ln + e >= zb ? d.tpos : d.tneg))) - 1;
+            through = __shfl_sync(FULL, c, at);
+            before = through - __shfl_sync(FULL, q, at);
+            return BPL * ln + at;
         };
-        const int c1 = cross_bin(d1);
-        const int c2 = TWO ? cross_bin(d2) : c1;
+        uint32_t L1 = 0, E1 = 0, L2 = 0, E2 = 0;
+        const int c1 = cross_bin(d1, L1, E1);
+        const int c2 = TWO ? cross_bin(d2, L2, E2) : c1;
         const int ca = TWO ? min(c1, c2) : c1, cb = TWO ? max(c1, c2) : c1;
-        __syncwarp();
         // ---- the coarse keys [lo, hi] around the crossing and their bins ----
         // r' of bin b: (2^23 + b - bm -+ 1/2) w1, up to a few keys
         const float ra = ((Z32 + (float)ca - bm) - 0.5f) * w1;
@@ -355,8 +359,8 @@ __device__ __forceinline__ int candidates32(const float *__restrict__ xf, const 
             continue;
         }
         if (!(va < vb)) return SEL_W64;  // also NaN: keys past the infinities
-        uint32_t L = hist[ca - 1];
-        const uint32_t W = hist[cb] - L;  // weight of the bins ca .. cb
+        uint32_t L = TWO && c2 < c1 ? L2 : L1;
+        const uint32_t W = (TWO && c2 > c1 ? E2 : E1) - L;  // weight of the bins ca .. cb
         __syncwarp();
         // ---- pass 2: flag the groups with a row in [va, vb], list those rows.
         // |fma(x, inv, -cen)| differs from |r' - cen| by at most 3 roundings
