@@ -128,6 +128,8 @@ template <typename T> struct LgPick {
     long long lq[LG_ROWS];
     int lcnt;                              // their number (read by the cluster)
     long long lsum[3];                     // in the bin, under it, below the range
+    int gcnt[LG_MAXC];                     // every CTA's lcnt and sums, copied here
+    long long gsum[3][LG_MAXC];
     int j1, ia, ib, first;
     long long fl, fw;                      // weight before the crossing bin, its own
     float wsumf[LG_NT / 32];
@@ -215,21 +217,27 @@ __device__ __forceinline__ void lg_bin(float z, uint32_t qh, uint32_t ql, uint32
 template <typename T, int U> struct LgRows {
     float4 vb[U], va[U];
     double2 d0[sizeof(T) == 8 ? U : 1], d1[sizeof(T) == 8 ? U : 1];
+    __device__ __forceinline__ void get(int g, const float *fj, const float *fk, const T *xj,
+                                        int64_t p) {
+        vb[g] = __ldg(reinterpret_cast<const float4 *>(fj) + p);
+        va[g] = __ldg(reinterpret_cast<const float4 *>(fk) + p);
+        if constexpr (sizeof(T) == 8) {
+            d0[g] = __ldg(reinterpret_cast<const double2 *>(xj) + 2 * p);
+            d1[g] = __ldg(reinterpret_cast<const double2 *>(xj) + 2 * p + 1);
+        }
+    }
     __device__ __forceinline__ void load(const float *fj, const float *fk, const T *xj, int64_t v,
                                          int64_t end) {
+        if (v + (U - 1) * LG_NT < end) {  // all but the last step
+#pragma unroll
+            for (int g = 0; g < U; ++g) get(g, fj, fk, xj, v + g * LG_NT);
+            return;
+        }
 #pragma unroll
         for (int g = 0; g < U; ++g) {
-            const int64_t p = v + g * LG_NT;
             vb[g] = va[g] = make_float4(0.f, 0.f, 0.f, 0.f);
             if constexpr (sizeof(T) == 8) d0[g] = d1[g] = make_double2(0.0, 0.0);
-            if (p < end) {
-                vb[g] = __ldg(reinterpret_cast<const float4 *>(fj) + p);
-                va[g] = __ldg(reinterpret_cast<const float4 *>(fk) + p);
-                if constexpr (sizeof(T) == 8) {
-                    d0[g] = __ldg(reinterpret_cast<const double2 *>(xj) + 2 * p);
-                    d1[g] = __ldg(reinterpret_cast<const double2 *>(xj) + 2 * p + 1);
-                }
-            }
+            if (v + g * LG_NT < end) get(g, fj, fk, xj, v + g * LG_NT);
         }
     }
     static __device__ __forceinline__ float at(const float4 &v, int u) {
@@ -402,16 +410,20 @@ __device__ int large_pick(const ScanArgs<T> &a, const ColInfo &ci, int64_t j, in
             h[u] = (long long)x;
             run += h[u];
         }
-        Sb = Sa = 0;
-        for (int r = 0; r < C; ++r) {
-            const unsigned long long *o = cl.map_shared_rank(&sm.tot[buf][0], r);
-            Sb += (long long)o[LG_BINS];
-            Sa += (long long)o[LG_BINS + 1];
+        if (tid < C) {
+            const unsigned long long *o = cl.map_shared_rank(&sm.tot[buf][0], tid);
+            pk.gsum[0][tid] = (long long)o[LG_BINS];
+            pk.gsum[1][tid] = (long long)o[LG_BINS + 1];
         }
         buf ^= 1;
         const long long incl = warp_scan_add(run, lane);
         if (lane == 31) pk.wsum[2][warp] = incl;
         __syncthreads();
+        Sb = Sa = 0;
+        for (int r = 0; r < C; ++r) {
+            Sb += pk.gsum[0][r];
+            Sa += pk.gsum[1][r];
+        }
         long long cum = Sb + incl - run, all = 0;
         for (int w = 0; w < LG_NT / 32; ++w) {
             if (w < warp) cum += pk.wsum[2][w];
@@ -513,14 +525,20 @@ __device__ int large_pick(const ScanArgs<T> &a, const ColInfo &ci, int64_t j, in
         }
         cl.sync();
         // ---- every CTA gathers the cluster's rows ----
+        if (tid < C) {
+            const LgPick<T> *o = cl.map_shared_rank(&pk, tid);
+            pk.gcnt[tid] = o->lcnt;
+            for (int q = 0; q < 3; ++q) pk.gsum[q][tid] = o->lsum[q];
+        }
+        __syncthreads();
         int c = 0;
         in_w = 0;
         long long L = pk.fl;
         for (int r = 0; r < C; ++r) {
             const LgPick<T> *o = cl.map_shared_rank(&pk, r);
-            const int cr = o->lcnt;
-            in_w += o->lsum[0];
-            L += o->lsum[2] - o->lsum[1];
+            const int cr = pk.gcnt[r];
+            in_w += pk.gsum[0][r];
+            L += pk.gsum[2][r] - pk.gsum[1][r];
             for (int e = tid; e < cr && c + e < LG_ROWS; e += LG_NT) {
                 pk.akey[c + e] = o->lkey[e];
                 pk.aq[c + e] = o->lq[e];
@@ -783,12 +801,20 @@ __global__ void __launch_bounds__(LG_NT, 2)
         int nrun = 0;
         for (int64_t v = v0 + tid; v < v1; v += LG_UR * LG_NT) {
             V vb[LG_UR], va[LG_UR];
+            if (v + (LG_UR - 1) * LG_NT < v1) {
 #pragma unroll
-            for (int g = 0; g < LG_UR; ++g) {
-                vb[g] = va[g] = V{};
-                if (v + g * LG_NT < v1) {
+                for (int g = 0; g < LG_UR; ++g) {
                     vb[g] = xjv[v + g * LG_NT];
                     va[g] = xkv[v + g * LG_NT];
+                }
+            } else {
+#pragma unroll
+                for (int g = 0; g < LG_UR; ++g) {
+                    vb[g] = va[g] = V{};
+                    if (v + g * LG_NT < v1) {
+                        vb[g] = xjv[v + g * LG_NT];
+                        va[g] = xkv[v + g * LG_NT];
+                    }
                 }
             }
 #pragma unroll
@@ -818,11 +844,14 @@ __global__ void __launch_bounds__(LG_NT, 2)
             sm.part[buf] = s;
         }
         cl.sync();  // every CTA's partial is visible
-        if (leader) {
+        if (rank == 0 && warp == 0) {  // read together, added in rank order
+            const double x = cl.map_shared_rank(&sm.part[0], min(lane, C - 1))[buf];
             double s = 0.0;
-            for (int r = 0; r < C; ++r) s += cl.map_shared_rank(&sm.part[0], r)[buf];
-            a.v_all[o] = vv;
-            a.s_all[o] = s + lam * (double)fabs(vv);
+            for (int r = 0; r < C; ++r) s += __shfl_sync(0xFFFFFFFFu, x, r);
+            if (leader) {
+                a.v_all[o] = vv;
+                a.s_all[o] = s + lam * (double)fabs(vv);
+            }
         }
         buf ^= 1;
     }
