@@ -214,6 +214,7 @@ int scan_setup(const T *X, int64_t n, int64_t m, const double *lambdas, int64_t 
     a.slow_count = reinterpret_cast<uint32_t *>(c.base + L.slow_count);
     a.slow = reinterpret_cast<SlowEntry *>(c.base + L.slow);
     a.force_exact = (flags & L1L_FLAG_FORCE_EXACT) ? 1 : 0;
+    a.v_only = 0;
     a.inst = 0;
     a.jlist = nullptr;
     a.nj = m;
@@ -394,6 +395,8 @@ int path_count_impl(const T *X, int64_t n, int64_t m, int64_t *offsets, void *ws
     L1L_TRY(scan_setup<T>(X, n, m, &k_zero_lambda, 1, nullptr, nullptr, nullptr, ws, ws_bytes,
                           stream, 0u, c));
     L1L_TRY(scan_prep<T>(X, c));
+    c.a.v_only = 1;
+    c.reduced = false;  // no z
     L1L_TRY(scan_pairs<T>(c, &k_zero_lambda, 1, nullptr, m));  // lambda = 0 medians
     if (launch_path<T>(true, c.a.Xt, c.a.Xf, c.a.ci, n, m, c.a.ldn, c.a.v_all, offsets,
                        reinterpret_cast<int64_t *>(c.base + P.scan_tmp), nullptr, nullptr, nullptr,

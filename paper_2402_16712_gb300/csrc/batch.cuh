@@ -40,6 +40,7 @@ __device__ __forceinline__ ScanArgs<T> inst_args(const BatchDesc<T> &bd, int b,
     a.slow_count = reinterpret_cast<uint32_t *>(ws + 256);
     a.slow = reinterpret_cast<SlowEntry *>(ws + BATCH_HEAD);
     a.force_exact = bd.force_exact;
+    a.v_only = 0;
     a.inst = b;
     a.jlist = nullptr;
     a.nj = a.m;

@@ -248,6 +248,7 @@ template <typename T> struct ScanArgs {
     uint32_t *slow_count;
     SlowEntry *slow;   // capacity n_lambda * m * m
     int force_exact;
+    int v_only;        // medians only: s and z are not needed (the penalty paths)
     int inst;          // instance index recorded in slow-list entries (batched calls)
     const int32_t *jlist;  // device list of the jhat to score (nullptr: all m)
     int64_t nj;            // entries of jlist (m when jlist is nullptr)

@@ -132,9 +132,18 @@ __device__ __forceinline__ double grid_lambda(double lmax, int i) {
     return i == NG - 1 ? lmax : lmax * (u * u);
 }
 
+// |x| as a double; a normal float by integer instructions, which leaves the
+// double pipe to the sums.
+__device__ __forceinline__ double abs64(float x) {
+    const uint32_t u = __float_as_uint(x) & 0x7FFFFFFFu;
+    if (u - 0x00800000u >= 0x7F000000u) return (double)__uint_as_float(u);  // 0, subnormal, inf, NaN
+    return __hiloint2double((int)((u >> 3) + (896u << 20)), (int)(u << 29));
+}
+__device__ __forceinline__ double abs64(double x) { return fabs(x); }
+
 // z_jhat, its right slope and the changes passed, on the grid: warps over k, a
 // lane per grid point, the entry holding there by binary search; sums in a
-// fixed order.  Bound by the three double instructions per pair and point.
+// fixed order.  Bound by the two double additions per pair and point.
 constexpr int EVT = 512;
 template <typename T>
 __global__ void __launch_bounds__(EVT) k_zeval(int64_t m, const int64_t *__restrict__ off,
@@ -161,7 +170,7 @@ __global__ void __launch_bounds__(EVT) k_zeval(int64_t m, const int64_t *__restr
                 hi = mid;
         }
         z += res[o + lo - 1];
-        s += fabs((double)val[o + lo - 1]);
+        s += abs64(val[o + lo - 1]);
         c += lo - 1;
     }
     sz[warp][lane] = z;

@@ -977,7 +977,7 @@ __device__ void emit_pair(const ScanArgs<T> &a, int t, int64_t j, int64_t k, int
         return;
     }
     const T v = Tr::value(ts);
-    const T res = pair_residual<T, CS>(a, j, k, xk, colb, n, v, lane);
+    const T res = a.v_only ? T(0) : pair_residual<T, CS>(a, j, k, xk, colb, n, v, lane);
     if (lane == 0) {
         a.v_all[o] = v;
         a.s_all[o] = (double)res + lam * (double)fabs(v);
