@@ -948,7 +948,8 @@ __device__ __forceinline__ T pair_residual(const ScanArgs<T> &a, int64_t j, int6
 }
 
 // Writes v and s of (lambda t0+tl, jhat, k), or lists the pair for the exact path.
-template <typename T, bool CS>
+// VO: the launch may ask for medians only (the kernels of one or two lambdas).
+template <typename T, bool CS, bool VO>
 __device__ void emit_pair(const ScanArgs<T> &a, int t, int64_t j, int64_t k, int st,
                           typename Traits<T>::K ts, const T *xk, const T *colb, int n,
                           double lam, int lane) {
@@ -977,7 +978,7 @@ __device__ void emit_pair(const ScanArgs<T> &a, int t, int64_t j, int64_t k, int
         return;
     }
     const T v = Tr::value(ts);
-    const T res = a.v_only ? T(0) : pair_residual<T, CS>(a, j, k, xk, colb, n, v, lane);
+    const T res = VO && a.v_only ? T(0) : pair_residual<T, CS>(a, j, k, xk, colb, n, v, lane);
     if (lane == 0) {
         a.v_all[o] = v;
         a.s_all[o] = (double)res + lam * (double)fabs(v);
@@ -985,7 +986,7 @@ __device__ void emit_pair(const ScanArgs<T> &a, int t, int64_t j, int64_t k, int
 }
 
 // One lambda of one pair: the full selection.
-template <typename T, bool CS>
+template <typename T, bool CS, bool VO>
 __device__ void solve_one(const ScanArgs<T> &a, const LamView &lp, int t0, int tl, int64_t j,
                           int64_t k, const T *xk, const float *xf, const WarpCtx<T> &w,
                           bool slow_pair, int lane) {
@@ -997,7 +998,7 @@ __device__ void solve_one(const ScanArgs<T> &a, const LamView &lp, int t0, int t
     } else if (w.cinfo.n_valid > 0) {
         st = select_pair<T>(xk, xf, w, lp, tl, ts, lane);
     }
-    emit_pair<T, CS>(a, t0 + tl, j, k, st, ts, xk, w.colb, w.n, lp.lam[tl], lane);
+    emit_pair<T, CS, VO>(a, t0 + tl, j, k, st, ts, xk, w.colb, w.n, lp.lam[tl], lane);
 }
 
 // Lambda batch (step A7).  The weighted median moves monotonically toward 0
@@ -1064,7 +1065,7 @@ __device__ bool lambda_path(const ScanArgs<T> &a, const LamView &lp, int t0, int
             a.s_all[o] = (double)r + lp.lam[tl] * (double)fabs(v);
         }
         for (unsigned left = __ballot_sync(FULL, on && !ok); left; left &= left - 1)
-            solve_one<T, CS>(a, lp, t0, tb + __ffs(left) - 1, j, k, xk, xf, w, false, lane);
+            solve_one<T, CS, false>(a, lp, t0, tb + __ffs(left) - 1, j, k, xk, xf, w, false, lane);
     }
     return true;
 }
@@ -1194,7 +1195,7 @@ __device__ void pairs_unit(const ScanArgs<T> &a, const LamView &lp, int t0, int 
             continue;
         }
         for (int tl = 0; tl < nlc; ++tl)
-            solve_one<T, CS>(a, lp, t0, tl, j, k, xk, xf, wc, slow_pair, lane);
+            solve_one<T, CS, !MULTI>(a, lp, t0, tl, j, k, xk, xf, wc, slow_pair, lane);
         __syncwarp();
     }
     __syncthreads();  // the CTA may stage another column next
