@@ -117,6 +117,7 @@ __global__ void __launch_bounds__(NT) k_colfeat(const T *__restrict__ Xt, int64_
     __shared__ uint32_t hist[256];
     __shared__ double red[NT / 32];
     __shared__ SelState sel;
+    next_may_start();
     const int64_t j = blockIdx.x;
     const T *x = Xt + j * ldn;
     double s1 = 0.0, s2 = 0.0;
@@ -153,7 +154,9 @@ __global__ void __launch_bounds__(NT) k_colfeat(const T *__restrict__ Xt, int64_
 // the sum reproducible), rounded to float.  Read from the column-major copy: a
 // warp's 32 rows are one line per column, and the next RN_U columns are loaded
 // while these are added.  Bound by the chain of m additions; a warp to a CTA
-// spreads the rows over the SMs.  5000 x 1000 float: 152 us from the row-major
+// spreads the rows over the SMs.  It runs beside the column features: launched
+// after them (and they after the staging had ended), it reads only the staged
+// copy and writes only rho, and waits for them when it is done.  5000 x 1000 float: 152 us from the row-major
 // matrix (one row per lane, 256 rows to a CTA), 83 us here (102 with 16 columns
 // ahead).
 template <typename T>
@@ -161,7 +164,10 @@ __global__ void __launch_bounds__(32) k_rownorm(const T *__restrict__ Xt, int64_
                                                  int64_t m, float *__restrict__ rho) {
     const int64_t i = (int64_t)blockIdx.x * 32 + threadIdx.x;
     constexpr int RN_U = sizeof(T) == 4 ? 64 : 32;
-    if (i >= n) return;
+    if (i >= n) {
+        wait_for_previous();
+        return;
+    }
     const T *x = Xt + i;
     double s = 0.0;
     T a[RN_U];
@@ -183,6 +189,7 @@ __global__ void __launch_bounds__(32) k_rownorm(const T *__restrict__ Xt, int64_
     }
     for (int64_t j = mu; j < m; ++j) s += fabs((double)x[j * ldn]);
     rho[i] = (float)fmin(s, (double)FLT_MAX);
+    wait_for_previous();
 }
 
 // Rows[r] of X (row-major n x m) into Y (row-major R x m).
@@ -757,9 +764,10 @@ template <typename T>
 cudaError_t launch_heavy_rows(const T *X, const T *Xt, int64_t ldn, int64_t n, int64_t m,
                               int64_t R, float *rho, int32_t *rows, T *Y, cudaStream_t st,
                               int &launches) {
-    k_rownorm<T><<<(unsigned)((n + 31) / 32), 32, 0, st>>>(Xt, ldn, n, m, rho);
+    // directly after launch_colfeat, which it overlaps
+    cudaError_t e = launch_after(k_rownorm<T>, dim3((unsigned)((n + 31) / 32)), dim3(32), 0, st, Xt,
+                                 ldn, n, m, rho);
     launches++;
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_topk<<<1, TK_NT, 0, st>>>(rho, n, (int)R, rows);
     launches++;
