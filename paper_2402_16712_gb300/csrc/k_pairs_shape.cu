@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(ShapeBounds<S>::threads, ShapeBounds<S>::block
         if (threadIdx.x == 0) atomicOr(a.status, ST_BADINDEX);
         return;
     }
-    pairs_unit<T, MULTI, CS>(a, lv, t0, nlc, (int)j, k0, k1, cap,
+    pairs_unit<T, MULTI, CS, sizeof(T) == 4>(a, lv, t0, nlc, (int)j, k0, k1, cap,
                              ((int)a.n + ROW_PAD - 1) & ~(ROW_PAD - 1), smem, s_dec);
 }
 
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(ShapeBounds<S>::threads, ShapeBounds<S>::block
         const BatchInst<T> &in = bd.inst[b];
         const ScanArgs<T> a = inst_args<T>(bd, b, ws);
         const LamView lv{bd.lam + bd.lam_begin[b], in.tl_min, in.tl_max};
-        pairs_unit<T, MULTI, CS>(a, lv, 0, in.nl, (int)(u - bd.unit_begin[b]), 0, in.m, cap,
+        pairs_unit<T, MULTI, CS, false>(a, lv, 0, in.nl, (int)(u - bd.unit_begin[b]), 0, in.m, cap,
                                  lay_npad, smem, s_dec);
     }
 }

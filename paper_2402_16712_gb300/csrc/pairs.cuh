@@ -948,7 +948,8 @@ __device__ __forceinline__ T pair_residual(const ScanArgs<T> &a, int64_t j, int6
 }
 
 // Writes v and s of (lambda t0+tl, jhat, k), or lists the pair for the exact path.
-// VO: the launch may ask for medians only (the kernels of one or two lambdas).
+// VO: the launch may ask for medians only (the kernels of one or two lambdas,
+// float: the question cost the double kernel 3%, 2000 x 2000 19.2 -> 19.8 ms).
 template <typename T, bool CS, bool VO>
 __device__ void emit_pair(const ScanArgs<T> &a, int t, int64_t j, int64_t k, int st,
                           typename Traits<T>::K ts, const T *xk, const T *colb, int n,
@@ -978,7 +979,9 @@ __device__ void emit_pair(const ScanArgs<T> &a, int t, int64_t j, int64_t k, int
         return;
     }
     const T v = Tr::value(ts);
-    const T res = VO && a.v_only ? T(0) : pair_residual<T, CS>(a, j, k, xk, colb, n, v, lane);
+    const T res = VO && sizeof(T) == 4 && a.v_only
+                      ? T(0)
+                      : pair_residual<T, CS>(a, j, k, xk, colb, n, v, lane);
     if (lane == 0) {
         a.v_all[o] = v;
         a.s_all[o] = (double)res + lam * (double)fabs(v);
@@ -1008,66 +1011,118 @@ __device__ void solve_one(const ScanArgs<T> &a, const LamView &lp, int t0, int t
 // between them serve every lambda.  32 lambdas are decided at a time, one per
 // lane, each against every candidate in turn; the residual is summed once per
 // value that any of them takes.  (Deciding one lambda at a time by the whole
-// warp took half of the kernel at 32 lambdas: 1000 x 500 float
-// 2.53 -> 1.39 ms; 30 x 100 x 100 double with 8 lambdas 1.09 -> 0.79 ms.)
-// Returns false (nothing written) when more than 31 rows lie between.
-template <typename T, bool CS>
+// warp took half of the kernel at 32 lambdas: 1000 x 500 float 2.53 -> 1.39 ms;
+// 30 x 100 x 100 double with 8 lambdas 1.09 -> 0.79 ms.)
+// When more than 31 rows lie between, or a bracket fails, returns false with
+// nothing written, and the caller takes the lambdas one by one.  RUNS, from
+// RUN_MIN lambdas on: they are ranked and taken in runs of neighbours instead,
+// halved until a run's rows fit; one or two left over take the full selection
+// each.  One by one left a CTA's 16 warps waiting for the one with such a pair:
+// 1000 x 500 float with 32 lambdas 1.41 -> 1.29 ms.  Only the float kernel of
+// single matrices does so: its code cost 30 x 100 x 100 double with 8 lambdas 11%.
+constexpr int RUN_MIN = 16;
+template <typename T, bool CS, bool RUNS>
 __device__ bool lambda_path(const ScanArgs<T> &a, const LamView &lp, int t0, int nlc, int64_t j,
                             int64_t k, const T *__restrict__ xk, const float *__restrict__ xf,
                             const WarpCtx<T> &w, int lane) {
     using Tr = Traits<T>;
     using K = typename Tr::K;
     const unsigned FULL = 0xFFFFFFFFu;
-    Cand32<T> f;
-    if (candidates32<T, true>(xf, xk, w, decide_for(w, lp, lp.tl_min), decide_for(w, lp, lp.tl_max),
-                              f, lane) != SEL_OK)
-        return false;
-    K fk = f.fk;
-    int64_t fq = (int64_t)f.fq;
-    warp_sort32(fk, fq, lane);
-    const int64_t P = f.L + warp_scan_add(fq, lane);
-    const K nxt = __shfl_down_sync(FULL, fk, 1);
-    // the last candidate of each key holds the weight up to it
-    const unsigned last = __ballot_sync(FULL, fk != Tr::NONE && (lane == 31 || nxt != fk));
-    const unsigned nonneg = __ballot_sync(FULL, fk >= Tr::KEY0);
-    for (int tb = 0; tb < nlc; tb += 32) {
-        const int tl = tb + lane;
-        const bool on = tl < nlc;
-        int first = -1, res = 0, below = 0;
-        {
-            const Dec32 dc = decide_for(w, lp, on ? tl : 0);
-            below = dc.cond(f.L, f.lo > CK0);
-            for (unsigned c = last; c; c &= c - 1) {
-                const int u = __ffs(c) - 1;
-                const int r = dc.cond(__shfl_sync(FULL, P, u), (nonneg >> u) & 1u);
-                if (first < 0 && r != 0) {
-                    first = u;
-                    res = r;
+    bool whole = true;             // the first attempt: all lambdas at once
+    int tb = -32, cnt = 0;         // then: the lambdas tb .. tb + cnt, one per lane,
+    int rank = 0, lo = 0, len = 0;  // this lane's place by size; the run [lo, lo + len)
+    for (;;) {
+        int t1 = lp.tl_min, t2 = lp.tl_max;
+        if (RUNS && !whole) {
+            if (lo >= cnt) {  // the next 32
+                tb += 32;
+                if (tb >= nlc) return true;
+                cnt = min(32, nlc - tb);
+                const double mine = lane < cnt ? lp.lam[tb + lane] : INFINITY;
+                rank = 0;
+                for (int u = 0; u < cnt; ++u) {
+                    const double o = __shfl_sync(FULL, mine, u);
+                    rank += o < mine || (o == mine && u < lane) ? 1 : 0;
+                }
+                if (lane >= cnt) rank = lane;
+                lo = 0;
+                len = nlc <= 32 ? (cnt + 1) / 2 : cnt;  // all of them just failed
+            }
+            len = min(len, cnt - lo);
+            t1 = tb + __ffs(__ballot_sync(FULL, rank == lo)) - 1;
+            t2 = tb + __ffs(__ballot_sync(FULL, rank == lo + len - 1)) - 1;
+        }
+        Cand32<T> f;
+        const bool few = RUNS && !whole && len < 3;
+        if (!few && candidates32<T, true>(xf, xk, w, decide_for(w, lp, t1), decide_for(w, lp, t2),
+                                          f, lane) != SEL_OK) {
+            if (!RUNS || nlc < RUN_MIN) return false;
+            if (whole)
+                whole = false;
+            else
+                len = (len + 1) / 2;
+            __syncwarp();
+            continue;
+        }
+        K fk = Tr::NONE;
+        int64_t P = 0;
+        unsigned last = 0, nonneg = 0;
+        if (!few) {
+            fk = f.fk;
+            int64_t fq = (int64_t)f.fq;
+            warp_sort32(fk, fq, lane);
+            P = f.L + warp_scan_add(fq, lane);
+            const K nxt = __shfl_down_sync(FULL, fk, 1);
+            // the last candidate of each key holds the weight up to it
+            last = __ballot_sync(FULL, fk != Tr::NONE && (lane == 31 || nxt != fk));
+            nonneg = __ballot_sync(FULL, fk >= Tr::KEY0);
+        }
+        const int ce = !RUNS || whole ? nlc : tb + 1;
+        for (int cb = !RUNS || whole ? 0 : tb; cb < ce; cb += 32) {
+            const int tl = cb + lane;
+            const bool on = tl < nlc && (!RUNS || whole || (rank >= lo && rank < lo + len));
+            bool ok = false;
+            if (!few) {
+                int first = -1, res = 0, below = 0;
+                {
+                    const Dec32 dc = decide_for(w, lp, on ? tl : 0);
+                    below = dc.cond(f.L, f.lo > CK0);
+                    for (unsigned c = last; c; c &= c - 1) {
+                        const int u = __ffs(c) - 1;
+                        const int r = dc.cond(__shfl_sync(FULL, P, u), (nonneg >> u) & 1u);
+                        if (first < 0 && r != 0) {
+                            first = u;
+                            res = r;
+                        }
+                    }
+                }
+                // else undecided here, or already passed below lo: full selection
+                ok = on && first >= 0 && res == 1 && below == 0;
+                const T v = Tr::value(__shfl_sync(FULL, fk, max(first, 0)));
+                T r = T(0);
+                for (unsigned todo = __ballot_sync(FULL, ok); todo;) {
+                    const int src = __ffs(todo) - 1;
+                    const T vs = __shfl_sync(FULL, v, src);
+                    const int u = __shfl_sync(FULL, first, src);
+                    const T rs = pair_residual<T, CS>(a, j, k, xk, w.colb, w.n, vs, lane);
+                    if (first == u) r = rs;
+                    todo &= ~__ballot_sync(FULL, first == u);
+                }
+                if (ok) {
+                    const int64_t o = L1L_CHK(((int64_t)(t0 + tl) * a.m + j) * a.m + k,
+                                              (int64_t)a.n_lambda * a.m * a.m);
+                    a.v_all[o] = v;
+                    a.s_all[o] = (double)r + lp.lam[tl] * (double)fabs(v);
                 }
             }
+            for (unsigned left = __ballot_sync(FULL, on && !ok); left; left &= left - 1)
+                solve_one<T, CS, false>(a, lp, t0, cb + __ffs(left) - 1, j, k, xk, xf, w, false,
+                                        lane);
         }
-        // undecided here, or already passed below lo: full selection
-        const bool ok = on && first >= 0 && res == 1 && below == 0;
-        const T v = Tr::value(__shfl_sync(FULL, fk, max(first, 0)));
-        T r = T(0);
-        for (unsigned todo = __ballot_sync(FULL, ok); todo;) {
-            const int src = __ffs(todo) - 1;
-            const T vs = __shfl_sync(FULL, v, src);
-            const int u = __shfl_sync(FULL, first, src);
-            const T rs = pair_residual<T, CS>(a, j, k, xk, w.colb, w.n, vs, lane);
-            if (first == u) r = rs;
-            todo &= ~__ballot_sync(FULL, first == u);
-        }
-        if (ok) {
-            const int64_t o = L1L_CHK(((int64_t)(t0 + tl) * a.m + j) * a.m + k,
-                                      (int64_t)a.n_lambda * a.m * a.m);
-            a.v_all[o] = v;
-            a.s_all[o] = (double)r + lp.lam[tl] * (double)fabs(v);
-        }
-        for (unsigned left = __ballot_sync(FULL, on && !ok); left; left &= left - 1)
-            solve_one<T, CS, false>(a, lp, t0, tb + __ffs(left) - 1, j, k, xk, xf, w, false, lane);
+        if (!RUNS || whole) return true;
+        lo += len;
+        __syncwarp();
     }
-    return true;
 }
 
 // One work unit: column jhat = j of an instance and the k in [k0, k1), all
@@ -1076,7 +1131,8 @@ __device__ bool lambda_path(const ScanArgs<T> &a, const LamView &lp, int t0, int
 // x_ijhat is staged in shared memory; otherwise the warps read it from the
 // column copy in global memory (L2-resident), which frees shared memory for
 // more resident warps when n is large.
-template <typename T, bool MULTI, bool CS>
+// RUNS: of lambda_path.
+template <typename T, bool MULTI, bool CS, bool RUNS>
 __device__ void pairs_unit(const ScanArgs<T> &a, const LamView &lp, int t0, int nlc, int j,
                            int64_t k0, int64_t k1, int cap, int lay_npad, unsigned char *smem,
                            Dec32 *s_dec) {
@@ -1190,7 +1246,7 @@ __device__ void pairs_unit(const ScanArgs<T> &a, const LamView &lp, int t0, int 
         const bool slow_pair = a.force_exact || jwide ||
                                (sizeof(T) == 8 && (a.ci[k].flags & COL_WIDE));
         if (MULTI && nlc >= 3 && !slow_pair && cinfo.n_valid > 0 &&
-            lambda_path<T, CS>(a, lp, t0, nlc, j, k, xk, xf, wc, lane)) {
+            lambda_path<T, CS, RUNS>(a, lp, t0, nlc, j, k, xk, xf, wc, lane)) {
             __syncwarp();
             continue;
         }
