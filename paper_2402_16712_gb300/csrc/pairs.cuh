@@ -948,8 +948,8 @@ __device__ __forceinline__ T pair_residual(const ScanArgs<T> &a, int64_t j, int6
 }
 
 // Writes v and s of (lambda t0+tl, jhat, k), or lists the pair for the exact path.
-// VO: the launch may ask for medians only (the kernels of one or two lambdas,
-// float: the question cost the double kernel 3%, 2000 x 2000 19.2 -> 19.8 ms).
+// VO: the launch may ask for medians only (the float kernels of one or two
+// lambdas).
 template <typename T, bool CS, bool VO>
 __device__ void emit_pair(const ScanArgs<T> &a, int t, int64_t j, int64_t k, int st,
                           typename Traits<T>::K ts, const T *xk, const T *colb, int n,
