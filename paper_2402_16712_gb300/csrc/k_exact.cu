@@ -7,6 +7,14 @@
 // a wide fixed-point integer whose unit is 2^-1074 (every finite double, and
 // so every float, is an integer multiple of it), reduced across the warp limb
 // by limb, and compared with the exact total W = sum w + lambda.
+//
+// Bound by the double divisions of its probes and the latency of one warp's
+// chain, so the listed pairs are dealt out over all SMs, CTA by CTA.  One CTA
+// of 1024 threads per SM (two do not fit): placed while the pair
+// kernel's last CTAs run, two CTAs of 128 per SM went 16 to an SM to the few SMs
+// that were free, and all pairs waited for those.  Every pair here (FORCE_EXACT),
+// double: 20,480 x 48 265 -> 61 ms, 2000 x 64 46 -> 12 ms; none here: no change
+// (200 x 20 fit 27.8 us, against 28.4 us with a launch that is not placed early).
 #include <algorithm>
 
 #include "common.cuh"
@@ -15,14 +23,16 @@
 
 namespace l1l {
 
+constexpr int EX_NT = 1024;
+
 template <typename T>
-__global__ void __launch_bounds__(128) k_exact(ScanArgs<T> a, const __grid_constant__ LambdaPack lp,
-                                               int t0) {
+__global__ void __launch_bounds__(EX_NT) k_exact(ScanArgs<T> a,
+                                                 const __grid_constant__ LambdaPack lp, int t0) {
     next_may_start();
     wait_for_previous();
     const int lane = threadIdx.x & 31;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    const uint32_t gw = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    const uint32_t nwarps = gridDim.x * (EX_NT / 32);
     const uint32_t count = *(volatile uint32_t *)a.slow_count;
     uint32_t acc[WL];
     uint32_t S[WL], W[WL];  // used by lane 0
@@ -39,7 +49,7 @@ cudaError_t launch_exact(const ScanArgs<T> &a, const double *lambdas, int t0, in
     lp.tl_min = lp.tl_max = 0;
     for (int q = 0; q < nlc; ++q) lp.lam[q] = lambdas[t0 + q];
     launches++;
-    return launch_after(k_exact<T>, dim3(num_sms * 2), dim3(128), 0, st, a, lp, t0);
+    return launch_after(k_exact<T>, dim3(num_sms), dim3(EX_NT), 0, st, a, lp, t0);
 }
 
 template cudaError_t launch_exact<float>(const ScanArgs<float> &, const double *, int, int, int,
