@@ -226,8 +226,8 @@ int scan_setup(const T *X, int64_t n, int64_t m, const double *lambdas, int64_t 
 template <typename T> int scan_prep(const T *X, Scan<T> &c) {
     L1L_RANGE("l1l::stage");
     ScanArgs<T> &a = c.a;
-    // status and slow_count are the first two 256-byte slots
-    if (cudaMemsetAsync(a.status, 0, c.L.slow_count + sizeof(uint32_t), c.st) != cudaSuccess)
+    // status and slow_count (two words) are the first two 256-byte slots
+    if (cudaMemsetAsync(a.status, 0, c.L.slow_count + 2 * sizeof(uint32_t), c.st) != cudaSuccess)
         return L1L_ERR_CUDA;
     c.counter_zero = true;
     if (launch_prep<T>(X, const_cast<T *>(a.Xt), const_cast<float *>(a.Xf),
@@ -249,7 +249,7 @@ int scan_pairs_large(Scan<T> &c, const double *lambdas, int64_t nl, const int32_
         const int nlc = (int)((nl - t0) < MAX_LAMBDA_PER_LAUNCH ? (nl - t0) : MAX_LAMBDA_PER_LAUNCH);
         const bool last = t0 + MAX_LAMBDA_PER_LAUNCH >= nl;
         if (!c.counter_zero &&
-            cudaMemsetAsync(a.slow_count, 0, sizeof(uint32_t), c.st) != cudaSuccess)
+            cudaMemsetAsync(a.slow_count, 0, 2 * sizeof(uint32_t), c.st) != cudaSuccess)
             return L1L_ERR_CUDA;
         c.counter_zero = false;
         if (prof && t0 == 0 && cudaEventRecord(g_ev_start, c.st) != cudaSuccess)
@@ -282,7 +282,7 @@ int scan_pairs(Scan<T> &c, const double *lambdas, int64_t nl, const int32_t *jli
         const int nlc = (int)((nl - t0) < MAX_LAMBDA_PER_LAUNCH ? (nl - t0) : MAX_LAMBDA_PER_LAUNCH);
         const bool last = t0 + MAX_LAMBDA_PER_LAUNCH >= nl;
         if (!c.counter_zero &&
-            cudaMemsetAsync(a.slow_count, 0, sizeof(uint32_t), c.st) != cudaSuccess)
+            cudaMemsetAsync(a.slow_count, 0, 2 * sizeof(uint32_t), c.st) != cudaSuccess)
             return L1L_ERR_CUDA;
         c.counter_zero = false;
         if (prof && t0 == 0 && cudaEventRecord(g_ev_start, c.st) != cudaSuccess)

@@ -245,7 +245,7 @@ template <typename T> struct ScanArgs {
     T *v_all;          // [n_lambda][m][m]
     double *s_all;     // [n_lambda][m][m]
     uint32_t *status;  // workspace status word
-    uint32_t *slow_count;
+    uint32_t *slow_count;  // entries of slow; then whether any lambda batch was put off
     SlowEntry *slow;   // capacity n_lambda * m * m
     int force_exact;
     int inst;          // instance index recorded in slow-list entries (batched calls)

@@ -41,12 +41,15 @@ __global__ void __launch_bounds__(256) k_colprep_b(const __grid_constant__ Batch
     colprep_column<T>(Xt + (int64_t)j * in.ldn, ci + j, in.n);
 }
 
+// As k_exact.
+constexpr int EXB_NT = 1024;
 template <typename T>
-__global__ void __launch_bounds__(128) k_exact_b(const __grid_constant__ BatchDesc<T> bd,
-                                                 unsigned char *ws) {
+__global__ void __launch_bounds__(EXB_NT) k_exact_b(const __grid_constant__ BatchDesc<T> bd,
+                                                    unsigned char *ws) {
     const int lane = threadIdx.x & 31;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    const uint32_t gw = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    const uint32_t nwarps = gridDim.x * (EXB_NT / 32);
+    __shared__ __align__(16) uint32_t hist[EXB_NT / 32][HIST_WORDS];
     const uint32_t count = *(volatile uint32_t *)(ws + 256);
     const SlowEntry *slow = reinterpret_cast<const SlowEntry *>(ws + BATCH_HEAD);
     uint32_t acc[WL];
@@ -54,7 +57,8 @@ __global__ void __launch_bounds__(128) k_exact_b(const __grid_constant__ BatchDe
     for (uint32_t e = gw; e < count; e += nwarps) {
         const SlowEntry en = slow[e];
         const ScanArgs<T> a = inst_args<T>(bd, en.inst, ws);
-        exact_entry<T>(a, en, bd.lam[bd.lam_begin[en.inst] + en.t], acc, S, W, lane);
+        listed_entry<T>(a, en, 0, bd.lam + bd.lam_begin[en.inst], a.n_lambda,
+                        hist[threadIdx.x >> 5], acc, S, W, lane);
     }
 }
 
@@ -132,15 +136,14 @@ cudaError_t launch_batch(const BatchDesc<T> &bd, unsigned char *ws, T *out_v, do
         const BatchClass &bc = classes[c];
         if (bc.u1 <= bc.u0) continue;
         switch (bc.plan.shape) {
-            case SHAPE_R80: e = launch_persist_sh<T, SHAPE_R80>(bd, ws, bc, c, multi, num_sms, st); break;
-            case SHAPE_R64: e = launch_persist_sh<T, SHAPE_R64>(bd, ws, bc, c, multi, num_sms, st); break;
-            case SHAPE_R128: e = launch_persist_sh<T, SHAPE_R128>(bd, ws, bc, c, multi, num_sms, st); break;
+            case SHAPE_R80: e = launch_persist_sh<T, SHAPE_R80>(bd, ws, bc, c, multi, num_sms, st, launches); break;
+            case SHAPE_R64: e = launch_persist_sh<T, SHAPE_R64>(bd, ws, bc, c, multi, num_sms, st, launches); break;
+            case SHAPE_R128: e = launch_persist_sh<T, SHAPE_R128>(bd, ws, bc, c, multi, num_sms, st, launches); break;
             default: e = cudaErrorInvalidConfiguration;
         }
         if (e != cudaSuccess) return e;
-        launches++;
     }
-    k_exact_b<T><<<num_sms * 2, 128, 0, st>>>(bd, ws);
+    k_exact_b<T><<<num_sms, EXB_NT, 0, st>>>(bd, ws);
     k_zreduce_b<T><<<bd.ztasks, 32, 0, st>>>(bd, ws);
     k_argmin_b<T><<<bd.lams, 256, 0, st>>>(bd, ws, out_v, out_obj, out_jstar);
     launches += 3;

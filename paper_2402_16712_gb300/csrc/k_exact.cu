@@ -23,22 +23,25 @@
 
 namespace l1l {
 
-constexpr int EX_NT = 1024;
+constexpr int EX_NT = 1024;  // threads per CTA at most
 
 template <typename T>
 __global__ void __launch_bounds__(EX_NT) k_exact(ScanArgs<T> a,
-                                                 const __grid_constant__ LambdaPack lp, int t0) {
+                                                 const __grid_constant__ LambdaPack lp, int t0,
+                                                 int nlc) {
     next_may_start();
     wait_for_previous();
     const int lane = threadIdx.x & 31;
     const uint32_t gw = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-    const uint32_t nwarps = gridDim.x * (EX_NT / 32);
+    const uint32_t nwarps = gridDim.x * (blockDim.x >> 5);
     const uint32_t count = *(volatile uint32_t *)a.slow_count;
+    extern __shared__ __align__(16) uint32_t hist[];  // HIST_WORDS per warp
     uint32_t acc[WL];
     uint32_t S[WL], W[WL];  // used by lane 0
     for (uint32_t e = gw; e < count; e += nwarps) {
         const SlowEntry en = a.slow[e];
-        exact_entry<T>(a, en, lp.lam[en.t - t0], acc, S, W, lane);
+        listed_entry<T>(a, en, t0, lp.lam, nlc, hist + (threadIdx.x >> 5) * HIST_WORDS, acc, S, W,
+                        lane);
     }
 }
 
@@ -48,8 +51,14 @@ cudaError_t launch_exact(const ScanArgs<T> &a, const double *lambdas, int t0, in
     LambdaPack lp;
     lp.tl_min = lp.tl_max = 0;
     for (int q = 0; q < nlc; ++q) lp.lam[q] = lambdas[t0 + q];
+    // few pairs: four warps to a CTA, as full ones lengthen an empty launch (200 x 20 fit
+    // 27.7 us, 28.5 with them); sizes between, of which two or more go to an SM, would
+    // bring the crowding back (20,480 x 48, 16 warps: 111 ms)
+    const int w = a.nj * a.m * nlc <= 4 * (int64_t)num_sms ? 4 : EX_NT / 32;
+    const size_t smem = (size_t)w * HIST_WORDS * 4;
+    static_assert(EX_NT / 32 * HIST_WORDS * 4 <= 48 * 1024, "needs no opt-in");
     launches++;
-    return launch_after(k_exact<T>, dim3(num_sms), dim3(EX_NT), 0, st, a, lp, t0);
+    return launch_after(k_exact<T>, dim3(num_sms), dim3((unsigned)w * 32), smem, st, a, lp, t0, nlc);
 }
 
 template cudaError_t launch_exact<float>(const ScanArgs<float> &, const double *, int, int, int,

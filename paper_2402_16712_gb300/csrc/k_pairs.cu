@@ -59,9 +59,9 @@ cudaError_t blocks_per_sm(const void *fn, int threads, size_t smem, int *out) {
     return cudaSuccess;
 }
 
-// Candidate slots of the 64-bit selection's list that hold its first bracket
-// at any width, 40% of the rows and at least 512 (or every row), and the bytes
-// such a list takes per warp beside its histogram.
+// The room that the limit on n and a caller's own d0 leave per warp beside its
+// histogram: that of a candidate list of 40% of the rows, at least 512 (or every row).
+// The selection keeps no list; limit and tuned launch shapes stay what they were.
 static int64_t list_slots(int64_t npad) {
     const int64_t c = std::max<int64_t>(512, (npad * 2 / 5 + 31) & ~int64_t(31));
     return std::min<int64_t>(npad, c) & ~int64_t(31);
@@ -100,12 +100,10 @@ template <typename T>
 static PairPlan plan_placement(int64_t npad, bool cs, int d0, const Tune &tune) {
     PairPlan p{0, 0, 0, 0, 0, 0, 0, 0, 0};
     const size_t cb = PairSmem<T>::col_bytes(npad, cs);
-    // Slots of the 64-bit selection's list.  That selection is the rare
-    // fallback, and with a short list it narrows its bracket by a counting
-    // pass first, so 128 slots leave the room to more resident warps and to
-    // L1.  A caller's own d0 gets a list that holds a bracket of that width:
-    // ~2.5% of the rows per sample position, i.e. mu = 0.025 d0 n/32 per lane,
-    // and mu + 3.5 sqrt(mu) + 1 for the busiest of 32 lanes.
+    // Slots of six bytes left free per warp: 128, or for a caller's own d0 as many
+    // as a list of its bracket took (~2.5% of the rows per sample position, i.e. mu
+    // = 0.025 d0 n/32 per lane, and mu + 3.5 sqrt(mu) + 1 for the busiest of 32
+    // lanes).
     const double mu = 0.025 * (double)d0 * (double)npad / 32.0;
     const int64_t qt_need = std::min<int64_t>(npad / 32, (int64_t)ceil(mu + 3.5 * sqrt(mu) + 1.0));
     const int64_t slots = std::min<int64_t>(npad, 128);
@@ -233,12 +231,11 @@ cudaError_t launch_pairs(const ScanArgs<T> &a, const double *lambdas, int t0, in
     }
     cudaError_t e;
     switch (plan.shape) {
-        case SHAPE_R80: e = launch_pairs_sh<T, SHAPE_R80>(a, lp, t0, nlc, plan, st); break;
-        case SHAPE_R64: e = launch_pairs_sh<T, SHAPE_R64>(a, lp, t0, nlc, plan, st); break;
-        case SHAPE_R128: e = launch_pairs_sh<T, SHAPE_R128>(a, lp, t0, nlc, plan, st); break;
+        case SHAPE_R80: e = launch_pairs_sh<T, SHAPE_R80>(a, lp, t0, nlc, plan, st, launches); break;
+        case SHAPE_R64: e = launch_pairs_sh<T, SHAPE_R64>(a, lp, t0, nlc, plan, st, launches); break;
+        case SHAPE_R128: e = launch_pairs_sh<T, SHAPE_R128>(a, lp, t0, nlc, plan, st, launches); break;
         default: e = cudaErrorInvalidConfiguration;
     }
-    launches++;
     return e;
 }
 

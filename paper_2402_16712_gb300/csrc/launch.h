@@ -62,7 +62,7 @@ struct PairPlan {
     size_t smem;
     int kchunk;
     int kchunks;
-    int cap;    // per-warp candidate-list capacity
+    int cap;    // slots left free per warp (k_pairs.cu)
     int ctas;   // CTAs per SM the shared memory is sized for
     int d0;     // first-bracket half-width of the selection
     int cs;     // 1: x_ijhat staged in shared memory; 0: read from global memory
@@ -88,7 +88,7 @@ cudaError_t launch_pairs(const ScanArgs<T> &a, const double *lambdas, int t0, in
 // The same for one shape S == plan.shape (k_pairs_shape.cu).
 template <typename T, int S>
 cudaError_t launch_pairs_sh(const ScanArgs<T> &a, const LambdaPack &lp, int t0, int nlc,
-                            const PairPlan &plan, cudaStream_t st);
+                            const PairPlan &plan, cudaStream_t st, int &launches);
 
 // Largest n of any scan or fit: the global-memory path's limit (row counts
 // and the exact path's row loop are 32-bit).
@@ -203,7 +203,8 @@ constexpr int MAX_BATCH_CLASSES = 3;
 // class's counter `slot`.
 template <typename T, int S>
 cudaError_t launch_persist_sh(const BatchDesc<T> &bd, unsigned char *ws, const BatchClass &bc,
-                              int slot, bool multi, int num_sms, cudaStream_t st);
+                              int slot, bool multi, int num_sms, cudaStream_t st,
+                              int &launches);
 
 // The batched fit: staging, one persistent pair kernel per size class, exact
 // path, sums, argmin.

@@ -17,21 +17,19 @@
 // arithmetic (the test of Lemma 1).
 //
 // The selection proper is in select32.cuh (32-bit weights, two passes over
-// the rows).  The 64-bit selection below is its fallback, for what the 32-bit
-// weights cannot settle: sampled pivots, a pass that compacts the rows between
-// them into a candidate list (or, when the list is too short, histograms all
-// rows), an exact 64-bin weight histogram of the list, narrowed to <= 31
-// candidates.  Then the residual sum_i |x_ik - v x_ijhat| over all rows
-// (Algorithm 1, objective).
+// the rows).  What it cannot settle -- a decision inside the certainty band of the
+// 32-bit weights, or more rows around the median than a warp's lanes -- is listed
+// for the kernel behind (exact.cuh), which first looks at the coarse keys that the
+// selection has left with 64-bit weights (narrow.cuh).  Then the residual sum_i
+// |x_ik - v x_ijhat| over all rows (Algorithm 1, objective).
 //
-// A decision the truncated fixed-point weights cannot settle, a column whose
-// magnitudes fall outside the approximation's range, or a candidate list that
-// cannot be narrowed sends the pair to the exact wide-accumulator kernel.
+// Also listed, for the exact wide-accumulator search: a column whose magnitudes fall
+// outside the approximation's range, and a decision that the 64-bit fixed-point
+// weights, truncated too, cannot settle.
 #pragma once
 #include <algorithm>
 #include <cmath>
 
-#include "binmap.cuh"
 #include "checks.cuh"
 #include "common.cuh"
 
@@ -66,7 +64,7 @@ template <> struct Approx<double> {
 };
 
 constexpr int NSAMP = 64;   // weight-proportional sample rows per column
-constexpr int HIST_WORDS = 4 * 64;  // per-warp exact histogram (4 chunks x 64 bins)
+constexpr int HIST_WORDS = 256;  // per-warp histogram
 
 template <typename T> struct PairSmem {
     // per CTA: x_ijhat (T; only when `cs`, else it is read from the column
@@ -76,16 +74,14 @@ template <typename T> struct PairSmem {
         return (cs ? al16(npad * sizeof(T)) : 0) + al16(npad * 4) + al16(npad * 4) +
                al16(NSAMP * 2);
     }
-    // per warp: the histogram (256 words, of either selection), then the
-    // 64-bit selection's candidate keys (uint32) and row indices (uint16; bit
-    // 15 = exact key)
+    // per warp: the histogram, and room that the planner's shapes were measured with
+    // (six bytes for each of `cap` slots; nothing is kept there)
     __host__ __device__ static size_t warp_bytes(int64_t cap) {
         return al16(HIST_WORDS * 4) + al16(cap * 4) + al16(cap * 2);
     }
 };
 
-constexpr uint16_t EXACT_BIT = 0x8000u;
-constexpr uint32_t CKMAX = 0xFFFFFFFEu;    // largest usable coarse key
+constexpr uint32_t CK0 = 0x80000000u;      // coarse key of 0
 constexpr uint32_t CKNONE = 0xFFFFFFFFu;
 
 // ---------------------------------------------------------------------------
@@ -105,30 +101,6 @@ __device__ __forceinline__ void warp_sort32(K &key, W &w, int lane) {
             if (take) {
                 key = ok;
                 w = ow;
-            }
-        }
-    }
-}
-
-// 64 keys, element g = e*32 + lane held in slot e; ascending in g.
-__device__ __forceinline__ void warp_sort64(uint32_t (&k)[2], int lane) {
-#pragma unroll
-    for (int size = 2; size <= 64; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            if (stride == 32) {  // only in the final merge: ascending
-                const uint32_t lo = min(k[0], k[1]), hi = max(k[0], k[1]);
-                k[0] = lo;
-                k[1] = hi;
-            } else {
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const uint32_t ok = __shfl_xor_sync(0xFFFFFFFFu, k[e], stride);
-                    const int g = e * 32 + lane;
-                    const bool up = (g & size) == 0;
-                    const bool lower = (lane & stride) == 0;
-                    k[e] = (lower == up) ? min(ok, k[e]) : max(ok, k[e]);
-                }
             }
         }
     }
@@ -199,17 +171,17 @@ __device__ __forceinline__ T warp_residual_pad(const T *__restrict__ xk, const T
     return s;
 }
 
-// Outcomes of select_v2.  Every code >= SEL_SLOW hands the pair to the exact
-// path; the code says why (kept in the slow list for diagnostics).
+// Outcomes of a selection.  Every code >= SEL_SLOW hands the pair to the kernel
+// behind; the code says why (kept in the slow list).
 enum {
     SEL_OK = 0,
     SEL_INTERNAL = 1,
-    SEL_SLOW = 2,        // column outside the approximate-key range / forced
-    SEL_SLOW_TRIES,      // level 0 kept missing the median
-    SEL_SLOW_CAP,        // too many rows between the closest pivots
-    SEL_SLOW_BAND,       // truncated weights cannot settle a decision
-    SEL_SLOW_LEVELS,     // candidate list did not shrink
-    SEL_SLOW_TIE         // double: one coarse key holds distinct exact keys
+    SEL_SLOW = 2,    // column outside the approximate-key range / forced
+    SEL_SLOW_BAND,   // truncated weights cannot settle a decision
+    SEL_W64 = 16,    // not settled on 32-bit weights
+    SEL_MANY,        // rows too close together for the bins (listed: of a batch of lambdas)
+    SEL_BELOW,       // narrow(): the median lies below the range looked at, above it
+    SEL_ABOVE
 };
 
 __device__ __forceinline__ uint32_t sat_sub(uint32_t a, uint32_t b) { return a > b ? a - b : 0u; }
@@ -217,108 +189,7 @@ __device__ __forceinline__ uint32_t sat_add(uint32_t a, uint32_t b) {
     return a < CKNONE - b ? a + b : CKNONE;
 }
 
-// Estimated index (0..ns-1) of the first sorted sample whose scaled cumulative
-// weight passes the crossing target; targets are relative to L.
-// Pivot estimates are float: they only steer the search (every decision that
-// matters is exact, in int64), and this GPU's double pipe is narrow.
-__device__ __forceinline__ float target_for(uint32_t key, float hneg, float hpos) {
-    return key >= CK0 ? hpos : hneg;
-}
-
-// ---------------------------------------------------------------------------
-// Exact weight histogram: XB bins, each an int64 sum kept as four 16-bit
-// chunks in 32-bit shared-memory counters (exact for up to 65,535 rows per
-// bin; 64-bit shared atomics are several times slower on this GPU).
-// ---------------------------------------------------------------------------
-constexpr int XB = 64;
 constexpr uint16_t ROW_MASK = 0x7FFFu;
-
-__device__ __forceinline__ void hist_zero(uint32_t *h, int lane) {
-#pragma unroll
-    for (int q = 0; q < (4 * XB) / 32; ++q) h[q * 32 + lane] = 0u;
-}
-__device__ __forceinline__ void hist_add(uint32_t *h, int bin, int64_t q) {
-    bin = L1L_CHK(bin, XB);
-    const uint64_t u = (uint64_t)q;
-    atomicAdd(&h[bin], (uint32_t)(u & 0xFFFFu));
-    atomicAdd(&h[XB + bin], (uint32_t)((u >> 16) & 0xFFFFu));
-    atomicAdd(&h[2 * XB + bin], (uint32_t)((u >> 32) & 0xFFFFu));
-    atomicAdd(&h[3 * XB + bin], (uint32_t)(u >> 48));
-}
-__device__ __forceinline__ int64_t hist_get(const uint32_t *h, int bin) {
-    return (int64_t)h[bin] + ((int64_t)h[XB + bin] << 16) + ((int64_t)h[2 * XB + bin] << 32) +
-           ((int64_t)h[3 * XB + bin] << 48);
-}
-
-// Among bins 0..nbins-1 of [base, top] (bin b = keys base + [b, b+1) << sh),
-// find the first whose upper key passes the exact test with S = Sbase + weight
-// of bins <= b.  Returns the bin (-1: none passes, -2: undecidable) and the
-// weight below it in *below.
-__device__ __forceinline__ int hist_cross(const uint32_t *h, int nbins, uint32_t base,
-                                          uint32_t top, int sh, int64_t Sbase,
-                                          const Decide &dc, int64_t *below, int lane) {
-    const unsigned FULL = 0xFFFFFFFFu;
-    const int b0 = 2 * lane, b1 = 2 * lane + 1;
-    const int64_t s0 = b0 < nbins ? hist_get(h, b0) : 0;
-    const int64_t s1 = b1 < nbins ? hist_get(h, b1) : 0;
-    const int64_t incl = warp_scan_add(s0 + s1, lane);
-    const int64_t ex = incl - s0 - s1;
-    auto bhi = [&](int b) -> uint32_t {
-        const uint64_t v = (uint64_t)base + ((uint64_t)(b + 1) << sh) - 1;
-        return v > top ? top : (uint32_t)v;
-    };
-    const int c0 = b0 < nbins ? dc.cond(Sbase + ex + s0, bhi(b0) >= CK0) : 0;
-    const int c1 = b1 < nbins ? dc.cond(Sbase + ex + s0 + s1, bhi(b1) >= CK0) : 0;
-    const unsigned m0 = __ballot_sync(FULL, c0 != 0), m1 = __ballot_sync(FULL, c1 != 0);
-    const unsigned any = m0 | m1;
-    if (!any) return -1;
-    const int ln = __ffs(any) - 1;
-    const bool first_is_b0 = (m0 >> ln) & 1u;
-    const int bsel = 2 * ln + (first_is_b0 ? 0 : 1);
-    const int csel = __shfl_sync(FULL, first_is_b0 ? c0 : c1, ln);
-    const int64_t bel = __shfl_sync(FULL, first_is_b0 ? ex : ex + s0, ln);
-    if (csel < 0) return -2;
-    *below = Sbase + bel;
-    return bsel;
-}
-
-// hist_cross over the bins of a BinMap (at most XB of them).
-__device__ __forceinline__ int hist_cross_map(const uint32_t *h, const BinMap &bm, int64_t Sbase,
-                                              const Decide &dc, int64_t *below, int lane) {
-    const unsigned FULL = 0xFFFFFFFFu;
-    const int nbins = bm.nbins();
-    const int b0 = 2 * lane, b1 = 2 * lane + 1;
-    const int64_t s0 = b0 < nbins ? hist_get(h, b0) : 0;
-    const int64_t s1 = b1 < nbins ? hist_get(h, b1) : 0;
-    const int64_t incl = warp_scan_add(s0 + s1, lane);
-    const int64_t ex = incl - s0 - s1;
-    const int c0 = b0 < nbins ? dc.cond(Sbase + ex + s0, bm.upper(b0) >= CK0) : 0;
-    const int c1 = b1 < nbins ? dc.cond(Sbase + ex + s0 + s1, bm.upper(b1) >= CK0) : 0;
-    const unsigned m0 = __ballot_sync(FULL, c0 != 0), m1 = __ballot_sync(FULL, c1 != 0);
-    const unsigned any = m0 | m1;
-    if (!any) return -1;
-    const int ln = __ffs(any) - 1;
-    const bool first_is_b0 = (m0 >> ln) & 1u;
-    const int bsel = 2 * ln + (first_is_b0 ? 0 : 1);
-    const int csel = __shfl_sync(FULL, first_is_b0 ? c0 : c1, ln);
-    const int64_t bel = __shfl_sync(FULL, first_is_b0 ? ex : ex + s0, ln);
-    if (csel < 0) return -2;
-    *below = Sbase + bel;
-    return bsel;
-}
-
-// The 64-bit fixed-point weight q_i of row i for the 64-bit selection,
-// computed from x_ijhat on the spot (the fast path stages 32-bit weights;
-// the 64-bit selection is its rare fallback).
-template <typename T> struct WqFly {
-    const T *colb;
-    int sigma;
-    __device__ __forceinline__ int64_t operator()(int i) const {
-        const T b = colb[i];
-        int e = 0;
-        return b != T(0) ? fixq(b < T(0) ? -b : b, sigma, e) : 0;
-    }
-};
 
 // The exact test on the 32-bit weights, with its thresholds as whole weights:
 // S passes at a negative ratio when S >= tneg, at a ratio >= 0 when S >= tpos
@@ -345,25 +216,43 @@ struct LamView {
     int tl_min, tl_max;  // positions of the smallest and largest lambda
 };
 
-// Everything one warp needs to solve the pairs of its CTA's column jhat.
+// What one warp needs to solve the pairs of its CTA's column jhat.
 // The fast path's weights are the 32-bit q32 (both input types); s_dec and
 // decide_for use the same scale.
 template <typename T> struct WarpCtx {
     const T *colb;
     const float *inv;
     const uint32_t *q32;
-    const uint16_t *samp;
-    uint32_t *hist;        // histogram of either selection
-    uint32_t *lk;          // 64-bit fallback's lists
-    uint16_t *li;
+    uint32_t *hist;       // the warp's histogram
     const Dec32 *s_dec;   // per-lambda thresholds for the first NDEC lambdas
-    int qt, n;
+    const ColInfo *ci;    // of column jhat
+    int n;
     int d0;               // first-bracket half-width in sample positions
     int srow;             // this lane's sample row and its 1/x_ijhat
     float sinv;
-    ColInfo cinfo;
 };
 constexpr int NDEC = 32;
+
+// The place in s_all, whose values are never negative, of a pair that the selection
+// has not settled: the sign bit, whether the median lies in the range that follows, among
+// few rows or many (or those of a whole batch do), and that range of coarse keys, rounded
+// outward to 2 and 4 keys to fit.
+enum : int { OFF_NONE = 0, OFF_RANGE, OFF_MANY, OFF_BATCH };
+__device__ __forceinline__ int64_t off_mark(int why, uint32_t lo, uint32_t hi) {
+    uint64_t range = (uint64_t)(lo >> 1) << 30 | min((hi >> 2) + 1u, (1u << 30) - 1u);
+    if (lo > hi) {  // not known
+        range = 0;
+        if (why != OFF_BATCH) why = OFF_NONE;
+    }
+    return (int64_t)(1ull << 63 | (uint64_t)why << 61 | range);
+}
+__device__ __forceinline__ int off_why(int64_t mark) { return (int)((uint64_t)mark >> 61) & 3; }
+// Whether it holds a range.
+__device__ __forceinline__ bool off_range(int64_t mark, uint32_t &lo, uint32_t &hi) {
+    lo = (uint32_t)((uint64_t)mark >> 30 & 0x7FFFFFFFu) << 1;
+    hi = ((uint32_t)mark & 0x3FFFFFFFu) << 2;
+    return hi != 0;
+}
 
 // The coarse key of an exact key.
 template <typename T>
@@ -377,399 +266,9 @@ __device__ __forceinline__ uint32_t coarse_of(typename Traits<T>::K k) {
 }  // namespace l1l
 
 #include "select32.cuh"
+#include "narrow.cuh"
 
 namespace l1l {
-
-// ---------------------------------------------------------------------------
-// Weighted median of one pair.  Returns SEL_* and the exact key in tstar.
-//
-// The candidate list is kept as 32 interleaved per-lane segments: lane l's
-// j-th candidate sits at slot j*32 + l (bank l, so every access is free of bank
-// conflicts) and each lane counts its own candidates against a quota of
-// qt = cap/32 slots; only the final <= 31 candidates are gathered across the
-// warp.  Row indices carry a flag bit, EXACT: the stored key is exact.  The
-// candidate arrays, the histogram and the column arrays never overlap (hence
-// __restrict__), so the loops over the list below, unrolled by two, can issue
-// the shared-memory loads of one candidate before the atomics of the other.
-// ---------------------------------------------------------------------------
-template <typename T, typename WQ>
-__device__ int select_v2(const T *__restrict__ xk, const float *__restrict__ xf,
-                         const T *__restrict__ colb, const float *__restrict__ inv,
-                         const WQ colq, const uint16_t *__restrict__ samp,
-                         uint32_t *__restrict__ lk, uint16_t *__restrict__ li,
-                         uint32_t *__restrict__ hist, int qt, int n, int d0, const Decide &dc,
-                         typename Traits<T>::K &tstar, int lane) {
-    using Tr = Traits<T>;
-    using K = typename Tr::K;
-    using A = Approx<T>;
-    constexpr uint32_t G = A::G;
-    const unsigned FULL = 0xFFFFFFFFu;
-    const float Qf = (float)dc.Q;
-    const float hneg0 = 0.5f * (Qf + (float)dc.Lf), hpos0 = 0.5f * (Qf - (float)dc.Lc);
-    const int nrow = (n + ROW_PAD - 1) & ~(ROW_PAD - 1);  // rows the columns hold
-    const int nslot = qt * 32;                             // candidate slots
-    (void)nrow;
-    (void)nslot;
-
-    // ---------------- level 0 -------------------------------------------
-    // 64 rows drawn in proportion to their weight (each stands for Q/64), so the
-    // sorted sample keys estimate the weighted quantiles directly.
-    uint32_t sk[2];
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-        const int i = L1L_CHK((int)samp[e * 32 + lane], nrow);
-        sk[e] = akey(__fmul_rn(xf[i], inv[i]));
-    }
-    warp_sort64(sk, lane);
-    int jx;
-    {
-        const float unit = Qf * (1.0f / 64.0f);
-        const bool c0 = (float)(lane + 1) * unit > target_for(sk[0], hneg0, hpos0);
-        const bool c1 = (float)(lane + 33) * unit > target_for(sk[1], hneg0, hpos0);
-        const unsigned m0 = __ballot_sync(FULL, c0), m1 = __ballot_sync(FULL, c1);
-        jx = m0 ? __ffs(m0) - 1 : (m1 ? 32 + __ffs(m1) - 1 : 63);
-    }
-    auto sample_key = [&](int g) -> uint32_t {
-        const uint32_t a0 = __shfl_sync(FULL, sk[0], g & 31);
-        const uint32_t a1 = __shfl_sync(FULL, sk[1], g & 31);
-        return g < 32 ? a0 : a1;
-    };
-    // the median's coarse key is known to lie in [lo0, hi0]; pivots stay inside
-    uint32_t lo0 = 0, hi0 = CKMAX;
-    auto pick = [&](int g, uint32_t dflt) -> uint32_t {
-        uint32_t kk = (g < 0 || g > 63) ? dflt : sample_key(g);
-        if (kk > CKMAX) kk = dflt;
-        return min(max(kk, lo0), hi0);
-    };
-    // d0: half-width of the first bracket in sample positions (6 of 64: ~15%
-    // of the rows in the bracket, ~1.5% misses)
-    // pivots 2G + 1 keys outside the sample keys, so that the sample rows (and
-    // rows tied with them) lie clear of the guard bands
-    uint32_t P1 = pick(jx - d0, lo0);
-    uint32_t P2 = pick(jx + d0, hi0);
-    P1 = max(sat_sub(P1, 2 * G + 1), lo0);
-    P2 = min(sat_add(P2, 2 * G + 1), hi0);
-    if (P1 > P2) P1 = P2;
-    bool sampled = true;     // the bracket still comes from the sample
-    // next attempt: narrow by a histogram over all rows (at once when the list
-    // is too short for a sample bracket)
-    bool count_pass = qt * 128 < n;
-
-    int64_t L = 0;   // exact weight of rows with coarse key < lo
-    uint32_t lo = 0, hi = CKMAX;
-    int cnt = 0;     // this lane's candidates
-    bool placed = false;
-    for (int attempt = 0; attempt < 12 && !placed; ++attempt) {
-        if (count_pass) {
-            // One pass over all rows straight into the exact histogram of
-            // [P1, P2] (rows near a bin edge are divided on the spot); nothing
-            // is stored, so it cannot overflow.  The median's bin becomes the
-            // next bracket, 1/64 of this one.
-            const uint32_t span = P2 - P1;
-            const int sh = span >= (uint32_t)XB ? (32 - __clz((int)span)) - 6 : 0;
-            const uint32_t bmask = (1u << sh) - 1u;
-            const int nbins = (int)(span >> sh) + 1;
-            const uint32_t bt = sat_sub(P1, G), at = min(sat_add(P2, G), CKMAX);
-            const uint32_t g1 = sat_add(P1, G), g2 = sat_sub(P2, G);
-            hist_zero(hist, lane);
-            __syncwarp();
-            int64_t Sb = 0;
-            for (int i = lane; i < n; i += 32) {
-                const float iv = inv[i];
-                if (isnan(iv)) continue;  // x_ijhat = 0 or a padding row
-                uint32_t kk = akey(__fmul_rn(xf[i], iv));
-                if (kk < bt) {
-                    Sb += colq(i);
-                    continue;
-                }
-                if (kk > at) continue;
-                const uint32_t off = (kk - P1) & bmask;
-                if (!(kk >= g1 && kk <= g2 && off >= G && off + G <= bmask))
-                    kk = A::exact_ck(xk[i], colb[i]);
-                if (kk < P1)
-                    Sb += colq(i);
-                else if (kk <= P2)
-                    hist_add(hist, (int)((kk - P1) >> sh), colq(i));
-            }
-            Sb = warp_sum_i64(Sb);
-            __syncwarp();
-            const int r1 = P1 == lo0 ? 0 : dc.cond(Sb, (P1 - 1) >= CK0);
-            if (r1 < 0) return SEL_SLOW_BAND;
-            if (r1 == 1) {
-                hi0 = P1 - 1;
-                P1 = lo0;
-                P2 = hi0;
-                continue;
-            }
-            int64_t below = 0;
-            const int bs = hist_cross(hist, nbins, P1, P2, sh, Sb, dc, &below, lane);
-            __syncwarp();
-            if (bs == -2) return SEL_SLOW_BAND;
-            if (bs < 0) {
-                if (P2 >= hi0) return SEL_INTERNAL;
-                lo0 = P2 + 1;
-                P1 = lo0;
-                P2 = hi0;
-                continue;
-            }
-            const uint32_t K1 = P1 + ((uint32_t)bs << sh);
-            const uint32_t K2 = min(P2, K1 + bmask);
-            lo0 = K1;
-            hi0 = K2;
-            P1 = K1;
-            P2 = K2;
-            sampled = false;
-            count_pass = false;
-            if (K1 == K2) {  // one coarse key holds the median
-                if (sizeof(T) == 4) {
-                    tstar = (K)K1;
-                    return SEL_OK;
-                }
-                return SEL_SLOW_CAP;  // double: its exact keys are not known here
-            }
-            continue;
-        }
-        // one pass over all rows: exact weight of rows certainly below P1; rows
-        // whose approximate key is within G of [P1, P2] become candidates
-        const uint32_t bt = sat_sub(P1, G);  // certain below: key' < bt
-        const uint32_t at = min(sat_add(P2, G), CKMAX);  // certain above: key' > at
-        int64_t Sb = 0;
-        cnt = 0;
-        // rows are visited in batches of 4 per lane; the global loads of the next
-        // batch are issued before the current one is classified, so the L2
-        // latency overlaps the work
-        // U * 32 = ROW_PAD rows per batch: every index below the padded row
-        // count is readable, and padding rows (reciprocal NaN) are neither
-        // below nor candidates
-        constexpr int U = 4;
-        static_assert(U * 32 == ROW_PAD, "one batch = one row pad");
-        float an[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) an[u] = xf[u * 32 + lane];
-        for (int i0 = 0; i0 < n; i0 += 32 * U) {
-            float ac[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) ac[u] = an[u];
-            if (i0 + 32 * U < n) {
-#pragma unroll
-                for (int u = 0; u < U; ++u) an[u] = xf[i0 + 32 * U + u * 32 + lane];
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                // branch-free
-                const int i = i0 + u * 32 + lane;
-                const float iv = inv[i];
-                const uint32_t kk = akey(__fmul_rn(ac[u], iv));
-                const bool below = kk < bt;
-                const bool cand = !below && kk <= at;
-                const int64_t q = colq(i);
-                Sb += below ? q : 0;
-                // speculative store: the slot is only kept when cnt advances
-                if (cnt < qt) {
-                    lk[L1L_CHK(cnt * 32 + lane, nslot)] = kk;
-                    li[cnt * 32 + lane] = (uint16_t)L1L_CHK(i, nrow);
-                }
-                cnt += cand ? 1 : 0;
-            }
-        }
-        Sb = warp_sum_i64(Sb);
-        __syncwarp();
-        if (__any_sync(FULL, cnt > qt)) {  // a lane overflowed: narrow by a count pass
-            if (P1 == P2) return SEL_SLOW_CAP;
-            count_pass = true;
-            continue;
-        }
-        // exact histogram of the candidates over the bins of [P1, P2]; rows
-        // within G of P1, P2 or their bin's edges are divided exactly first;
-        // Sb2 = exact weight below P1
-        BinMap bm;
-        bm.init(P1, P2, XB);
-        const uint32_t g1 = sat_add(P1, G), g2 = sat_sub(P2, G);
-        hist_zero(hist, lane);
-        __syncwarp();
-        int64_t Sb2 = 0;
-#pragma unroll 2
-        for (int j = 0; j < cnt; ++j) {
-            const int p = L1L_CHK(j * 32 + lane, nslot);
-            uint32_t kk = lk[p];
-            const uint16_t id = (uint16_t)L1L_CHK((int)li[p], nrow);
-            // clear: the keys G either side fall in the same bin
-            const bool clear = kk >= g1 && kk <= g2 && bm.bin(kk - G) == bm.bin(kk + G);
-            if (!clear) {
-                kk = A::exact_ck(xk[id], colb[id]);
-                lk[p] = kk;
-                li[p] = id | EXACT_BIT;
-            }
-            const int64_t q = colq(id);
-            if (kk < P1)
-                Sb2 += q;
-            else if (kk <= P2)
-                hist_add(hist, bm.bin(kk), q);
-        }
-        Sb += warp_sum_i64(Sb2);
-        __syncwarp();
-        const int r1 = P1 == lo0 ? 0 : dc.cond(Sb, (P1 - 1) >= CK0);
-        if (r1 < 0) return SEL_SLOW_BAND;
-        if (r1 == 1) {  // median below P1: retry under P1
-            hi0 = P1 - 1;
-            P2 = hi0;
-            P1 = sampled ? max(sat_sub(pick(jx - 3 * max(d0, 1) - 1, lo0), 2 * G + 1), lo0) : lo0;
-            if (P1 > P2) P1 = lo0;
-            continue;
-        }
-        int64_t below = 0;
-        const int bs = hist_cross_map(hist, bm, Sb, dc, &below, lane);
-        __syncwarp();
-        if (bs == -2) return SEL_SLOW_BAND;
-        if (bs < 0) {  // median above P2: retry over P2
-            if (P2 >= hi0) return SEL_INTERNAL;
-            lo0 = P2 + 1;
-            P1 = lo0;
-            P2 = sampled ? min(sat_add(pick(jx + 3 * max(d0, 1) + 1, hi0), 2 * G + 1), hi0) : hi0;
-            if (P2 < P1) P2 = hi0;
-            continue;
-        }
-        // the median is in bin bs: keep its candidates (lane-local, in place)
-        const uint32_t K1 = bm.lower(bs);
-        const uint32_t K2 = bm.upper(bs);
-        int w = 0;
-#pragma unroll 2
-        for (int j = 0; j < cnt; ++j) {
-            const int p = j * 32 + lane;
-            const uint32_t kk = lk[p];
-            const uint16_t id = li[p];
-            lk[w * 32 + lane] = kk;  // w <= j: kept only if w advances
-            li[w * 32 + lane] = id;
-            w += (kk >= K1 && kk <= K2) ? 1 : 0;
-        }
-        __syncwarp();
-        cnt = w;
-        L = below;
-        lo = K1;
-        hi = K2;
-        placed = true;
-    }
-    if (!placed) return SEL_SLOW_TRIES;
-
-    // ---------------- levels on the candidate list: exact histograms ------
-    int c = __reduce_add_sync(FULL, cnt);
-    for (int level = 0; c > 31 && lo < hi; ++level) {
-        if (level >= 8) return SEL_SLOW_LEVELS;
-        const uint32_t span = hi - lo;
-        const int sh = span >= (uint32_t)XB ? (32 - __clz((int)span)) - 6 : 0;
-        const uint32_t bmask = (1u << sh) - 1u;
-        const int nbins = (int)(span >> sh) + 1;
-        hist_zero(hist, lane);
-        __syncwarp();
-#pragma unroll 2
-        for (int j = 0; j < cnt; ++j) {
-            const int p = L1L_CHK(j * 32 + lane, nslot);
-            uint32_t kk = lk[p];
-            uint16_t id = li[p];
-            (void)L1L_CHK((int)(id & ROW_MASK), nrow);  // counted in the checked build
-            const uint32_t off = (kk - lo) & bmask;
-            if (!(id & EXACT_BIT) && (off < G || off + G > bmask)) {
-                const int row = id & ROW_MASK;
-                kk = A::exact_ck(xk[row], colb[row]);
-                lk[p] = kk;
-                id = (uint16_t)row | EXACT_BIT;
-                li[p] = id;
-            }
-            hist_add(hist, (int)((kk - lo) >> sh), colq(id & ROW_MASK));
-        }
-        __syncwarp();
-        int64_t below = 0;
-        const int bs = hist_cross(hist, nbins, lo, hi, sh, L, dc, &below, lane);
-        __syncwarp();
-        if (bs == -2) return SEL_SLOW_BAND;
-        if (bs < 0) return SEL_INTERNAL;
-        const uint32_t K1 = lo + ((uint32_t)bs << sh);
-        const uint32_t K2 = min(hi, K1 + bmask);
-        int w = 0;
-#pragma unroll 2
-        for (int j = 0; j < cnt; ++j) {
-            const int p = j * 32 + lane;
-            const uint32_t kk = lk[p];
-            const uint16_t id = li[p];
-            lk[w * 32 + lane] = kk;
-            li[w * 32 + lane] = id;
-            w += (kk >= K1 && kk <= K2) ? 1 : 0;
-        }
-        __syncwarp();
-        cnt = w;
-        L = below;
-        lo = K1;
-        hi = K2;
-        c = __reduce_add_sync(FULL, cnt);
-    }
-
-    // ---------------- final: exact keys of the candidates ------------------
-    if (sizeof(T) == 4 && lo == hi) {  // coarse keys are the exact keys for float
-        tstar = (K)lo;
-        return SEL_OK;
-    }
-    if (c > 31) {  // one coarse key left, many rows: all exact keys equal?
-        K kmin = Tr::NONE, kmax = 0;
-#pragma unroll 2
-        for (int j = 0; j < cnt; ++j) {
-            const int row = li[j * 32 + lane] & ROW_MASK;
-            const K ke = Tr::key(Tr::div_rn(xk[row], colb[row]));
-            kmin = min(kmin, ke);
-            kmax = max(kmax, ke);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            kmin = min(kmin, __shfl_xor_sync(FULL, kmin, o));
-            kmax = max(kmax, __shfl_xor_sync(FULL, kmax, o));
-        }
-        const bool zero_in = lo <= CK0 && CK0 <= hi;
-        if (kmin == kmax && !(zero_in && kmin != Tr::KEY0)) {
-            tstar = kmin;
-            return SEL_OK;
-        }
-        return SEL_SLOW_TIE;
-    }
-    // gather the <= 31 candidate rows into lanes 0..c-1 (via the histogram buffer)
-    {
-        const int excl = warp_scan_add(cnt, lane) - cnt;
-        uint16_t *stage = reinterpret_cast<uint16_t *>(hist);
-        for (int j = 0; j < cnt; ++j)
-            stage[L1L_CHK(excl + j, 31)] = li[L1L_CHK(j * 32 + lane, nslot)] & ROW_MASK;
-    }
-    __syncwarp();
-    K fk = Tr::NONE;
-    int64_t fq = 0;
-    if (lane < c) {
-        const int row = L1L_CHK((int)reinterpret_cast<const uint16_t *>(hist)[lane], nrow);
-        fk = Tr::key(Tr::div_rn(xk[row], colb[row]));
-        fq = colq(row);
-    } else if (lane == c && lo <= CK0 && CK0 <= hi) {
-        fk = Tr::KEY0;
-        fq = 0;
-    }
-    __syncwarp();
-    // Rank form of "sort, prefix-sum, take the first key that passes": each
-    // candidate sums the weight of the candidates whose key is <= its own
-    // (equal keys get equal sums), tests it, and the smallest key that passes
-    // (or cannot be settled) is the answer.  A few candidates remain here, so
-    // this costs a few shuffles per candidate instead of a 32-lane sort.
-    const int nv = c + ((lo <= CK0 && CK0 <= hi) ? 1 : 0);
-    int64_t S = 0;
-    for (int u = 0; u < nv; ++u) {
-        const K ku = __shfl_sync(FULL, fk, u);
-        const int64_t qu = __shfl_sync(FULL, fq, u);
-        S += ku <= fk ? qu : 0;
-    }
-    int r = 0;
-    if (lane < nv) r = dc.cond(L + S, fk >= Tr::KEY0);
-    K kmin = r != 0 ? fk : Tr::NONE;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) kmin = min(kmin, __shfl_xor_sync(FULL, kmin, o));
-    if (kmin == Tr::NONE) return SEL_INTERNAL;
-    if (__any_sync(FULL, r == -1 && fk == kmin)) return SEL_SLOW_BAND;
-    tstar = kmin;
-    return SEL_OK;
-}
 
 // The exact test of lambda tl on the fast path's weight scale (q32).
 template <typename T>
@@ -778,50 +277,8 @@ __device__ __forceinline__ Dec32 decide_for(const WarpCtx<T> &w, const LamView &
     if (tl < NDEC)
         dc = w.s_dec[tl];
     else
-        dc.set(w.cinfo, lp.lam[tl]);
+        dc.set(*w.ci, lp.lam[tl]);
     return dc;
-}
-
-// The 64-bit selection of a pair that the 32-bit weights could not settle
-// (rare): a separate, not inlined function, so that its code stays out of the
-// hot loop's instruction stream.  Weights are computed from x_ijhat.
-template <typename T>
-__device__ __noinline__ int select_fallback64(const T *xk, const float *xf, const T *colb,
-                                              const float *inv, const uint16_t *samp,
-                                              uint32_t *lk, uint16_t *li, uint32_t *hist,
-                                              int qt, int n, int d0, int64_t Q, int sigma,
-                                              int inexact, double lam,
-                                              typename Traits<T>::K *ts, int lane) {
-    Decide d64;
-    d64.init_at(Q, sigma, inexact, lam);
-    typename Traits<T>::K k = 0;
-    const int st = select_v2<T>(xk, xf, colb, inv, WqFly<T>{colb, sigma}, samp, lk, li, hist, qt,
-                                n, d0, d64, k, lane);
-    *ts = k;
-    return st;
-}
-
-// The full selection of one (lambda, pair): the 32-bit weights first, and the
-// pair again on 64-bit weights (computed from x_ijhat) when those cannot
-// settle it.
-template <typename T>
-__device__ __forceinline__ int select_pair(const T *xk, const float *xf, const WarpCtx<T> &w,
-                                           const LamView &lp, int tl,
-                                           typename Traits<T>::K &ts, int lane) {
-    const Dec32 dc = decide_for(w, lp, tl);
-    typename Traits<T>::K t32 = 0;
-    const int st = select_w32<T>(xf, xk, w, dc, t32, lane);
-    if (st != SEL_W64) {
-        ts = t32;
-        return st;
-    }
-    __syncwarp();
-    typename Traits<T>::K t64 = 0;
-    const int st64 = select_fallback64<T>(xk, xf, w.colb, w.inv, w.samp, w.lk, w.li, w.hist, w.qt,
-                                          w.n, w.d0, w.cinfo.Q, w.cinfo.sigma, w.cinfo.n_inexact,
-                                          lp.lam[tl], &t64, lane);
-    ts = t64;
-    return st64;
 }
 
 // ---------------------------------------------------------------------------
@@ -967,6 +424,7 @@ __device__ void emit_pair(const ScanArgs<T> &a, int t, int64_t j, int64_t k, int
             e.inst = (int16_t)a.inst;
             e.reason = (int16_t)st;
             a.slow[slot] = e;
+            a.s_all[o] = 0.0;  // no mark of a pair put off
         }
         return;
     }
@@ -988,159 +446,244 @@ __device__ void emit_pair(const ScanArgs<T> &a, int t, int64_t j, int64_t k, int
     }
 }
 
-// One lambda of one pair: the full selection.
+// Lists pair (t, j, k), not settled by the selection: `why` SEL_W64, or SEL_MANY for all
+// lambdas of the launch.
+template <typename T>
+__device__ __forceinline__ void list_off(const ScanArgs<T> &a, int t, int64_t j, int64_t k,
+                                         int why, int64_t mark, int lane) {
+    if (lane == 0) {
+        reinterpret_cast<int64_t *>(a.s_all)[((int64_t)t * a.m + j) * a.m + k] = mark;
+        a.slow[atomicAdd(a.slow_count, 1u)] =
+            SlowEntry{t, (int32_t)j, (int32_t)k, (int16_t)a.inst, (int16_t)why};
+    }
+}
+
+// One lambda of one pair (valid: x_ijhat != 0 somewhere; batch: one of several, whose
+// ties are settled together: the mark of that in whole).  What the selection cannot settle is listed: with a call
+// here, what lived across it was spilled in the hot loop, and a pair that takes several
+// times as long as the others held up its CTA (2000 x 2000 float 11.1 ms with the
+// fallback in this place, 10.5 without).  Returns whether the batch is listed.
 template <typename T, bool CS, bool VO>
-__device__ void solve_one(const ScanArgs<T> &a, const LamView &lp, int t0, int tl, int64_t j,
-                          int64_t k, const T *xk, const float *xf, const WarpCtx<T> &w,
-                          bool slow_pair, int lane) {
+__device__ __forceinline__ bool solve_one(const ScanArgs<T> &a, const LamView &lp, int t0, int tl,
+                                          int64_t j, int64_t k, const T *xk, const float *xf,
+                                          const WarpCtx<T> &w, bool slow_pair, bool valid,
+                                          bool batch, int64_t whole, int lane) {
     using Tr = Traits<T>;
     typename Tr::K ts = Tr::KEY0;
     int st = SEL_OK;
     if (slow_pair) {
         st = SEL_SLOW;
-    } else if (w.cinfo.n_valid > 0) {
-        st = select_pair<T>(xk, xf, w, lp, tl, ts, lane);
+    } else if (valid) {
+        int64_t mark = 0;
+        const int sel = select_w32<T>(xf, xk, w, decide_for(w, lp, tl), ts, mark, lane);
+        if (sel != SEL_OK) {
+            const bool all = batch && sel == SEL_MANY;
+            list_off(a, t0 + tl, j, k, all ? SEL_MANY : SEL_W64, all ? whole : mark, lane);
+            return all;
+        }
     }
     emit_pair<T, CS, VO>(a, t0 + tl, j, k, st, ts, xk, w.colb, w.n, lp.lam[tl], lane);
+    return false;
+}
+
+// A batch of lambdas against candidates between two penalties' medians: lane l holds
+// the weight P up to its key fk, ascending; `last`: the lanes that end a run of equal
+// keys, `nonneg`: those with a key >= 0; L, after_zero: the weight below them and
+// whether the penalty point lies there.
+template <typename T> struct LamCand {
+    typename Traits<T>::K fk;
+    int64_t P, L;
+    unsigned last, nonneg;
+    bool after_zero;
+    __device__ __forceinline__ void init(typename Traits<T>::K key, int64_t fq, int64_t below,
+                                         bool zero_below, int lane) {
+        using Tr = Traits<T>;
+        fk = key;
+        warp_sort32(fk, fq, lane);
+        P = below + warp_scan_add(fq, lane);
+        const typename Tr::K nxt = __shfl_down_sync(0xFFFFFFFFu, fk, 1);
+        // the last candidate of each key holds the weight up to it
+        last = __ballot_sync(0xFFFFFFFFu, fk != Tr::NONE && (lane == 31 || nxt != fk));
+        nonneg = __ballot_sync(0xFFFFFFFFu, fk >= Tr::KEY0);
+        L = below;
+        after_zero = zero_below;
+    }
+};
+
+// The lambdas of the lanes with `on`, one per lane (t: of the call; lam, dc: its value
+// and test), each against every candidate in turn; the residual is summed once per value
+// that any of them takes.  Writes what they decide and returns those lanes; for the
+// others they are undecided, or none passes.
+template <typename T, bool CS, typename D>
+__device__ __forceinline__ unsigned lambda_decide(const ScanArgs<T> &a, const LamCand<T> &f,
+                                                  const D &dc, int t, double lam, bool on,
+                                                  int64_t j, int64_t k,
+                                                  const T *__restrict__ xk, const T *colb, int n,
+                                                  int lane) {
+    using Tr = Traits<T>;
+    const unsigned FULL = 0xFFFFFFFFu;
+    int first = -1, res = 0;
+    const int below = dc.cond(f.L, f.after_zero);
+    for (unsigned c = f.last; c; c &= c - 1) {
+        const int u = __ffs(c) - 1;
+        const int r = dc.cond(__shfl_sync(FULL, f.P, u), (f.nonneg >> u) & 1u);
+        if (first < 0 && r != 0) {
+            first = u;
+            res = r;
+        }
+    }
+    const bool ok = on && first >= 0 && res == 1 && below == 0;
+    const T v = Tr::value(__shfl_sync(FULL, f.fk, max(first, 0)));
+    T r = T(0);
+    const unsigned done = __ballot_sync(FULL, ok);
+    for (unsigned todo = done; todo;) {
+        const int src = __ffs(todo) - 1;
+        const T vs = __shfl_sync(FULL, v, src);
+        const int u = __shfl_sync(FULL, first, src);
+        const T rs = pair_residual<T, CS>(a, j, k, xk, colb, n, vs, lane);
+        if (first == u) r = rs;
+        todo &= ~__ballot_sync(FULL, first == u);
+    }
+    if (ok) {
+        const int64_t o = L1L_CHK(((int64_t)t * a.m + j) * a.m + k,
+                                  (int64_t)a.n_lambda * a.m * a.m);
+        a.v_all[o] = v;
+        a.s_all[o] = (double)r + lam * (double)fabs(v);
+    }
+    return done;
 }
 
 // Lambda batch (step A7).  The weighted median moves monotonically toward 0
 // as lambda grows (the penalty point only gains weight), so every lambda's
 // median lies between those of the smallest and the largest lambda: one
 // selection brackets both, and one sort and prefix scan of the candidates
-// between them serve every lambda.  32 lambdas are decided at a time, one per
-// lane, each against every candidate in turn; the residual is summed once per
-// value that any of them takes.  (Deciding one lambda at a time by the whole
-// warp took half of the kernel at 32 lambdas: 1000 x 500 float 2.53 -> 1.39 ms;
-// 30 x 100 x 100 double with 8 lambdas 1.09 -> 0.79 ms.)
-// When more than 31 rows lie between, or a bracket fails, returns false with
-// nothing written, and the caller takes the lambdas one by one.  RUNS, from
-// RUN_MIN lambdas on: they are ranked and taken in runs of neighbours instead,
-// halved until a run's rows fit; one or two left over take the full selection
-// each.  One by one left a CTA's 16 warps waiting for the one with such a pair:
-// 1000 x 500 float with 32 lambdas 1.41 -> 1.29 ms.  Only the float kernel of
-// single matrices does so: its code cost 30 x 100 x 100 double with 8 lambdas 11%.
-constexpr int RUN_MIN = 16;
-template <typename T, bool CS, bool RUNS>
-__device__ bool lambda_path(const ScanArgs<T> &a, const LamView &lp, int t0, int nlc, int64_t j,
-                            int64_t k, const T *__restrict__ xk, const float *__restrict__ xf,
-                            const WarpCtx<T> &w, int lane) {
-    using Tr = Traits<T>;
-    using K = typename Tr::K;
-    const unsigned FULL = 0xFFFFFFFFu;
-    bool whole = true;             // the first attempt: all lambdas at once
-    int tb = -32, cnt = 0;         // then: the lambdas tb .. tb + cnt, one per lane,
-    int rank = 0, lo = 0, len = 0;  // this lane's place by size; the run [lo, lo + len)
-    for (;;) {
-        int t1 = lp.tl_min, t2 = lp.tl_max;
-        if (RUNS && !whole) {
-            if (lo >= cnt) {  // the next 32
-                tb += 32;
-                if (tb >= nlc) return true;
-                cnt = min(32, nlc - tb);
-                const double mine = lane < cnt ? lp.lam[tb + lane] : INFINITY;
-                rank = 0;
-                for (int u = 0; u < cnt; ++u) {
-                    const double o = __shfl_sync(FULL, mine, u);
-                    rank += o < mine || (o == mine && u < lane) ? 1 : 0;
-                }
-                if (lane >= cnt) rank = lane;
-                lo = 0;
-                len = nlc <= 32 ? (cnt + 1) / 2 : cnt;  // all of them just failed
-            }
-            len = min(len, cnt - lo);
-            t1 = tb + __ffs(__ballot_sync(FULL, rank == lo)) - 1;
-            t2 = tb + __ffs(__ballot_sync(FULL, rank == lo + len - 1)) - 1;
+// between them serve every lambda, 32 at a time.  (Deciding one lambda at a time
+// by the whole warp took half of the kernel at 32 lambdas: 1000 x 500 float 2.53 ->
+// 1.39 ms; 30 x 100 x 100 double with 8 lambdas 1.09 -> 0.79 ms.)  Returns SEL_OK, or
+// why not all of them are settled and, where known, the range of their medians.
+template <typename T, bool CS>
+__device__ __forceinline__ int lambda_whole(const ScanArgs<T> &a, const LamView &lp, int t0,
+                                             int nlc, int64_t j, int64_t k,
+                                             const T *__restrict__ xk,
+                                             const float *__restrict__ xf, const WarpCtx<T> &w,
+                                             uint32_t &lo, uint32_t &hi, int lane) {
+    Cand32<T> f;
+    f.lo = 1;
+    f.hi = 0;
+    int st = candidates32<T, true>(xf, xk, w, decide_for(w, lp, lp.tl_min),
+                                         decide_for(w, lp, lp.tl_max), f, lane);
+    if (st == SEL_OK) {
+        LamCand<T> c;
+        c.init(f.fk, (int64_t)f.fq, f.L, f.lo > CK0, lane);
+        for (int cb = 0; cb < nlc; cb += 32) {
+            const bool on = cb + lane < nlc;
+            const int tl = on ? cb + lane : 0;
+            if (lambda_decide<T, CS>(a, c, decide_for(w, lp, tl), t0 + tl, lp.lam[tl], on, j, k,
+                                     xk, w.colb, w.n, lane) != __ballot_sync(0xFFFFFFFFu, on))
+                st = SEL_W64;
         }
+    }
+    lo = f.lo;
+    hi = f.hi;
+    return st;
+}
+
+// The batch in parts, where the whole has more than 31 rows between its medians or a
+// bracket fails: runs of neighbouring lambdas, halved until a run's rows fit; their
+// candidates serve whatever other lambda they decide.  One by one left a CTA's 16 warps
+// waiting for the one with such a pair: 1000 x 500 float with 32 lambdas 1.41 -> 1.29 ms;
+// in a kernel of its own, so that the first attempt's does not spill, 1.03 ms.  From
+// RUN_MIN lambdas on; fewer are taken one by one at once.
+constexpr int RUN_MIN = 16;
+template <typename T, bool CS>
+__device__ void lambda_parts(const ScanArgs<T> &a, const LamView &lp, int t0, int nlc, int64_t j,
+                             int64_t k, const T *xk, const float *xf, const WarpCtx<T> &w,
+                             int64_t whole, int lane) {
+    const unsigned FULL = 0xFFFFFFFFu;
+    int tb = -32, cnt = 0;    // the lambdas tb .. tb + cnt, one per lane,
+    unsigned left = 0;        // those of them still to do,
+    int rank = 0, len = 1;    // this lane's place by size, and the run's length
+    for (;;) {
+        if (left == 0) {  // the next 32, ranked
+            tb += 32;
+            if (tb >= nlc) return;
+            cnt = min(32, nlc - tb);
+            left = FULL >> (32 - cnt);
+            const double mine = lane < cnt ? lp.lam[tb + lane] : INFINITY;
+            rank = 0;
+            for (int u = 0; u < cnt; ++u) {
+                const double o = __shfl_sync(FULL, mine, u);
+                rank += o < mine || (o == mine && u < lane) ? 1 : 0;
+            }
+            if (lane >= cnt) rank = lane;
+            len = nlc <= 32 ? (cnt + 1) / 2 : cnt;  // all of them just failed
+        }
+        const bool mine = (left >> lane) & 1u;
+        const int r0 = __reduce_min_sync(FULL, mine ? rank : 32);
+        const unsigned part = __ballot_sync(FULL, mine && rank < r0 + len);
+        const int r1 = __reduce_max_sync(FULL, (part >> lane) & 1u ? rank : 0);
+        const int t1 = tb + __ffs(__ballot_sync(FULL, rank == r0)) - 1;
+        const int t2 = tb + __ffs(__ballot_sync(FULL, rank == r1)) - 1;
         Cand32<T> f;
-        const bool few = RUNS && !whole && len < 3;
-        if (!few && candidates32<T, true>(xf, xk, w, decide_for(w, lp, t1), decide_for(w, lp, t2),
-                                          f, lane) != SEL_OK) {
-            if (!RUNS || nlc < RUN_MIN) return false;
-            if (whole)
-                whole = false;
-            else
-                len = (len + 1) / 2;
-            __syncwarp();
+        const int st = candidates32<T, true>(xf, xk, w, decide_for(w, lp, t1),
+                                             decide_for(w, lp, t2), f, lane, t1 == t2);
+        __syncwarp();
+        if (st == SEL_MANY) {
+            list_off(a, t0 + t1, j, k, SEL_MANY, whole, lane);
+            return;
+        }
+        if (st != SEL_OK && len > 1) {
+            len = len > 2 ? (len + 1) / 2 : 1;
             continue;
         }
-        K fk = Tr::NONE;
-        int64_t P = 0;
-        unsigned last = 0, nonneg = 0;
-        if (!few) {
-            fk = f.fk;
-            int64_t fq = (int64_t)f.fq;
-            warp_sort32(fk, fq, lane);
-            P = f.L + warp_scan_add(fq, lane);
-            const K nxt = __shfl_down_sync(FULL, fk, 1);
-            // the last candidate of each key holds the weight up to it
-            last = __ballot_sync(FULL, fk != Tr::NONE && (lane == 31 || nxt != fk));
-            nonneg = __ballot_sync(FULL, fk >= Tr::KEY0);
+        unsigned ok = 0;
+        if (st == SEL_OK) {
+            LamCand<T> c;
+            c.init(f.fk, (int64_t)f.fq, f.L, f.lo > CK0, lane);
+            const int tl = mine ? tb + lane : 0;
+            ok = lambda_decide<T, CS>(a, c, decide_for(w, lp, tl), t0 + tl, lp.lam[tl], mine, j,
+                                      k, xk, w.colb, w.n, lane);
         }
-        const int ce = !RUNS || whole ? nlc : tb + 1;
-        for (int cb = !RUNS || whole ? 0 : tb; cb < ce; cb += 32) {
-            const int tl = cb + lane;
-            const bool on = tl < nlc && (!RUNS || whole || (rank >= lo && rank < lo + len));
-            bool ok = false;
-            if (!few) {
-                int first = -1, res = 0, below = 0;
-                {
-                    const Dec32 dc = decide_for(w, lp, on ? tl : 0);
-                    below = dc.cond(f.L, f.lo > CK0);
-                    for (unsigned c = last; c; c &= c - 1) {
-                        const int u = __ffs(c) - 1;
-                        const int r = dc.cond(__shfl_sync(FULL, P, u), (nonneg >> u) & 1u);
-                        if (first < 0 && r != 0) {
-                            first = u;
-                            res = r;
-                        }
-                    }
-                }
-                // else undecided here, or already passed below lo: full selection
-                ok = on && first >= 0 && res == 1 && below == 0;
-                const T v = Tr::value(__shfl_sync(FULL, fk, max(first, 0)));
-                T r = T(0);
-                for (unsigned todo = __ballot_sync(FULL, ok); todo;) {
-                    const int src = __ffs(todo) - 1;
-                    const T vs = __shfl_sync(FULL, v, src);
-                    const int u = __shfl_sync(FULL, first, src);
-                    const T rs = pair_residual<T, CS>(a, j, k, xk, w.colb, w.n, vs, lane);
-                    if (first == u) r = rs;
-                    todo &= ~__ballot_sync(FULL, first == u);
-                }
-                if (ok) {
-                    const int64_t o = L1L_CHK(((int64_t)(t0 + tl) * a.m + j) * a.m + k,
-                                              (int64_t)a.n_lambda * a.m * a.m);
-                    a.v_all[o] = v;
-                    a.s_all[o] = (double)r + lp.lam[tl] * (double)fabs(v);
-                }
-            }
-            for (unsigned left = __ballot_sync(FULL, on && !ok); left; left &= left - 1)
-                solve_one<T, CS, false>(a, lp, t0, cb + __ffs(left) - 1, j, k, xk, xf, w, false,
-                                        lane);
+        left &= ~(ok | part);
+        for (unsigned rest = part & ~ok; rest; rest &= rest - 1) {  // undecided: each by itself
+            if (solve_one<T, CS, false>(a, lp, t0, tb + __ffs(rest) - 1, j, k, xk, xf, w, false,
+                                        true, true, whole, lane))
+                return;
+            __syncwarp();
         }
-        if (!RUNS || whole) return true;
-        lo += len;
         __syncwarp();
     }
 }
 
 // One work unit: column jhat = j of an instance and the k in [k0, k1), all
 // lambdas of the launch.  Called by every thread of a CTA; `smem` is laid out
-// for lay_npad rows (column arrays, then one candidate list per warp).  CS:
+// for lay_npad rows (column arrays, then one histogram per warp).  CS:
 // x_ijhat is staged in shared memory; otherwise the warps read it from the
 // column copy in global memory (L2-resident), which frees shared memory for
 // more resident warps when n is large.
-// RUNS: of lambda_path.
-template <typename T, bool MULTI, bool CS, bool RUNS>
+// What a unit is: the lambdas one by one; as a batch; the batches put off by that (where
+// `parts` says that such units follow).
+enum : int { UNIT_ONE, UNIT_BATCH, UNIT_PARTS };
+template <typename T, int WHAT, bool CS>
 __device__ void pairs_unit(const ScanArgs<T> &a, const LamView &lp, int t0, int nlc, int j,
-                           int64_t k0, int64_t k1, int cap, int lay_npad, unsigned char *smem,
-                           Dec32 *s_dec) {
+                           int64_t k0, int64_t k1, int cap, int lay_npad, bool parts,
+                           unsigned char *smem, Dec32 *s_dec) {
     const int n = (int)a.n;
     const int64_t m = a.m, ldn = a.ldn;
     const int npad = lay_npad;  // shared-memory layout stride (>= n rounded up to 32)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
+    auto mark_of = [&](int64_t k) -> int64_t {
+        const int64_t o = L1L_CHK(((int64_t)t0 * m + j) * m + k, (int64_t)a.n_lambda * m * m);
+        // k = jhat: s is lambda, which may be -0
+        return k == j ? 0 : reinterpret_cast<const int64_t *>(a.s_all)[o];
+    };
+    auto put_off = [](int64_t mark) { return mark < 0 && off_why(mark) == OFF_BATCH; };
+    if (WHAT == UNIT_PARTS) {
+        int any = 0;
+        for (int64_t k = k0 + threadIdx.x; k < k1; k += blockDim.x) any |= put_off(mark_of(k));
+        if (!__syncthreads_or(any)) return;
+    }
     const T *xj = a.Xt + (int64_t)j * ldn;
     T *colb_s = reinterpret_cast<T *>(smem);
     const T *colb = CS ? colb_s : xj;
@@ -1154,8 +697,6 @@ __device__ void pairs_unit(const ScanArgs<T> &a, const LamView &lp, int t0, int 
     unsigned char *wbase =
         smem + PairSmem<T>::col_bytes(npad, CS) + (size_t)warp * PairSmem<T>::warp_bytes(cap);
     uint32_t *hist = reinterpret_cast<uint32_t *>(wbase);
-    uint32_t *lk = hist + HIST_WORDS;
-    uint16_t *li = reinterpret_cast<uint16_t *>(lk + cap);
     // prologue scratch: the first 256 bytes of warp 0's histogram
     long long *s_wsum = reinterpret_cast<long long *>(smem + PairSmem<T>::col_bytes(npad, CS));
 
@@ -1211,17 +752,13 @@ __device__ void pairs_unit(const ScanArgs<T> &a, const LamView &lp, int t0, int 
     wc.colb = colb;
     wc.inv = inv;
     wc.q32 = q32;
-    wc.samp = samp;
-    wc.lk = lk;
-    wc.li = li;
     wc.hist = hist;
     wc.srow = L1L_CHK((int)samp[2 * lane + 1], npad);
     wc.sinv = inv[wc.srow];
     wc.s_dec = s_dec;
-    wc.qt = cap / 32;
+    wc.ci = a.ci + j;
     wc.d0 = a.d0;
     wc.n = n;
-    wc.cinfo = cinfo;
 
     const bool jwide = (cinfo.flags & COL_WIDE) != 0;
     // a warp takes the next k when it is done with its pair: pairs cost
@@ -1232,6 +769,14 @@ __device__ void pairs_unit(const ScanArgs<T> &a, const LamView &lp, int t0, int 
         if (lane == 0) idx = atomicAdd(&s_knext, 1);
         const int64_t k = k0 + __shfl_sync(0xFFFFFFFFu, idx, 0);
         if (k >= k1) break;
+        const T *xk = a.Xt + k * ldn;
+        const float *xf = a.Xf + k * ldn;
+        if constexpr (WHAT == UNIT_PARTS) {
+            const int64_t mark = mark_of(k);
+            if (put_off(mark)) lambda_parts<T, CS>(a, lp, t0, nlc, j, k, xk, xf, wc, mark, lane);
+            __syncwarp();
+            continue;
+        }
         if (k == j) {  // v_jhat = 1: zero residual, penalty lambda * 1
             for (int tl = lane; tl < nlc; tl += 32) {
                 int64_t o = L1L_CHK(((int64_t)(t0 + tl) * m + j) * m + k,
@@ -1241,17 +786,31 @@ __device__ void pairs_unit(const ScanArgs<T> &a, const LamView &lp, int t0, int 
             }
             continue;
         }
-        const T *xk = a.Xt + k * ldn;
-        const float *xf = a.Xf + k * ldn;
         const bool slow_pair = a.force_exact || jwide ||
                                (sizeof(T) == 8 && (a.ci[k].flags & COL_WIDE));
-        if (MULTI && nlc >= 3 && !slow_pair && cinfo.n_valid > 0 &&
-            lambda_path<T, CS, RUNS>(a, lp, t0, nlc, j, k, xk, xf, wc, lane)) {
-            __syncwarp();
-            continue;
+        const bool batch = WHAT != UNIT_ONE && nlc >= 3 && !slow_pair && cinfo.n_valid > 0;
+        int64_t whole = 0;
+        if (batch) {
+            uint32_t lo, hi;
+            const int st = lambda_whole<T, CS>(a, lp, t0, nlc, j, k, xk, xf, wc, lo, hi, lane);
+            if (st == SEL_OK) continue;
+            whole = off_mark(OFF_BATCH, lo, hi);
+            if (st == SEL_MANY) {
+                list_off(a, t0, j, k, SEL_MANY, whole, lane);
+                continue;
+            }
+            if (parts && nlc >= RUN_MIN) {
+                if (lane == 0) {
+                    reinterpret_cast<int64_t *>(a.s_all)[((int64_t)t0 * m + j) * m + k] = whole;
+                    a.slow_count[1] = 1;
+                }
+                continue;
+            }
         }
         for (int tl = 0; tl < nlc; ++tl)
-            solve_one<T, CS, !MULTI>(a, lp, t0, tl, j, k, xk, xf, wc, slow_pair, lane);
+            if (solve_one<T, CS, WHAT == UNIT_ONE>(a, lp, t0, tl, j, k, xk, xf, wc, slow_pair,
+                                                   cinfo.n_valid > 0, batch, whole, lane))
+                break;
         __syncwarp();
     }
     __syncthreads();  // the CTA may stage another column next

@@ -33,10 +33,10 @@
 // weights must add up to the histogram's (no weighted row of the range is
 // missing), the weight below lo must fail the test of Lemma 1, and a key in
 // [lo, hi] must pass it.  A pair that does not meet this, more than 31 rows
-// in the range that no narrower bins separate (ties), a decision inside the
-// certainty band of the truncated weights (Decide, e = n_inexact32), or a
-// bracket too wide or narrow for float steps returns SEL_W64, and the caller
-// repeats the pair on 64-bit weights.
+// in the range (ties), a decision inside the certainty band of the truncated
+// weights (Decide, e = n_inexact32), or a bracket too wide for float steps is
+// listed for the kernel behind, with the range where it is known (exact.cuh,
+// narrow.cuh).
 //
 // Bound (2000 x 2000 float, 32 resident warps): the L1/shared data pipe, ~730
 // wavefronts of 128 bytes per pair at 70% of its rate (pass 1: x, 1/x_ijhat,
@@ -56,7 +56,6 @@
 
 namespace l1l {
 
-constexpr int SEL_W64 = 16;  // repeat this pair on 64-bit weights
 constexpr int NB32 = 256;     // bins of the bracket histogram
 constexpr int BPL = NB32 / 32;  // bins per lane of its scan
 constexpr int NB32_SIDE = 8;  // bins kept free either side of the bracket
@@ -209,11 +208,13 @@ template <typename T> struct Cand32 {
 // of penalty d2 (the same for one penalty).  xf: column k as float (global,
 // rows padded to a multiple of 128 with zeros; the column itself for float
 // input, its float copy for double input); xk, w.colb: column k and x_ijhat in
-// the input type, read for the exact divisions.  Returns SEL_OK or SEL_W64.
+// the input type, read for the exact divisions.  Returns SEL_OK, SEL_W64 or
+// SEL_MANY: more than 31 rows lie in [out.lo, out.hi] (for two penalties: that no
+// bins separate; `one` says that the two are equal).
 template <typename T, bool TWO>
 __device__ __forceinline__ int candidates32(const float *__restrict__ xf, const T *__restrict__ xk,
                                             const WarpCtx<T> &w, const Dec32 &d1, const Dec32 &d2,
-                                            Cand32<T> &out, int lane) {
+                                            Cand32<T> &out, int lane, bool one = false) {
     using Tr = Traits<T>;
     using K = typename Tr::K;
     constexpr uint32_t G = Approx<T>::G;  // guard band of the approximate keys
@@ -243,10 +244,11 @@ __device__ __forceinline__ int candidates32(const float *__restrict__ xf, const 
     if (jb > 31) b += b - a;
 
     for (int attempt = 0; attempt < 4; ++attempt) {
-        // ---- bins: steps of w1, no finer than 16 keys of the largest ratio
-        const float w1 = fmaxf((b - a) * (1.0f / (NB32 - 2 * NB32_SIDE)),
-                               fmaxf(fabsf(a), fabsf(b)) * 0x1p-19f);
-        if (!(w1 > 0x1p-100f && w1 < 0x1p100f)) return SEL_W64;
+        // ---- bins: steps of w1, no finer than 16 keys of the largest ratio (or
+        // 2^-99, where the whole bracket is 0: sparse columns)
+        const float wf = fmaxf(fmaxf(fabsf(a), fabsf(b)) * 0x1p-19f, 0x1p-99f);
+        const float w1 = fmaxf((b - a) * (1.0f / (NB32 - 2 * NB32_SIDE)), wf);
+        if (!(w1 < 0x1p100f)) return SEL_W64;
         const float sc = __frcp_rn(w1);
         const float bm = __fmaf_rn(-a, sc, Z32 + (float)NB32_SIDE);
         // ---- pass 1 ------------------------------------------------------
@@ -407,10 +409,15 @@ __device__ __forceinline__ int candidates32(const float *__restrict__ xf, const 
                     in &= in - 1;
                     c += __popc(m);
                 }
+                if (c > 31) mask = 0;
             }
         }
         __syncwarp();
-        if (c > 31) {  // finer bins over the range, unless it hardly shrank
+        if (c > 31) {
+            out.lo = ka + G;
+            out.hi = kb - G;
+            if (!TWO || one || w1 == wf) return SEL_MANY;
+            // two penalties: finer bins over the range, unless it hardly shrank
             if (!(vb - va < 0.25f * (b - a))) return SEL_W64;
             a = va;
             b = vb;
@@ -454,19 +461,26 @@ __device__ __forceinline__ int candidates32(const float *__restrict__ xf, const 
     return SEL_W64;
 }
 
-// Weighted median of pair (jhat, k) at one penalty: SEL_OK with its exact key
-// in tstar, or SEL_W64.
+// Weighted median of pair (jhat, k) at one penalty: SEL_OK with its exact key in
+// tstar, else SEL_MANY or SEL_W64 and the mark to list it with.
 template <typename T>
 __device__ __forceinline__ int select_w32(const float *__restrict__ xf, const T *__restrict__ xk,
                                           const WarpCtx<T> &w, const Dec32 &dc,
-                                          typename Traits<T>::K &tstar, int lane) {
+                                          typename Traits<T>::K &tstar, int64_t &mark,
+                                          int lane) {
     using Tr = Traits<T>;
     using K = typename Tr::K;
     const unsigned FULL = 0xFFFFFFFFu;
     Cand32<T> f;
-    if (candidates32<T, false>(xf, xk, w, dc, dc, f, lane) != SEL_OK) return SEL_W64;
+    if (const int st = candidates32<T, false>(xf, xk, w, dc, dc, f, lane); st != SEL_OK) {
+        mark = st == SEL_MANY ? off_mark(OFF_MANY, f.lo, f.hi) : off_mark(OFF_NONE, 1, 0);
+        return st;
+    }
     // no key below lo passes
-    if (dc.cond(f.L, f.lo > CK0) != 0) return SEL_W64;
+    if (dc.cond(f.L, f.lo > CK0) != 0) {
+        mark = off_mark(OFF_RANGE, f.lo, f.hi);
+        return SEL_W64;
+    }
     // each candidate's cumulative weight: the weight of candidates with a key
     // at or below its own (equal keys alike); the smallest key that passes
     uint32_t S = 0;
@@ -487,8 +501,10 @@ __device__ __forceinline__ int select_w32(const float *__restrict__ xf, const T 
             kmin = y < kmin ? y : kmin;
         }
     }
-    if (kmin == Tr::NONE) return SEL_W64;
-    if (__any_sync(FULL, r == -1 && f.fk == kmin)) return SEL_W64;
+    if (kmin == Tr::NONE || __any_sync(FULL, r == -1 && f.fk == kmin)) {
+        mark = off_mark(OFF_RANGE, f.lo, f.hi);
+        return SEL_W64;
+    }
     tstar = kmin;
     return SEL_OK;
 }
