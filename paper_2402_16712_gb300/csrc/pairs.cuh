@@ -232,6 +232,8 @@ template <typename T> struct WarpCtx {
     float sinv;
 };
 constexpr int NDEC = 32;
+// Static shared memory of the pair kernels, for the planner: s_dec and the counters.
+constexpr int PAIR_STATIC = NDEC * (int)sizeof(Dec32) + 16;
 
 // The place in s_all, whose values are never negative, of a pair that the selection
 // has not settled: the sign bit, whether the median lies in the range that follows, among
