@@ -20,7 +20,12 @@
 //            in the pair kernel's selection no step before has to be trusted:
 //            the rows' weights must add up to the bin's, and the weight below
 //            must fail the test.
-//   descent  what that cannot settle (ties, a wide column, few valid rows): a
+//   keys     more rows there than the list holds (from some 5 million rows on), or a
+//            sample that is dense around the median (ties, nearly collinear columns;
+//            in place of bins and rows): the smallest and largest exact key of the
+//            rows next to it, and if these differ passes that histogram the weights
+//            of the rows between by 2048 equal steps of the key, one or two for float.
+//   descent  what that cannot settle (a wide column, few valid rows): a
 //            radix descent over the order-preserving key of the correctly
 //            rounded ratio r_i = x_ik / x_ijhat, 11 key bits per pass (float:
 //            3 passes, double: 6).  A pass histograms the weights of the rows
@@ -136,6 +141,8 @@ template <typename T> struct LgPick {
     long long wsum[3][LG_NT / 32];
     K kmin;
     int und;
+    K kmn[3], kmx[3];                      // large_keys: of each part (read by the cluster);
+    uint32_t klo, khi, clo, chi;           // their range, and the middle one's
 };
 
 template <typename T> struct LgSmem {
@@ -266,6 +273,238 @@ __device__ __forceinline__ long long lg_sum(long long x, long long *ws) {
     return r;
 }
 
+// A key into the CTA's smallest and largest.
+template <typename T>
+__device__ __forceinline__ void lg_min_max(LgPick<T> &pk, int part, typename Traits<T>::K k) {
+    using K = typename Traits<T>::K;
+    if (k < *(volatile K *)&pk.kmn[part]) smem_min(&pk.kmn[part], k);
+    if (k > *(volatile K *)&pk.kmx[part]) smem_max(&pk.kmx[part], k);
+}
+
+// The median among the rows with a coarse key in [lo, hi] by their exact keys, LG_SEARCH
+// where it lies elsewhere.  listed: as the last step of the rows pass, whose list they
+// exceed: L is their exact weight below and at least `thr` lies at or below hi.  Else a
+// pass sums the weights below, and of those under, in and over [pk.clo, pk.chi].
+// k_large, 100,000 and 1,000,000 x 6 float: small integers 194 -> 80, 670 -> 229 us (by a
+// bracket that does not serve and the descent), multiples of one column 296 -> 229, 973 ->
+// 639 us; continuous, 8,000,000 x 4, 2.66 -> 0.80 ms.
+template <typename T>
+__device__ __noinline__ int large_keys(int sigma, const Decide &dec, const float *fj,
+                                       const float *fk, const T *xj, const T *xk, int64_t c0,
+                                       int64_t c1, uint32_t lo, uint32_t hi, bool listed,
+                                       long long L, long long thr, LgSmem<T> &sm, int &buf,
+                                       typename Traits<T>::K &key) {
+    using Tr = Traits<T>;
+    using K = typename Tr::K;
+    constexpr uint32_t G = Approx<T>::G;
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = (int)cl.num_blocks();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    LgPick<T> &pk = *reinterpret_cast<LgPick<T> *>(&sm.copies[0][0]);
+    // rows that |fma(x, 1/b, -cen)| < delta does not flag lie outside [lo, hi]
+    const float va = akey_value(sat_sub(lo, G)), vb = akey_value(sat_add(hi, G));
+    const float cen = 0.5f * va + 0.5f * vb;
+    const float delta = (0.5f * vb - 0.5f * va) * (1.0f + 0x1p-20f) +
+                        0x1p-21f * fmaxf(fabsf(va), fabsf(vb)) + 0x1p-148f;
+    if (!(delta < 0x1p126f) || !(fabsf(cen) < 0x1p126f)) return LG_SEARCH;
+    K A = Tr::NONE, B = 0;
+    if (listed) {
+        for (int e = tid; e < min(pk.lcnt, LG_ROWS); e += LG_NT) lg_min_max(pk, 0, pk.lkey[e]);
+        cl.sync();
+        for (int r = 0; r < C; ++r) {
+            const LgPick<T> *o = cl.map_shared_rank(&pk, r);
+            A = o->kmn[0] < A ? o->kmn[0] : A;
+            B = o->kmx[0] > B ? o->kmx[0] : B;
+        }
+        cl.sync();  // the histograms overlap what the cluster read
+        if (lo <= CK0 && CK0 <= hi) {  // the penalty point
+            A = Tr::KEY0 < A ? Tr::KEY0 : A;
+            B = Tr::KEY0 > B ? Tr::KEY0 : B;
+        }
+    } else {
+        const uint32_t clo = pk.clo, chi = pk.chi;
+        if (tid < 3) {  // the penalty point among them
+            const bool zero = lo <= CK0 && CK0 <= hi && tid == (CK0 < clo ? 0 : (CK0 <= chi ? 1 : 2));
+            pk.kmn[tid] = zero ? Tr::KEY0 : Tr::NONE;
+            pk.kmx[tid] = zero ? Tr::KEY0 : 0;
+        }
+        __syncthreads();
+        long long below = 0, part[3] = {0, 0, 0};
+        for (int64_t v = c0 + tid; v < c1; v += LG_UB * LG_NT) {
+            LgRows<T, LG_UB> x;
+            x.load(fj, fk, xj, v, c1);
+#pragma unroll
+            for (int g = 0; g < LG_UB; ++g)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const T b = x.w(g, u);
+                    const float z = __fmaf_rn(x.a(g, u), rcp_approx(x.b(g, u)), -cen);
+                    int e = 0;
+                    if (fabsf(z) < delta) {  // b != 0: else z is infinite or NaN
+                        const K k = Tr::key(Tr::div_rn(xk[4 * (v + g * LG_NT) + u], b));
+                        const uint32_t ck = coarse_of<T>(k);
+                        const long long q = fixq(fabs(b), sigma, e);
+                        if (ck < lo) below += q;
+                        if (ck >= lo && ck <= hi) {
+                            const int p = ck < clo ? 0 : (ck <= chi ? 1 : 2);
+#pragma unroll
+                            for (int r = 0; r < 3; ++r) part[r] += p == r ? q : 0;
+                            lg_min_max(pk, p, k);
+                        }
+                    } else if (z <= -delta) {
+                        below += fixq(fabs(b), sigma, e);
+                    }
+                }
+        }
+        below = lg_sum(below, pk.wsum[0]);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) part[r] = lg_sum(part[r], pk.wsum[r]);
+        if (tid == 0) {
+            sm.tot[buf][0] = (unsigned long long)below;
+            for (int r = 0; r < 3; ++r) sm.tot[buf][r + 1] = (unsigned long long)part[r];
+        }
+        cl.sync();
+        long long t[4] = {0, 0, 0, 0};
+        K mn[3] = {Tr::NONE, Tr::NONE, Tr::NONE}, mx[3] = {0, 0, 0};
+        for (int r = 0; r < C; ++r) {
+            const LgPick<T> *o = cl.map_shared_rank(&pk, r);
+            const unsigned long long *ot = cl.map_shared_rank(&sm.tot[buf][0], r);
+#pragma unroll
+            for (int p = 0; p < 4; ++p) t[p] += (long long)ot[p];
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+                mn[p] = o->kmn[p] < mn[p] ? o->kmn[p] : mn[p];
+                mx[p] = o->kmx[p] > mx[p] ? o->kmx[p] : mx[p];
+            }
+        }
+        buf ^= 1;
+        cl.sync();  // the histograms overlap what the cluster read
+        thr = t[0];
+        int res = dec.cond(thr, lo > CK0);
+        if (res != 0) return LG_SEARCH;
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+            if (res == 0 && mn[p] <= mx[p]) {  // the first part whose last key passes
+                L = thr;
+                thr += t[p + 1];
+                A = mn[p];
+                B = mx[p];
+                res = dec.cond(thr, B >= Tr::KEY0);
+            }
+        if (res == 0) return LG_SEARCH;
+        if (res < 0) return LG_EXACT;
+    }
+    if (!(A <= B) || (listed && dec.cond(L, lo > CK0) != 0)) return LG_SEARCH;
+    if (A == B && dec.cond(thr, A >= Tr::KEY0) == 1) {  // a tie, the only key there
+        key = A;
+        return LG_FOUND;
+    }
+    for (int pass = 0; pass < 6; ++pass) {
+        const K span = B - A;
+        int sh = 0;
+        if (span >= (K)LG_NB)
+            sh = (sizeof(K) == 4 ? 32 - __clz((int)span) : 64 - __clzll((long long)span)) - LG_BITS;
+        for (int b = tid; b < LG_COPIES * LG_NB; b += LG_NT) (&sm.copies[0][0])[b] = 0ull;
+        if (tid == 0) sm.dec.first = LG_NB;
+        __syncthreads();
+        unsigned long long *cp = sm.copies[warp % LG_COPIES];
+        int cur = -1;
+        unsigned long long csum = 0;
+        for (int64_t v = c0 + tid; v < c1; v += LG_UR * LG_NT) {
+            LgRows<float, LG_UR> x;
+            x.load(fj, fk, fj, v, c1);
+            uint32_t hit = 0;
+#pragma unroll
+            for (int g = 0; g < LG_UR; ++g)
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (fabsf(__fmaf_rn(x.a(g, u), rcp_approx(x.b(g, u)), -cen)) < delta)
+                        hit |= 1u << (4 * g + u);
+            for (; hit; hit &= hit - 1) {
+                const int bit = __ffs(hit) - 1;
+                const int64_t i = 4 * (v + (bit >> 2) * LG_NT) + (bit & 3);
+                const T b = xj[i];
+                if (b == T(0)) continue;
+                const K k = Tr::key(Tr::div_rn(xk[i], b));
+                if (k < A || k > B) continue;
+                int e = 0;
+                const unsigned long long q = (unsigned long long)fixq(fabs(b), sigma, e);
+                const int bin = L1L_CHK((int)((k - A) >> sh), LG_NB);
+                if (bin != cur) {
+                    if (cur >= 0) atomicAdd(&cp[cur], csum);
+                    cur = bin;
+                    csum = 0;
+                }
+                csum += q;
+            }
+        }
+        if (cur >= 0) atomicAdd(&cp[cur], csum);
+        __syncthreads();
+        for (int b = tid; b < LG_NB; b += LG_NT) {
+            unsigned long long t = 0;
+#pragma unroll
+            for (int c = 0; c < LG_COPIES; ++c) t += sm.copies[c][b];
+            sm.tot[buf][b] = t;
+        }
+        cl.sync();  // every CTA's totals are complete and visible
+        long long h[LG_BPT], run = 0;
+#pragma unroll
+        for (int u = 0; u < LG_BPT; ++u) {
+            unsigned long long t = 0;
+            for (int r = 0; r < C; ++r)
+                t += cl.map_shared_rank(&sm.tot[buf][0], r)[tid * LG_BPT + u];
+            h[u] = (long long)t;
+            run += h[u];
+        }
+        buf ^= 1;
+        const long long incl = warp_scan_add(run, lane);
+        if (lane == 31) sm.wsum[warp] = incl;
+        __syncthreads();
+        long long acc = L + incl - run;
+        for (int w = 0; w < warp; ++w) acc += sm.wsum[w];
+        // first bin whose test at its last key is true or undecidable
+        int mine = LG_NB, mine_res = 0;
+        long long mine_below = 0;
+#pragma unroll
+        for (int u = 0; u < LG_BPT; ++u) {
+            const int b = tid * LG_BPT + u;
+            const long long below = acc;
+            acc += h[u];
+            if (mine == LG_NB && (K)b <= span >> sh) {
+                const K first = A + ((K)b << sh), in = ((K)1 << sh) - 1;
+                const K last = B - first < in ? B : first + in;
+                const int res = dec.cond(acc, last >= Tr::KEY0);
+                if (res != 0) {
+                    mine = b;
+                    mine_res = res;
+                    mine_below = below;
+                }
+            }
+        }
+        if (mine < LG_NB) atomicMin(&sm.dec.first, mine);
+        __syncthreads();
+        if (mine < LG_NB && mine == sm.dec.first) {
+            sm.dec.sbelow = mine_below;
+            sm.dec.state = mine_res;
+        }
+        __syncthreads();
+        const int first = sm.dec.first;
+        if (first == LG_NB) return LG_SEARCH;
+        const int res = sm.dec.state;
+        L = sm.dec.sbelow;
+        __syncthreads();  // sm.dec is rewritten by the next pass
+        if (res < 0) return LG_EXACT;
+        A += (K)first << sh;
+        if (sh == 0) {
+            key = A;
+            return LG_FOUND;
+        }
+        const K in = ((K)1 << sh) - 1;
+        B = B - A < in ? B : A + in;
+    }
+    return LG_SEARCH;
+}
+
 // The weighted median of a pair by the cluster: LG_FOUND with its key, LG_EXACT
 // where the weights cannot settle it, LG_SEARCH where the descent has to look.
 // Every CTA returns the same.  c0, c1: this CTA's rows in vectors of four.
@@ -356,12 +595,50 @@ __device__ int large_pick(const ScanArgs<T> &a, const ColInfo &ci, int64_t j, in
         a0 = pk.key[max(pk.ia - 1, 0)];
         b0 = pk.key[pk.ib];
     }
+    auto keys = [&](uint32_t klo, uint32_t khi, bool listed, long long L, long long thr) -> int {
+        const Decide dk = dec;  // in memory from here on, as the others
+        int bk = buf;
+        K kk = 0;
+        const int st = large_keys<T>(ci.sigma, dk, fj, fk, xj, xk, c0, c1, klo, khi, listed, L,
+                                     thr, sm, bk, kk);
+        buf = bk;
+        key = kk;
+        return st;
+    };
+    // Five of the samples up to 48 (three deviations of the crossing) either side within
+    // 64 coarse keys: ties or nearly collinear columns, of which the bins below would
+    // hold more rows than their halves sum (512).  Looked at by exact keys instead, those
+    // at the crossing apart from those under and over them.
+    {
+        const int j0 = max(max(pk.ia - 1, pk.j1 - 48), 0), j2 = min(pk.ib, pk.j1 + 48);
+        const int t = j0 + tid;
+        const bool run = t + 4 <= j2 && pk.key[t + 4] < INFINITY &&
+                         akey(pk.key[t + 4]) - akey(pk.key[t]) <= 64u;
+        if (__syncthreads_or(run)) {
+            if (tid == 0) {
+                auto at = [&](int i) { return akey(pk.key[i]); };
+                int e = j2, p = pk.j1, q = pk.j1;
+                while (e > pk.j1 && pk.key[e] == INFINITY) --e;  // x_ijhat = 0
+                while (p > j0 && at(p) - at(p - 1) <= 64u) --p;
+                while (q < e && at(q + 1) - at(q) <= 64u) ++q;
+                pk.klo = sat_sub(at(j0), G + 4);
+                pk.khi = sat_add(at(e), G + 4);
+                pk.clo = max(pk.klo, sat_sub(at(p), G + 4));
+                pk.chi = min(pk.khi, sat_add(at(q), G + 4));
+            }
+            __syncthreads();
+            const int st = keys(pk.klo, pk.khi, false, 0, 0);
+            if (st != LG_SEARCH) return st;
+            __syncthreads();
+        }
+    }
 
     for (int attempt = 0; attempt < 3; ++attempt) {
         // ---- bins: steps of w1, no finer than 16 keys of the largest ratio ----
+        // (or 2^-99, where the whole bracket is 0: sparse columns)
         const float w1 = fmaxf((b0 - a0) * (1.0f / (LG_BINS - 2 * LG_SIDE)),
-                               fmaxf(fabsf(a0), fabsf(b0)) * 0x1p-19f);
-        if (!(w1 > 0x1p-100f && w1 < 0x1p100f)) return LG_SEARCH;
+                               fmaxf(fmaxf(fabsf(a0), fabsf(b0)) * 0x1p-19f, 0x1p-99f));
+        if (!(w1 < 0x1p100f)) return LG_SEARCH;
         const float sc = __frcp_rn(w1);
         const float bm = __fmaf_rn(-a0, sc, Z32 + (float)LG_SIDE);
         constexpr float ZT = Z32 + (float)LG_BINS;
@@ -455,6 +732,8 @@ __device__ int large_pick(const ScanArgs<T> &a, const ColInfo &ci, int64_t j, in
             pk.lcnt = 0;
             pk.kmin = Tr::NONE;
             pk.und = 0;
+            pk.kmn[0] = Tr::NONE;
+            pk.kmx[0] = 0;
         }
         __syncthreads();
         if (ca < 1 || ca >= LG_BINS) {  // missed: further out on that side
@@ -507,10 +786,14 @@ __device__ int large_pick(const ScanArgs<T> &a, const ColInfo &ci, int64_t j, in
                 if (ck < lo) {
                     below_w += q;
                 } else if (ck <= hi) {
-                    const int at = atomicAdd(&pk.lcnt, 1);
+                    // not counted on once the list is full: ties would queue for the count
+                    const int at = *(volatile int *)&pk.lcnt > LG_ROWS ? LG_ROWS
+                                                                       : atomicAdd(&pk.lcnt, 1);
                     if (at < LG_ROWS) {
                         pk.lkey[at] = fkey;
                         pk.lq[at] = q;
+                    } else {
+                        lg_min_max(pk, 0, fkey);
                     }
                 }
             }
@@ -545,9 +828,10 @@ __device__ int large_pick(const ScanArgs<T> &a, const ColInfo &ci, int64_t j, in
             }
             c += cr;
         }
-        const long long W = pk.fw;
+        const long long W = pk.fw, thr = pk.fl + W;
         cl.sync();  // the lists are free again
-        if (c > LG_ROWS || in_w != W || dec.cond(L, lo > CK0) != 0) return LG_SEARCH;
+        if (in_w != W || dec.cond(L, lo > CK0) != 0) return LG_SEARCH;
+        if (c > LG_ROWS) return keys(lo, hi, true, L, thr);
         if (lo <= CK0 && CK0 <= hi) {  // the penalty point; lambda sits in the test
             if (tid == 0) {
                 pk.akey[c] = Tr::KEY0;
