@@ -564,8 +564,15 @@ __device__ void build_unit(int64_t m, int64_t u, int i, const int64_t *__restric
     }
     __syncthreads();
     // prefix sums, one piece per distinct lambda (the last change at that
-    // lambda closes it)
+    // lambda closes it) that is another line than the piece before: a step between
+    // values that differ in the last place can leave intercept and slope as they are
+    struct Line {
+        double I, s;
+    };
+    Line *line = reinterpret_cast<Line *>(sm.a);  // the chunk's, in order
+    static_assert(sizeof(sm.a) >= ZT * sizeof(Line), "a line per thread");
     int64_t cI = 0, cs = 0, cw = 0;
+    Line held{0.0, 0.0};  // of the last piece of the chunks before
     for (int64_t e0 = 0; e0 < cnt; e0 += ZT) {
         const int64_t e = e0 + tid;
         Piece p{};
@@ -576,15 +583,25 @@ __device__ void build_unit(int64_t m, int64_t u, int i, const int64_t *__restric
                                       __double_as_longlong(p.lam);
         }
         const int64_t x = __double_as_longlong(p.I), y = __double_as_longlong(p.s);
-        int64_t tI, ts, tw;
+        int64_t tI, ts, tl, tw;
         const int64_t eI = block_excl_scan(x, smi, tI);
         const int64_t es = block_excl_scan(y, smi, ts);
-        const int64_t ew = block_excl_scan(end ? 1 : 0, smi, tw);
+        const int64_t el = block_excl_scan(end ? 1 : 0, smi, tl);
         if (end) {
             p.I = unfix(cI + eI + x, shI);
             p.s = unfix(cs + es + y, shs);
-            out[cw + ew] = p;
+            line[el] = Line{p.I, p.s};
         }
+        __syncthreads();
+        bool keep = end;
+        if (end && (cw != 0 || el != 0)) {
+            const Line q = el != 0 ? line[el - 1] : held;
+            keep = q.I != p.I || q.s != p.s;
+        }
+        if (tl != 0) held = line[tl - 1];
+        const int64_t ew = block_excl_scan(keep ? 1 : 0, smi, tw);
+        if (keep) out[cw + ew] = p;
+        __syncthreads();
         cI += tI;
         cs += ts;
         cw += tw;
