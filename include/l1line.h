@@ -245,7 +245,9 @@ int l1line_path_write_f64(const double *X, int64_t n, int64_t m, const int64_t *
  * double sums of the residuals (relative error ~ entries x 2^-53); values and
  * slopes agreeing to a relative 1e-12 are taken as equal.  The workspace
  * (l1line_solution_path_workspace_bytes, 256-byte aligned) starts with a
- * status word that l1line_status reads.
+ * status word that l1line_status reads: L1L_ERR_NONFINITE when a residual or
+ * v is not finite, or a pair's residuals do not lie between its first and its
+ * last (as those of the calls above do).
  */
 size_t l1line_solution_path_workspace_bytes(int64_t m, int64_t entries);
 int l1line_solution_path_f32(int64_t m, const int64_t *offsets, const double *lambda,

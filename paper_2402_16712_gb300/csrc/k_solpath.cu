@@ -80,10 +80,11 @@ struct SolWs {
     Piece *buf[3];    // entries + NG m pieces each
 };
 
-// The largest sh with b 2^sh < 2^61 (b >= 0).
-__device__ __forceinline__ int fix_shift(double b) {
+// The largest sh with b 2^(e + sh) < 2^61 (b >= 0; as for 2^-1022 where b is less: the
+// mantissa of a double is shifted by 9 bits at most).
+__device__ __forceinline__ int fix_shift(double b, int e) {
     if (!(b > 0.0) || isinf(b)) return 0;
-    return 60 - ilog2_pos(b);
+    return 60 - e - max(ilog2_pos(b), -1022);
 }
 
 // The largest breakpoint of all, and the fixed-point scales of jhat: a pair's
@@ -95,33 +96,43 @@ __global__ void __launch_bounds__(256) k_zrange(int64_t m, const int64_t *__rest
                                                 const T *__restrict__ val,
                                                 const double *__restrict__ res, SolWs w) {
     const int64_t j = blockIdx.x;
-    double bI = 0.0, bs = 0.0;
-    unsigned long long mx = 0;
-    for (int64_t k = threadIdx.x; k < m; k += blockDim.x) {
-        const int64_t o = off[j * m + k], l = o + len[j * m + k] - 1;
-        bI += fabs(res[o]) + fabs(res[l]);
-        bs += fabs((double)val[o]) + fabs((double)val[l]);
-        mx = max(mx, (unsigned long long)__double_as_longlong(lam[l]));
-    }
-    bI = warp_sum_f64(bI);
-    bs = warp_sum_f64(bs);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
     __shared__ double sm[2][8];
-    if ((threadIdx.x & 31) == 0) {
-        sm[0][threadIdx.x >> 5] = bI;
-        sm[1][threadIdx.x >> 5] = bs;
-        if (mx != 0) atomicMax(&w.h->lmax, mx);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int q = 1; q < 8; ++q) {
+    unsigned long long mx = 0;
+    // both bounds; scaled down where they overflow, which the values need not
+    for (int e = 0;; e = 64) {
+        auto term = [&](double x) { return e != 0 ? fabs(x) * 0x1p-64 : fabs(x); };
+        double bI = 0.0, bs = 0.0;
+        for (int64_t k = threadIdx.x; k < m; k += blockDim.x) {
+            const int64_t o = off[j * m + k], l = o + len[j * m + k] - 1;
+            bI += term(res[o]) + term(res[l]);
+            bs += term((double)val[o]) + term((double)val[l]);
+            mx = max(mx, (unsigned long long)__double_as_longlong(lam[l]));
+        }
+        bI = warp_sum_f64(bI);
+        bs = warp_sum_f64(bs);
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0) {
+            sm[0][threadIdx.x >> 5] = bI;
+            sm[1][threadIdx.x >> 5] = bs;
+        }
+        __syncthreads();
+        bI = bs = 0.0;
+        for (int q = 0; q < 8; ++q) {
             bI += sm[0][q];
             bs += sm[1][q];
         }
-        w.shI[j] = fix_shift(bI);
-        w.shs[j] = fix_shift(bs);
+        const bool finite = bI < INFINITY && bs < INFINITY;  // NaN: not
+        if (!finite && e == 0) continue;
+        if (threadIdx.x == 0) {
+            if (!finite) atomicOr(&w.h->status, (uint32_t)ST_NONFINITE);
+            w.shI[j] = fix_shift(bI, e);
+            w.shs[j] = fix_shift(bs, e);
+        }
+        break;
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+    if ((threadIdx.x & 31) == 0 && mx != 0) atomicMax(&w.h->lmax, mx);
 }
 
 // The grid: squares, since most breakpoints lie near 0 (a pair's last one is
@@ -342,14 +353,16 @@ __global__ void __launch_bounds__(ZL) k_zlist(int64_t m, SolWs w) {
 // x 2^sh rounded to an integer (half up), |x| 2^sh < 2^62.  Sums of these are
 // exact, so a function's intercept at any piece is the rounded sum of its
 // pairs' current entries, whatever the order, to within m 2^-62 of the bound.
-__device__ __forceinline__ int64_t fix_rn(double x, int sh) {
+// bad: x is above the bound or not finite (not a path of l1line_path_write).
+__device__ __forceinline__ int64_t fix_rn(double x, int sh, bool &bad) {
     const uint64_t u = (uint64_t)__double_as_longlong(x);
     const int be = (int)((u >> 52) & 0x7FF);
     uint64_t f = u & 0xFFFFFFFFFFFFFull;
     if (be) f |= 0x10000000000000ull;
     const int s = (be ? be : 1) - 1075 + sh;
+    bad |= s > 9 && f != 0;
     if (s >= 0)
-        f = s > 9 ? 0 : f << s;  // s > 9: above the bound (not a finite input)
+        f = s > 9 ? 0 : f << s;
     else if (s > -60)
         f = (f + (1ull << (-s - 1))) >> -s;
     else
@@ -427,6 +440,7 @@ __device__ void build_unit(int64_t m, int64_t u, int i, const int64_t *__restric
     };
     __syncthreads();
     // the entry of each pair holding at g_i, and the changes inside the interval
+    bool bad = false;
     int64_t I0 = 0, s0 = 0, cnt = 1;  // element 0: the piece holding at g_i
     for (int64_t kb = 0; kb < m; kb += ZT) {
         const int64_t k = kb + tid;
@@ -452,8 +466,8 @@ __device__ void build_unit(int64_t m, int64_t u, int i, const int64_t *__restric
                 else
                     top = mid;
             }
-            I0 += fix_rn(res[o + lo - 1], shI);
-            s0 += fix_rn(fabs((double)val[o + lo - 1]), shs);
+            I0 += fix_rn(res[o + lo - 1], shI, bad);
+            s0 += fix_rn(fabs((double)val[o + lo - 1]), shs, bad);
         }
         int64_t tot;
         const int64_t dst = cnt + block_excl_scan((int64_t)max(hi - lo, 0), smi, tot);
@@ -551,8 +565,9 @@ __device__ void build_unit(int64_t m, int64_t u, int i, const int64_t *__restric
         }
         int64_t dI = I0, ds = s0;
         if (x.src >= 0) {
-            dI = fix_rn(res[x.src], shI) - fix_rn(res[x.src - 1], shI);
-            ds = fix_rn(fabs((double)val[x.src]), shs) - fix_rn(fabs((double)val[x.src - 1]), shs);
+            dI = fix_rn(res[x.src], shI, bad) - fix_rn(res[x.src - 1], shI, bad);
+            ds = fix_rn(fabs((double)val[x.src]), shs, bad) -
+                 fix_rn(fabs((double)val[x.src - 1]), shs, bad);
         }
         Piece p;
         p.lam = __longlong_as_double(x.key);
@@ -562,6 +577,7 @@ __device__ void build_unit(int64_t m, int64_t u, int i, const int64_t *__restric
         p.pad = 0;
         sorted[L1L_CHK(pos, room)] = p;
     }
+    if (bad) atomicOr(&w.h->status, (uint32_t)ST_NONFINITE);
     __syncthreads();
     // prefix sums, one piece per distinct lambda (the last change at that
     // lambda closes it) that is another line than the piece before: a step between
