@@ -447,12 +447,11 @@ int path_write_impl(const T *X, int64_t n, int64_t m, const int64_t *offsets, do
 template <typename T>
 int proposer_features(const T *X, int64_t n, int64_t m, double lambda, Scan<T> &c,
                       const ProposedLayout &P, float *raw, float *stdz) {
-    if (launch_colfeat<T>(c.a.Xt, c.a.ldn, n, m, raw, c.st, c.launches) != cudaSuccess)
-        return L1L_ERR_CUDA;
     float *rho = reinterpret_cast<float *>(c.base + P.rho);
     int32_t *rows = reinterpret_cast<int32_t *>(c.base + P.rows);
     T *xr = reinterpret_cast<T *>(c.base + P.xr);
-    if (launch_heavy_rows<T>(X, c.a.Xt, c.a.ldn, n, m, P.R, rho, rows, xr, c.st, c.launches) != cudaSuccess)
+    if (launch_colfeat_rows<T>(X, c.a.Xt, c.a.ldn, n, m, P.R, raw, rho, rows, xr, c.st,
+                               c.launches) != cudaSuccess)
         return L1L_ERR_CUDA;
     Scan<T> p;
     L1L_TRY(scan_setup<T>(xr, P.R, m, &lambda, 1, nullptr, nullptr, nullptr, c.base + P.pws,

@@ -272,7 +272,8 @@ constexpr int MAX_LAMBDA_PER_LAUNCH = 256;
 // the stream be placed while its own last CTAs run (next_may_start, first
 // thing), and waits for the end of the one before it, whose writes it then
 // sees, before it touches memory (wait_for_previous; no wait where it was
-// launched without the attribute).
+// launched without the attribute).  One kernel waits last: k_rownorm, which runs
+// beside the ordinary launch ahead of it (launch_colfeat_rows).
 __device__ __forceinline__ void next_may_start() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

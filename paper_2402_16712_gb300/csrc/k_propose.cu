@@ -742,17 +742,6 @@ size_t mlp_smem_bytes() { return sizeof(MlpSmemBwd); }
 
 L1L_CHECKS_READER(l1l_checks_propose)
 
-template <typename T>
-cudaError_t launch_colfeat(const T *Xt, int64_t ldn, int64_t n, int64_t m, float *raw,
-                           cudaStream_t st, int &launches) {
-    const size_t smem = (size_t)n * 4;
-    cudaError_t e = ensure_smem(reinterpret_cast<const void *>(k_colfeat<T>), smem);
-    if (e != cudaSuccess) return e;
-    k_colfeat<T><<<(unsigned)m, NT, smem, st>>>(Xt, ldn, (int)n, raw);
-    launches++;
-    return cudaGetLastError();
-}
-
 cudaError_t launch_featstd(const float *raw, int64_t m, float *stdz, cudaStream_t st,
                            int &launches) {
     k_featstd<<<NF, NT, 0, st>>>(raw, m, stdz);
@@ -761,11 +750,18 @@ cudaError_t launch_featstd(const float *raw, int64_t m, float *stdz, cudaStream_
 }
 
 template <typename T>
-cudaError_t launch_heavy_rows(const T *X, const T *Xt, int64_t ldn, int64_t n, int64_t m,
-                              int64_t R, float *rho, int32_t *rows, T *Y, cudaStream_t st,
-                              int &launches) {
-    // directly after launch_colfeat, which it overlaps
-    cudaError_t e = launch_after(k_rownorm<T>, dim3((unsigned)((n + 31) / 32)), dim3(32), 0, st, Xt,
+cudaError_t launch_colfeat_rows(const T *X, const T *Xt, int64_t ldn, int64_t n, int64_t m,
+                                int64_t R, float *raw, float *rho, int32_t *rows, T *Y,
+                                cudaStream_t st, int &launches) {
+    const size_t smem = (size_t)n * 4;
+    cudaError_t e = ensure_smem(reinterpret_cast<const void *>(k_colfeat<T>), smem);
+    if (e != cudaSuccess) return e;
+    // an ordinary launch: it starts when the staging has ended, and k_rownorm, which reads
+    // the staged copy without a wait of its own, starts when this has started
+    k_colfeat<T><<<(unsigned)m, NT, smem, st>>>(Xt, ldn, (int)n, raw);
+    launches++;
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_after(k_rownorm<T>, dim3((unsigned)((n + 31) / 32)), dim3(32), 0, st, Xt,
                                  ldn, n, m, rho);
     launches++;
     if (e != cudaSuccess) return e;
@@ -858,15 +854,11 @@ cudaError_t launch_topk(const float *score, int64_t m, int K, int32_t *out, cuda
     return cudaGetLastError();
 }
 
-template cudaError_t launch_colfeat<float>(const float *, int64_t, int64_t, int64_t, float *,
-                                           cudaStream_t, int &);
-template cudaError_t launch_colfeat<double>(const double *, int64_t, int64_t, int64_t, float *,
-                                            cudaStream_t, int &);
-template cudaError_t launch_heavy_rows<float>(const float *, const float *, int64_t, int64_t,
-                                              int64_t, int64_t, float *, int32_t *, float *,
-                                              cudaStream_t, int &);
-template cudaError_t launch_heavy_rows<double>(const double *, const double *, int64_t, int64_t,
-                                               int64_t, int64_t, float *, int32_t *, double *,
-                                               cudaStream_t, int &);
+template cudaError_t launch_colfeat_rows<float>(const float *, const float *, int64_t, int64_t,
+                                                int64_t, int64_t, float *, float *, int32_t *,
+                                                float *, cudaStream_t, int &);
+template cudaError_t launch_colfeat_rows<double>(const double *, const double *, int64_t, int64_t,
+                                                 int64_t, int64_t, float *, float *, int32_t *,
+                                                 double *, cudaStream_t, int &);
 
 }  // namespace l1l

@@ -131,19 +131,16 @@ cudaError_t launch_deflate(const T *X, T *Y, int64_t n, int64_t m, const int32_t
 // ---- learned jhat proposer (k_propose.cu) ----
 constexpr int MLP_TILE = 64;  // samples per CTA of the network kernels
 size_t mlp_smem_bytes();
-// Column features 0..2 of the staged copy into raw [m][L1L_MLP_FEATURES].
-template <typename T>
-cudaError_t launch_colfeat(const T *Xt, int64_t ldn, int64_t n, int64_t m, float *raw,
-                           cudaStream_t st, int &launches);
 // Standardises every feature column of raw over the m columns.
 cudaError_t launch_featstd(const float *raw, int64_t m, float *stdz, cudaStream_t st,
                            int &launches);
-// The R rows of largest l1 norm of the row-major X (rho: row norms [n],
-// rows: their indices in ascending order [R]) copied into Y (R x m).
+// Column features 0..2 of the staged copy into raw [m][L1L_MLP_FEATURES], and beside that
+// the R rows of largest l1 norm of the row-major X (rho: row norms [n], rows: their indices
+// in ascending order [R]) copied into Y (R x m).
 template <typename T>
-cudaError_t launch_heavy_rows(const T *X, const T *Xt, int64_t ldn, int64_t n, int64_t m,
-                              int64_t R, float *rho, int32_t *rows, T *Y, cudaStream_t st,
-                              int &launches);
+cudaError_t launch_colfeat_rows(const T *X, const T *Xt, int64_t ldn, int64_t n, int64_t m,
+                                int64_t R, float *raw, float *rho, int32_t *rows, T *Y,
+                                cudaStream_t st, int &launches);
 // *dst |= *src (device status words), one thread.
 cudaError_t launch_status_or(uint32_t *dst, const uint32_t *src, cudaStream_t st, int &launches);
 // raw[j][c] = z[j] for j < m.
