@@ -161,7 +161,7 @@ template <typename T> struct ListedPair {
     __device__ __forceinline__ ListedPair(const ScanArgs<T> &a, const SlowEntry &en)
         : j(L1L_CHK(en.j, (int32_t)a.m)), k(L1L_CHK(en.k, (int32_t)a.m)), xk(a.Xt + k * a.ldn),
           xj(a.Xt + j * a.ldn), xf(a.Xf + k * a.ldn),
-          col{a.Xf + j * a.ldn, xj, a.ci[j].sigma} {}
+          col(a.Xf + j * a.ldn, xj, a.ci[j].sigma) {}
     __device__ __forceinline__ int64_t at(const ScanArgs<T> &a, int t) const {
         return L1L_CHK(((int64_t)t * a.m + j) * a.m + k, (int64_t)a.n_lambda * a.m * a.m);
     }

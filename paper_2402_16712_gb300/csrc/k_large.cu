@@ -155,12 +155,6 @@ template <typename T> struct LgSmem {
     LgDecision<K> dec;
 };
 
-__device__ __forceinline__ float rcp_approx(float x) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 // floor(w 2^sigma) as hi 2^b + lo.  Float: w 2^(sigma - b) < 2^23, so adding
 // 2^23 rounding down leaves its floor in the mantissa, and the remainder, exact,
 // the same way.  up: 2^(sigma - b), dn: 2^b.

@@ -19,27 +19,41 @@
 // that all lanes divide) and three shared-memory words per row inside.  2000 x 64 of
 // small integers, double, where such a pair went to the exact kernel (64 bisection
 // steps with all rows): 47 -> 0.16 ms; near-multiples (spread 1e-5): 49 -> 0.25 ms.
+// A few listed pairs cost the latency of one warp (at 1/4 instruction per cycle, those
+// fetched for the first time more): 2000 rows 13 us, 22 with a rounded reciprocal, the
+// weight's bits taken apart for every row and x_ijhat loaded where it is used.
 #pragma once
 
 namespace l1l {
 
-// Column jhat for narrow(), from the column copies: 1/x_ijhat of four rows from i on
-// (NaN: x_ijhat = 0), x_ijhat and the 64-bit weight of row i.
+// Column jhat for narrow(), from the column copies: x_ijhat as float and as it is, and
+// its 64-bit weight, floor(|b| 2^sigma).  Float: the scaling by a power of two, in two
+// steps, is exact where the weight is not 0.
 template <typename T> struct ReadCol {
     const float *xf;
     const T *x;
     int sigma;
-    __device__ __forceinline__ float4 inv(int i) const {
-        const float4 b = __ldg(reinterpret_cast<const float4 *>(xf + i));
-        auto one = [](float v) { return v != 0.0f ? __frcp_rn(v) : __int_as_float(0x7FFFFFFF); };
-        return make_float4(one(b.x), one(b.y), one(b.z), one(b.w));
+    float s0, s1;  // 2^sigma in two factors
+    __device__ __forceinline__ ReadCol(const float *xf_, const T *x_, int sigma_)
+        : xf(xf_), x(x_), sigma(sigma_) {
+        s0 = __int_as_float((127 + sigma / 2) << 23);
+        s1 = __int_as_float((127 + sigma - sigma / 2) << 23);
     }
     __device__ __forceinline__ T at(int i) const { return __ldg(x + i); }
-    __device__ __forceinline__ unsigned long long q(int i) const {
-        int e = 0;
-        return (unsigned long long)fixq(__ldg(x + i), sigma, e);
+    __device__ __forceinline__ unsigned long long weight(T b) const {
+        if constexpr (sizeof(T) == 4) {
+            return __float2ull_rz(fabsf(b) * s0 * s1);
+        } else {
+            int e = 0;
+            return (unsigned long long)fixq(b, sigma, e);
+        }
     }
 };
+__device__ __forceinline__ float rcp_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
 
 constexpr int NARROW_PEND = 64;  // rows queued for the division
 
@@ -95,6 +109,7 @@ __device__ int narrow(const float *__restrict__ xf, const T *__restrict__ xk,
         const float delta = (0.5f * vb - 0.5f * va) * (1.0f + 0x1p-20f) +
                             0x1p-21f * fmaxf(fabsf(va), fabsf(vb)) + 0x1p-148f;
         if (!(delta < 0x1p126f) || !(fabsf(cen) < 0x1p126f) || !(A <= B)) return SEL_W64;
+        int c = 0;  // rows listed
         const K span = B - A;
         int sh = 0;
         if (span >= 32) {
@@ -110,13 +125,20 @@ __device__ int narrow(const float *__restrict__ xf, const T *__restrict__ xk,
             sh = 0;
             base = A + ((span - 31) >> 1);
         }
-        bins.mn[lane] = Tr::NONE;
-        bins.mx[lane] = 0;
-        bins.w[lane] = 0;
-        bins.cnt[lane] = 0;
+        {
+            // the penalty point is there from the start
+            const bool zero = A <= Tr::KEY0 && Tr::KEY0 <= B;
+            const int at =
+                list || Tr::KEY0 <= base ? 0 : (int)min((Tr::KEY0 - base) >> sh, (K)31);
+            bins.mn[lane] = zero && lane == at ? Tr::KEY0 : Tr::NONE;
+            bins.mx[lane] = zero && lane == at ? Tr::KEY0 : 0;
+            bins.w[lane] = 0;
+            bins.cnt[lane] = zero && lane == at ? 1 : 0;
+            c = zero ? 1 : 0;
+        }
         __syncwarp();
         int64_t below = 0;
-        int c = 0, np = 0;  // rows listed, rows queued
+        int np = 0;  // rows queued
         // a lane holds back the sums of the bin it met last: ties meet one bin
         int cur = -1;
         W csum = 0;
@@ -158,64 +180,75 @@ __device__ int narrow(const float *__restrict__ xf, const T *__restrict__ xk,
             W q = 0;
             if (on) {
                 const T x = __ldg(xk + i);
-                key = x == T(0) ? Tr::KEY0 : Tr::key(Tr::div_rn(x, col.at(i)));
-                q = col.q(i);
+                const T b = col.at(i);
+                key = x == T(0) ? Tr::KEY0 : Tr::key(Tr::div_rn(x, b));
+                q = col.weight(b);
             }
             if (pass == 0 && key < A) below += (int64_t)q;
             put(on && key >= A && key <= B, key, q);
         };
-        auto flush = [&](int cnt) {  // the queue's first 32 rows (fewer at the end)
-            const bool on = lane < cnt;
-            take(on, L1L_CHK(on ? (int)bins.pend[lane] : 0, ng * 128));
-        };
-        put(lane == 0 && A <= Tr::KEY0 && Tr::KEY0 <= B, Tr::KEY0, 0);  // the penalty point
-        for (int g0 = 0; g0 < ng; g0 += 8) {  // 8 groups: a bit per row of the lane
-            const int ge = min(ng, g0 + 8);
-            uint32_t mask = 0;
-            float4 xn = __ldg(reinterpret_cast<const float4 *>(xf) + g0 * 32 + lane);
-            for (int g = g0; g < ge; ++g) {
-                const float4 x4 = xn;
-                if (g + 1 < ge) xn = __ldg(reinterpret_cast<const float4 *>(xf) + (g + 1) * 32 + lane);
-                const int i0 = L1L_CHK(g * 128 + 4 * lane, ng * 128);
-                const float4 v4 = col.inv(i0);
-                // NaN (x_ijhat = 0, a padding row): neither inside nor below
-                const float z[4] = {fmaf(x4.x, v4.x, -cen), fmaf(x4.y, v4.y, -cen),
-                                    fmaf(x4.z, v4.z, -cen), fmaf(x4.w, v4.w, -cen)};
-                uint32_t f = 0;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (fabsf(z[u]) < delta) f |= 1u << u;
-                    if (pass == 0 && z[u] <= -delta) below += (int64_t)col.q(i0 + u);
-                }
-                if (__popc(__ballot_sync(FULL, f == 15u)) >= 24) {  // most rows: as they lie
-#pragma unroll 1
-                    for (int u = 0; u < 4; ++u) take((f >> u) & 1u, i0 + u);
-                    f = 0;
-                }
-                mask |= f << (4 * (g - g0));
+        float4 an = __ldg(reinterpret_cast<const float4 *>(xf) + lane);
+        float4 bn = __ldg(reinterpret_cast<const float4 *>(col.xf) + lane);
+        uint32_t mask = 0;  // 8 groups: a bit per row of the lane
+        for (int g = 0; g < ng; ++g) {
+            const float4 a4 = an, b4 = bn;
+            const int i0 = L1L_CHK(g * 128 + 4 * lane, ng * 128);
+            if (g + 1 < ng) {
+                an = __ldg(reinterpret_cast<const float4 *>(xf + 128 + i0));
+                bn = __ldg(reinterpret_cast<const float4 *>(col.xf + 128 + i0));
             }
-            unsigned m;
-            while ((m = __ballot_sync(FULL, mask != 0)) != 0) {
+            const float b[4] = {b4.x, b4.y, b4.z, b4.w};
+            // x_ijhat = 0 (a padding row): infinite or NaN; neither inside nor, with its
+            // weight of 0, of account below
+            const float z[4] = {fmaf(a4.x, rcp_approx(b4.x), -cen), fmaf(a4.y, rcp_approx(b4.y), -cen),
+                                fmaf(a4.z, rcp_approx(b4.z), -cen), fmaf(a4.w, rcp_approx(b4.w), -cen)};
+            uint32_t f = 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (fabsf(z[u]) < delta) f |= 1u << u;
+                if (pass == 0) {
+                    T w;
+                    if constexpr (sizeof(T) == 4)
+                        w = b[u];
+                    else
+                        w = z[u] <= -delta ? col.at(i0 + u) : 0.0;
+                    const int64_t q = (int64_t)col.weight(w);
+                    below += z[u] <= -delta ? q : 0;
+                }
+            }
+            if (__popc(__ballot_sync(FULL, f == 15u)) >= 24) {  // most rows: as they lie
+#pragma unroll 1
+                for (int u = 0; u < 4; ++u) take((f >> u) & 1u, i0 + u);
+                f = 0;
+            }
+            mask |= f << (4 * (g & 7));
+            const bool end = g == ng - 1;
+            if ((g & 7) != 7 && !end) continue;
+            // the others by way of the queue, 32 at a time
+            for (;;) {
+                const unsigned m = __ballot_sync(FULL, mask != 0);
                 if (mask != 0) {
                     const int bit = __ffs(mask) - 1;
                     mask &= mask - 1;
                     bins.pend[L1L_CHK(np + __popc(m & ((1u << lane) - 1u)), NARROW_PEND)] =
-                        (uint16_t)((g0 + (bit >> 2)) * 128 + 4 * lane + (bit & 3));
+                        (uint16_t)(((g & ~7) + (bit >> 2)) * 128 + 4 * lane + (bit & 3));
                 }
                 np += __popc(m);
                 __syncwarp();
-                if (np >= 32) {
-                    flush(32);
+                if (np >= 32 || (end && m == 0 && np > 0)) {
+                    const bool on = lane < np;
+                    take(on, L1L_CHK(on ? (int)bins.pend[lane] : 0, ng * 128));
                     __syncwarp();
                     const uint16_t up = bins.pend[32 + lane];
                     __syncwarp();
                     bins.pend[lane] = up;
-                    np -= 32;
+                    np = max(np - 32, 0);
                     __syncwarp();
                 }
+                if (m == 0) break;
             }
         }
-        if (np > 0) flush(np);
+        __syncwarp();
         // what the lanes hold: a bin of many lanes is summed across them first (64-bit
         // atomics in shared memory take their turns)
         if (const unsigned on = __ballot_sync(FULL, cur >= 0)) {
