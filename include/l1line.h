@@ -209,11 +209,11 @@ int l1line_fit_subset_f64(const double *X, int64_t n, int64_t m, const double *l
  * input dtype), both of at least offsets[m*m] entries, and out_len (DEVICE
  * int32 [m*m], the number of entries each pair used).  out_resid (DEVICE
  * double, same size, or NULL) receives each entry's residual
- * sum_i |x_ik - v x_ijhat| (double sums), so that on the entry's lambda
+ * sum_i |x_ik - v x_ijhat|, accumulated in double, so that on the entry's lambda
  * interval the pair's term of z_jhat is out_resid + lambda |out_v|.
  *
  * n is limited by the path kernels' shared memory (one staged column and
- * eight 256-entry lists per CTA): l1line_path_max_rows(dtype) returns the
+ * its warps' lists, the shortest near the limit, per CTA): l1line_path_max_rows(dtype) returns the
  * largest n; larger n make l1line_path_workspace_bytes return 0 and the
  * calls return L1L_ERR_UNSUPPORTED.
  */
@@ -465,12 +465,12 @@ int64_t l1line_check_hits(int reset, int *line);
  *                for up to 16 resident warps, 80 for 17-24 (CTAs of at most
  *                8 warps; 17-24 resident warps in larger CTAs is not a plan),
  *                64 for 25-32 (planner: the most resident warps whose
- *                candidate lists fit; on a tie the fewer CTAs)
+ *                column arrays and histograms fit; on a tie the fewer CTAs)
  *   kchunk       k per CTA of single-instance calls (the batched call always
  *                gives a CTA a whole column jhat)
- *   d0           half-width, in positions of the 64 weight-proportional
- *                samples of column jhat, of the first bracket around the
- *                weighted median, 1..24 (planner: 6)
+ *   d0           half-width, in positions of the 32 sampled rows (every
+ *                second of column jhat's 64 weight-proportional ones), of the
+ *                first bracket around the weighted median, 1..24 (planner: 6)
  *   batch_classes  size classes of a batched call, 1..3: the instances,
  *                ordered by n, are cut into that many runs (where the
  *                planner's occupancy model places the cuts), each run
@@ -484,8 +484,9 @@ int64_t l1line_check_hits(int reset, int *line);
  *                for float input global only when that admits more resident
  *                warps; l1line_plan reports 1 or 2)
  * l1line_set_tuning applies to the later calls of the calling thread (NULL
- * restores the planner); a tuning whose candidate lists do not fit shared
- * memory makes those calls return L1L_ERR_UNSUPPORTED.  l1line_plan reports
+ * restores the planner); a tuning whose column arrays and histograms, and for
+ * a d0 of its own the room that goes with it, do not fit shared memory makes
+ * those calls return L1L_ERR_UNSUPPORTED.  l1line_plan reports
  * the plan such a call would use for nj scored jhat (nj = m for a full scan)
  * on the current device.
  */

@@ -428,7 +428,7 @@ int path_write_impl(const T *X, int64_t n, int64_t m, const int64_t *offsets, do
                        reinterpret_cast<const ColInfo *>(base + P.L.colinfo), n, m, P.L.ldn,
                        reinterpret_cast<const T *>(base + P.L.v_all),
                        const_cast<int64_t *>(offsets), nullptr, out_lam, out_v, out_res,
-                       // the count call's objectives have served their purpose
+                       // the objectives' place: no call of the path computes any
                        reinterpret_cast<float *>(base + P.L.z_all), out_len,
                        reinterpret_cast<int32_t *>(base + P.big),
                        reinterpret_cast<uint32_t *>(base + P.big_count), base + P.scratch,

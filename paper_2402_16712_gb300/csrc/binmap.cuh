@@ -1,6 +1,7 @@
-// binmap.cuh -- the bins of the exact histogram over a level-0 bracket of
-// coarse keys (host and device code, so that a host test can check the
-// layout).
+// binmap.cuh -- the bins of an exact histogram over a bracket of coarse keys
+// (host and device code).  No kernel includes it: the selection's bins are equal
+// steps of the ratio (select32.cuh) or of the key (narrow.cuh).  The layout stays,
+// with its host test, as the reference for bins that are uniform in the key.
 #pragma once
 #include <cstdint>
 

@@ -252,18 +252,19 @@ template <typename T> struct ScanArgs {
     const int32_t *jlist;  // device list of the jhat to score (nullptr: all m)
     int64_t nj;            // entries of jlist (m when jlist is nullptr)
     int d0;                // first-bracket half-width of the selection, sample positions
-    // medians only: s and z are not needed (the penalty paths).  Last, in what was
+    // medians only: s and z are not needed (the penalty paths).  Float leaves the
+    // residual pass out, the double kernels compute it all the same.  Last, in what was
     // padding: ahead of `inst` it moved the kernels' parameters, and the double
     // pair kernel took 3% longer (2000 x 2000: 19.2 -> 19.8 ms)
     int v_only;
 };
 
-// Default first-bracket half-width (of NSAMP = 64 weight-proportional samples).
-// +-6 samples keep ~15-20% of the rows as candidates and rarely miss the
-// median; narrower brackets (d0 = 4) are faster when the weights are not
-// concentrated in few rows (5% outliers) but miss often when they are (20%
-// outlier rows holding most of the weight), so the narrower choice is left to
-// the autotuner, which measures it per shape.
+// Default first-bracket half-width, in positions of the 32 sampled rows (every second
+// of NSAMP = 64 weight-proportional ones): +-6 of them bracket ~37% of the weight and
+// rarely miss the median.  A narrower bracket gives finer bins and fewer candidates
+// when the weights are not concentrated in few rows (5% outliers) but misses often
+// when they are (20% outlier rows holding most of the weight), and a miss costs the
+// passes again, so that choice is left to the autotuner, which measures it per shape.
 constexpr int D0_DEFAULT = 6;
 
 constexpr int MAX_LAMBDA_PER_LAUNCH = 256;

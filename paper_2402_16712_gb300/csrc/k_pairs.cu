@@ -70,8 +70,9 @@ static size_t list_bytes(int64_t slots) {
     return std::max(al16(slots * 8) + 256, al16(slots * 4) + al16(slots * 2) + HIST_WORDS * 4);
 }
 
-// The limit on n is a fixed one (20,608 float, 16,000 double): the rows whose
-// column arrays and one warp with a full list fit a CTA.
+// The limit on n is a fixed one (20,608 rows, of either type: column x_ijhat may stay
+// in global memory): the rows whose other column arrays and one warp with a full list
+// fit a CTA.
 template <typename T> int64_t max_rows_pairs() {
     const size_t budget = 227 * 1024;
     int64_t n = ROW_PAD;
@@ -110,10 +111,10 @@ static PairPlan plan_placement(int64_t npad, bool cs, int d0, const Tune &tune) 
     // Over 1-3 CTAs per SM and 1-16 warps per CTA (or the caller's choice),
     // up to 32 resident warps in one of the launch shapes (pair_shape), keep
     // the plan with the most resident warps that fits 228 KB of shared memory
-    // (1 KB reserved per CTA, and the static arrays: with 1 KB allowed for
-    // these, 7296 to 7552 float rows and 10,880 to 11,392 double ones got plans
-    // of two CTAs of which one fitted, 7296 x 512 3.9 ms, 2.9 now); on a tie the fewer,
-    // larger CTAs (column jhat staged fewer times).
+    // (1 KB reserved per CTA, and the static arrays: with 1 KB allowed for these,
+    // 7296 to 7552 float rows and 10,880 to 11,392 double ones got plans of two CTAs
+    // of which one fitted, 7296 x 512 3.9 ms, 2.9 now); on a tie the fewer, larger
+    // CTAs (column jhat staged fewer times).
     int w = 0, cap = 0, best = 0, nc = 0;
     const int c_hi = tune.ctas > 0 ? tune.ctas : 3, c_lo = tune.ctas > 0 ? tune.ctas : 1;
     const int w_hi = tune.warps > 0 ? tune.warps : 16, w_lo = tune.warps > 0 ? tune.warps : 1;

@@ -156,9 +156,9 @@ __global__ void __launch_bounds__(NT) k_colfeat(const T *__restrict__ Xt, int64_
 // while these are added.  Bound by the chain of m additions; a warp to a CTA
 // spreads the rows over the SMs.  It runs beside the column features: launched
 // after them (and they after the staging had ended), it reads only the staged
-// copy and writes only rho, and waits for them when it is done.  5000 x 1000 float: 152 us from the row-major
-// matrix (one row per lane, 256 rows to a CTA), 83 us here (102 with 16 columns
-// ahead).
+// copy and writes only rho, and waits for them when it is done.  5000 x 1000 float:
+// 152 us from the row-major matrix (one row per lane, 256 rows to a CTA), 83 us here
+// (102 with 16 columns ahead).
 template <typename T>
 __global__ void __launch_bounds__(32) k_rownorm(const T *__restrict__ Xt, int64_t ldn, int64_t n,
                                                  int64_t m, float *__restrict__ rho) {
