@@ -461,10 +461,11 @@ __device__ __forceinline__ void list_off(const ScanArgs<T> &a, int t, int64_t j,
 }
 
 // One lambda of one pair (valid: x_ijhat != 0 somewhere; batch: one of several, whose
-// ties are settled together: the mark of that in whole).  What the selection cannot settle is listed: with a call
-// here, what lived across it was spilled in the hot loop, and a pair that takes several
-// times as long as the others held up its CTA (2000 x 2000 float 11.1 ms with the
-// fallback in this place, 10.5 without).  Returns whether the batch is listed.
+// ties are settled together: the mark of that in whole).  What the selection cannot
+// settle is listed: with a call here, what lived across it was spilled in the hot
+// loop, and a pair that takes several times as long as the others held up its CTA
+// (2000 x 2000 float 11.1 ms with the fallback in this place, 10.5 without).  Returns
+// whether the batch is listed.
 template <typename T, bool CS, bool VO>
 __device__ __forceinline__ bool solve_one(const ScanArgs<T> &a, const LamView &lp, int t0, int tl,
                                           int64_t j, int64_t k, const T *xk, const float *xf,
@@ -708,7 +709,7 @@ __device__ void pairs_unit(const ScanArgs<T> &a, const LamView &lp, int t0, int 
         if (CS) colb_s[i] = b;
         // rows with x_ijhat = 0 (and padding rows) get a NaN reciprocal: their
         // approximate key is the NaN key CKNONE, above every bracket (bounds
-        // stop at CKMAX), so the level-0 pass needs no validity test.  Their
+        // stop at CKMAX), so the passes need no validity test.  Their
         // weight is 0, so even a NaN of the other sign (a key near 0) could
         // only add zero-weight candidates, which never decide the median.
         inv[i] = b != T(0) ? Approx<T>::inv_of(b) : __int_as_float(0x7FFFFFFF);
@@ -764,7 +765,7 @@ __device__ void pairs_unit(const ScanArgs<T> &a, const LamView &lp, int t0, int 
 
     const bool jwide = (cinfo.flags & COL_WIDE) != 0;
     // a warp takes the next k when it is done with its pair: pairs cost
-    // different times (bracket misses, overflows), and a fixed share per warp
+    // different times (bracket misses), and a fixed share per warp
     // leaves the CTA waiting for its slowest warp
     for (;;) {
         int idx = 0;

@@ -28,6 +28,11 @@ def test_planned_ctas_fit(dtype, m):
         assert need * p["ctas_per_sm"] <= 228 * 1024, (n, p)
 
 
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_limit_on_rows_does_not_depend_on_the_type(dtype):
+    assert l1line.max_rows(dtype) == 20608
+
+
 def test_a_callers_shape_beyond_that_is_still_taken():
     l1line.set_tuning({"warps": 15, "ctas_per_sm": 2})
     try:
