@@ -166,10 +166,6 @@ struct Decide {
     __device__ __forceinline__ void init(const ColInfo &ci, double lambda) {
         init_at(ci.Q, ci.sigma, ci.n_inexact, lambda);
     }
-    // The same test on the 32-bit weights q32 (scale sigma - shift32).
-    __device__ __forceinline__ void init32(const ColInfo &ci, double lambda) {
-        init_at((int64_t)ci.Q32, ci.sigma - ci.shift32, ci.n_inexact32, lambda);
-    }
     __device__ __forceinline__ void init_at(int64_t Qs, int sigma, int64_t inexact,
                                             double lambda) {
         Q = Qs;

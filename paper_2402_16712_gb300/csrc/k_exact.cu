@@ -51,10 +51,13 @@ cudaError_t launch_exact(const ScanArgs<T> &a, const double *lambdas, int t0, in
     LambdaPack lp;
     lp.tl_min = lp.tl_max = 0;
     for (int q = 0; q < nlc; ++q) lp.lam[q] = lambdas[t0 + q];
-    // few pairs: four warps to a CTA, as full ones lengthen an empty launch (200 x 20 fit
-    // 27.7 us, 28.5 with them); sizes between, of which two or more go to an SM, would
-    // bring the crowding back (20,480 x 48, 16 warps: 111 ms)
-    const int w = a.nj * a.m * nlc <= 4 * (int64_t)num_sms ? 4 : EX_NT / 32;
+    // little work whatever is listed: four or eight warps to a CTA, as full ones, which the
+    // pair kernel's leave no room beside, lengthen an empty launch (200 x 20 fit 27.7 us,
+    // 28.5 with them; 1315 x 36 36.8 and 38.4, 343 x 39 29.5 and 30.8).  With more work, sizes
+    // of which two or more go to an SM bring the crowding back (every pair listed: 20,480 x
+    // 48, 16 warps, 111 ms; 2000 x 64, 8 warps, 0.24 ms, 0.13 with 32; up to the line 0 to 7 us)
+    const int64_t most = a.nj * a.m * nlc;
+    const int w = most <= 4 * (int64_t)num_sms ? 4 : most * a.n <= (1 << 21) ? 8 : EX_NT / 32;
     const size_t smem = (size_t)w * HIST_WORDS * 4;
     static_assert(EX_NT / 32 * HIST_WORDS * 4 <= 48 * 1024, "needs no opt-in");
     launches++;

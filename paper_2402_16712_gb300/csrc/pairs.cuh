@@ -191,14 +191,21 @@ __device__ __forceinline__ uint32_t sat_add(uint32_t a, uint32_t b) {
 
 constexpr uint16_t ROW_MASK = 0x7FFFu;
 
-// The exact test on the 32-bit weights, with its thresholds as whole weights:
-// S passes at a negative ratio when S >= tneg, at a ratio >= 0 when S >= tpos
-// (untruncated weights; the search steers by them, the test decides).
+// The exact test on the 32-bit weights q32 (scale sigma - shift32), with its thresholds
+// as whole weights: S passes at a negative ratio when S >= tneg, at a ratio >= 0 when
+// S >= tpos (untruncated weights; the search steers by them, the test decides).
+//
+// The band: of the weights' remainders, R < e in all, S lacks some r of 0 .. R, so the
+// true 2S - Q is D + 2r - R, within e of D.  The 64-bit total tells R to within its own
+// truncation; a remainder of up to 1 for each row, in S and in Q (Decide), is a band
+// three times as wide, and as many more pairs go to the list.
 struct Dec32 : Decide {
     uint32_t tneg, tpos;
     float fneg, fpos, Qf;  // for the sample: the same, and Q / 32
     __device__ __forceinline__ void set(const ColInfo &ci, double lambda) {
-        init32(ci, lambda);
+        // R is less than this
+        const int64_t R = ((ci.Q + ci.n_inexact) >> ci.shift32) + 1 - (int64_t)ci.Q32;
+        init_at((int64_t)ci.Q32, ci.sigma - ci.shift32, ci.n_inexact32 ? R : 0, lambda);
         auto clamp = [](int64_t x) -> uint32_t {
             return x < 0 ? 0u : (x > 0xFFFFFFFFll ? 0xFFFFFFFFu : (uint32_t)x);
         };
@@ -207,6 +214,19 @@ struct Dec32 : Decide {
         fneg = (float)tneg;
         fpos = (float)tpos;
         Qf = (float)Q * (1.0f / 32.0f);
+    }
+    // 1 = true, 0 = false, -1 = undecidable at this precision.
+    __device__ __forceinline__ int cond(int64_t S, bool t_nonneg) const {
+        int64_t D = 2 * S - Q;
+        if (e == 0) return t_nonneg ? (D > -Lc) : (D > Lf);
+        if (t_nonneg) {
+            if (D - e >= -Lf) return 1;
+            if (D + e <= -Lc) return 0;
+        } else {
+            if (D - e >= Lc) return 1;
+            if (D + e <= Lf) return 0;
+        }
+        return -1;
     }
 };
 
