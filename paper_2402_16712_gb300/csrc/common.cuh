@@ -80,7 +80,7 @@ struct ColInfo {
     // q_i >> shift32 = floor(w_i 2^(sigma - shift32)), with shift32 the
     // fewest bits that bring the total Q32 below 2^32, so every partial sum
     // of q32 fits a uint32 exactly.  n_inexact32 counts the rows whose q32
-    // was truncated (the certainty band of the 32-bit decisions).
+    // was truncated (none: no band around the 32-bit decisions).
     uint32_t Q32;
     int32_t shift32;
     int32_t n_inexact32;

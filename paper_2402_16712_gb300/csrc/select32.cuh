@@ -34,17 +34,17 @@
 // missing), the weight below lo must fail the test of Lemma 1, and a key in
 // [lo, hi] must pass it.  A pair that does not meet this, more than 31 rows
 // in the range (ties), a decision inside the certainty band of the truncated
-// weights (Decide, e = n_inexact32), or a bracket too wide for float steps is
-// listed for the kernel behind, with the range where it is known (exact.cuh,
-// narrow.cuh).
+// weights (Dec32), or a bracket too wide for float steps is listed for the
+// kernel behind, with the range where it is known (exact.cuh, narrow.cuh).
 //
 // Bound (2000 x 2000 float, 32 resident warps): the L1/shared data pipe, ~690
 // wavefronts of 128 bytes per pair at 85% of its rate (pass 1: x, 1/x_ijhat,
 // q and ~2.5 per histogram atomic; pass 2: x and 1/x_ijhat; residual: x and
-// x_ijhat), and ~2200 instructions per pair at 69% of the issue slots.  Against the selection that kept every row of the
-// bracket in a per-lane list: 13.66 -> 11.14 ms there; 1000 x 500 with 32 lambdas
-// 5.62 -> 2.61 ms (one selection instead of two and a pass); and without the lists
-// 5000 rows keep 32 warps resident instead of 16, 5000 x 1000 10.23 -> 7.61 ms.
+// x_ijhat), and ~2200 instructions per pair at 69% of the issue slots.  Against the
+// selection that kept every row of the bracket in a per-lane list: 13.66 -> 11.14 ms
+// there; 1000 x 500 with 32 lambdas 5.62 -> 2.61 ms (one selection instead of two and a
+// pass); and without the lists 5000 rows keep 32 warps resident instead of 16, 5000 x
+// 1000 10.23 -> 7.61 ms.
 // Finding the crossing lane before the bin in it, instead of every bin's prefix
 // sum and test: 11.14 -> 11.06 ms, double 19.36 -> 19.19 ms.  Pairs that are not
 // settled here listed, not taken through a fallback in the same kernel: 11.06 ->
