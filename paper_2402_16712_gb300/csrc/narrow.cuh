@@ -21,14 +21,18 @@
 // steps with all rows): 47 -> 0.16 ms; near-multiples (spread 1e-5): 49 -> 0.25 ms.
 // A few listed pairs cost the latency of one warp (at 1/4 instruction per cycle, those
 // fetched for the first time more): 2000 rows 13 us, 22 with a rounded reciprocal, the
-// weight's bits taken apart for every row and x_ijhat loaded where it is used.
+// weight's bits taken apart for every row and x_ijhat loaded where it is used.  Double:
+// all four x_ijhat of a lane loaded at once and their weights without a branch, where each
+// had a load and a wait of its own for the rows below: 701 x 103, one pair listed, 106.6 ->
+// 102.2 us; 5000 x 32 of small integers 219 -> 190.
 #pragma once
 
 namespace l1l {
 
 // Column jhat for narrow(), from the column copies: x_ijhat as float and as it is, and
 // its 64-bit weight, floor(|b| 2^sigma).  Float: the scaling by a power of two, in two
-// steps, is exact where the weight is not 0.
+// steps, is exact where the weight is not 0.  Double: fixq's value by shifts alone, which
+// the FP64 pipe would slow where many pairs are listed.
 template <typename T> struct ReadCol {
     const float *xf;
     const T *x;
@@ -40,12 +44,19 @@ template <typename T> struct ReadCol {
         s1 = __int_as_float((127 + sigma - sigma / 2) << 23);
     }
     __device__ __forceinline__ T at(int i) const { return __ldg(x + i); }
+    // rows i .. i + 3 (i a multiple of 4, padded rows included)
+    __device__ __forceinline__ void rows(int i, double2 &a, double2 &b) const {
+        a = __ldg(reinterpret_cast<const double2 *>(x + i));
+        b = __ldg(reinterpret_cast<const double2 *>(x + i) + 1);
+    }
     __device__ __forceinline__ unsigned long long weight(T b) const {
         if constexpr (sizeof(T) == 4) {
             return __float2ull_rz(fabsf(b) * s0 * s1);
         } else {
-            int e = 0;
-            return (unsigned long long)fixq(b, sigma, e);
+            const uint64_t u = (uint64_t)__double_as_longlong(b) & 0x7FFFFFFFFFFFFFFFull;
+            const int be = (int)(u >> 52), s = max(be, 1) - 1075 + sigma;
+            const uint64_t m = (u & 0xFFFFFFFFFFFFFull) | (be ? 0x10000000000000ull : 0);
+            return s >= 0 ? m << s : m >> min(-s, 63);
         }
     }
 };
@@ -193,6 +204,10 @@ __device__ int narrow(const float *__restrict__ xf, const T *__restrict__ xk,
         for (int g = 0; g < ng; ++g) {
             const float4 a4 = an, b4 = bn;
             const int i0 = L1L_CHK(g * 128 + 4 * lane, ng * 128);
+            double2 c2 = {}, d2 = {};  // the weights' rows (double)
+            if constexpr (sizeof(T) == 8) {
+                if (pass == 0) col.rows(i0, c2, d2);
+            }
             if (g + 1 < ng) {
                 an = __ldg(reinterpret_cast<const float4 *>(xf + 128 + i0));
                 bn = __ldg(reinterpret_cast<const float4 *>(col.xf + 128 + i0));
@@ -202,17 +217,18 @@ __device__ int narrow(const float *__restrict__ xf, const T *__restrict__ xk,
             // weight of 0, of account below
             const float z[4] = {fmaf(a4.x, rcp_approx(b4.x), -cen), fmaf(a4.y, rcp_approx(b4.y), -cen),
                                 fmaf(a4.z, rcp_approx(b4.z), -cen), fmaf(a4.w, rcp_approx(b4.w), -cen)};
+            T e[4];
+            if constexpr (sizeof(T) == 4) {
+                e[0] = b[0], e[1] = b[1], e[2] = b[2], e[3] = b[3];
+            } else {
+                e[0] = c2.x, e[1] = c2.y, e[2] = d2.x, e[3] = d2.y;
+            }
             uint32_t f = 0;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 if (fabsf(z[u]) < delta) f |= 1u << u;
                 if (pass == 0) {
-                    T w;
-                    if constexpr (sizeof(T) == 4)
-                        w = b[u];
-                    else
-                        w = z[u] <= -delta ? col.at(i0 + u) : 0.0;
-                    const int64_t q = (int64_t)col.weight(w);
+                    const int64_t q = (int64_t)col.weight(e[u]);
                     below += z[u] <= -delta ? q : 0;
                 }
             }
