@@ -18,7 +18,7 @@
 // Bound by instructions, ~12 per row outside the range and a division (queued, so
 // that all lanes divide) and three shared-memory words per row inside.  2000 x 64 of
 // small integers, double, where such a pair went to the exact kernel (64 bisection
-// steps with all rows): 47 -> 0.16 ms; near-multiples (spread 1e-5): 49 -> 0.25 ms.
+// steps with all rows): 47 -> 0.15 ms; near-multiples (spread 1e-5): 49 -> 0.24 ms.
 // A few listed pairs cost the latency of one warp (at 1/4 instruction per cycle, those
 // fetched for the first time more): 2000 rows 13 us, 22 with a rounded reciprocal, the
 // weight's bits taken apart for every row and x_ijhat loaded where it is used.  Double:
